@@ -159,6 +159,10 @@ struct ibm_ctx {
   double* partials = nullptr;
   DevScalars* sc = nullptr;
   DevScalars* sc_host = nullptr;  // pinned mirror
+  // FP64 sweeps kept on chip (precision 0)
+  Sor64Plan sor64;
+  Sor64Tiles sor64_tiles{};
+  Sor64Result *sor64_res = nullptr, *sor64_host = nullptr;  // device; pinned, behind sc_host
   // history
   double *cl_d = nullptr, *cd_d = nullptr;
   int hist_cap = 0;
@@ -803,6 +807,45 @@ int read_norm(ibm_ctx* c, const unsigned long long* dev_bits, double* out) {
   return IBM_OK;
 }
 
+// The sweeps and checks of solve_poisson on the device (k_sor64.cu); the host
+// waits once per launch of up to kChunk64 sweeps.
+constexpr int kChunk64 = 8192;
+int solve_poisson_chip(ibm_ctx* c, double thr, int m, int maxs, int* sweeps, double* res) {
+  const Geo& g = c->geo;
+  Sor64Tiles t = c->sor64_tiles;
+  t.phi2 = c->phi2;
+  for (int done = 0;;) {
+    const Sor64Args a{g.nx, g.ny, g.pitch, at(0, 0, g.pitch), g.pE, g.pW, g.pN, g.pS, c->phi, c->b, c->invd_p,
+                      c->P.omega_p, thr, m, maxs - done, kChunk64};
+    if (c->profiling) CUDA_TRY(cudaEventRecord(c->ev0, c->stream));
+    CUDA_TRY(launch_sor64(c->stream, c->sor64, a, t, c->sor64_res));
+    if (c->profiling) CUDA_TRY(cudaEventRecord(c->ev1, c->stream));
+    CUDA_TRY(cudaMemcpyAsync(c->sor64_host, c->sor64_res, sizeof(Sor64Result), cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(cudaStreamSynchronize(c->stream));
+    const Sor64Result& r = *c->sor64_host;
+    c->prof.launches += 1;
+    if (c->profiling) {
+      float ms = 0.f;
+      CUDA_TRY(cudaEventElapsedTime(&ms, c->ev0, c->ev1));
+      c->prof.sweep_ms += ms;
+      c->prof.sweep_launches += 1;
+      c->prof.sweep_cells += (long long)c->nx * c->ny;
+    }
+    if (r.late) return fail(IBM_E_TIMEOUT, "pressure solve: a block waited too long for its neighbours");
+    *sweeps = done + r.checked;
+    *res = bits_to_double(r.bits);
+    done += r.sweeps;
+    switch (r.status) {
+      case SOR64_OK: return IBM_OK;
+      case SOR64_DIVERGED:
+        return fail(IBM_E_DIVERGED, "pressure residual is not finite after %d sweeps", *sweeps);
+      case SOR64_NOCONV:
+        return fail(IBM_E_NOCONV, "pressure solve: %d sweeps, residual %.3e > %.3e", done, *res, thr);
+      default: break;
+    }
+  }
+}
+
 // Red-black SOR for the pressure: residual checked before the first sweep
 // and every m sweeps.
 int solve_poisson(ibm_ctx* c, double tol, double rtol, int m, int maxs, int* sweeps, double* res) {
@@ -817,6 +860,7 @@ int solve_poisson(ibm_ctx* c, double tol, double rtol, int m, int maxs, int* swe
     thr = std::fmax(tol, rtol * bmax);
   }
   if (m < 1) m = 1;
+  if (c->sor64.kind != Sor64Plan::NONE) return solve_poisson_chip(c, thr, m, maxs, sweeps, res);
   const double omega = c->P.omega_p;
   int pending = 0;  // sweep launches inside the open event bracket
   for (int s = 0;; ++s) {
@@ -1883,8 +1927,22 @@ int ibm_create_grid(const ibm_grid_params* params, ibm_ctx** out) {
   rc |= c->alloc(&c->sc, 1);
   rc |= c->alloc(&c->partials, 4 * RED_BLOCKS);
   if (!rc) rc = setup_geometry(c);
-  if (!rc && cudaMallocHost((void**)&c->sc_host, sizeof(DevScalars)) != cudaSuccess) rc = IBM_E_CUDA;
+  if (!rc && cudaMallocHost((void**)&c->sc_host, sizeof(DevScalars) + sizeof(Sor64Result)) != cudaSuccess)
+    rc = IBM_E_CUDA;
   if (!rc) rc = ensure_history(c, 1024);
+  if (!rc && P.precision == 0) {
+    c->sor64 = sor64_plan(P.nx, P.ny, true);
+    if (c->sor64.kind != Sor64Plan::NONE) {
+      // one block: two norms and two flags per tile, the result
+      const size_t nt = sor64_max_tiles();
+      unsigned char* blk = nullptr;
+      rc |= c->alloc(&blk, 24 * nt + sizeof(Sor64Result));
+      c->sor64_tiles.norms = (unsigned long long*)blk;
+      c->sor64_tiles.flags = (unsigned*)(blk + 16 * nt);
+      c->sor64_res = (Sor64Result*)(blk + 24 * nt);
+      c->sor64_host = (Sor64Result*)(c->sc_host + 1);
+    }
+  }
   // band arrays exist (1 x 1) even without a body
   if (!rc) {
     rc |= c->alloc(&c->fu, 1);

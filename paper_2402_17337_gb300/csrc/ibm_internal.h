@@ -118,6 +118,41 @@ void launch_poisson_res(cudaStream_t s, const Geo& g, const double* phi, const d
 // by launch_poisson_res
 void launch_poisson_res2(cudaStream_t s, const Geo& g, const double* phi_a, const double* phi_b, const double* b,
                          unsigned long long* bits_a, unsigned long long* bits_b);
+// FP64 SOR with the grid kept on chip and the residual checks on the device
+// (k_sor64.cu): one launch runs until the tolerance is met, maxs sweeps are
+// done or chunk sweeps have passed.  Element (i, j) of phi, b and invd lies at
+// off + j pitch + i; invd may be null for the cluster kernel (recomputed).
+struct Sor64Args {
+  int nx, ny, pitch;
+  size_t off;
+  const double *pE, *pW, *pN, *pS;
+  double* phi;
+  const double *b, *invd;
+  double omega, thr;
+  int m, maxs, chunk;  // check every m sweeps
+};
+struct Sor64Tiles {
+  int nbx, nby, K;
+  double* phi2;                // a second pitched field (exchanges alternate between it and phi)
+  unsigned* flags;             // 2 per tile
+  unsigned long long* norms;   // 2 per tile
+};
+enum { SOR64_MORE = 0, SOR64_OK, SOR64_NOCONV, SOR64_DIVERGED };
+struct Sor64Result {
+  unsigned long long bits;  // norm of the last check
+  int checked, sweeps;      // sweeps at the last check, sweeps done
+  int status, late;         // late: a CTA gave up a wait
+};
+struct Sor64Plan {
+  enum Kind { NONE, CLUSTER, TILES } kind = NONE;
+  int nbx = 0, nby = 0, K = 0;
+  size_t smem = 0;
+};
+// tiles: the caller can pass Sor64Tiles
+Sor64Plan sor64_plan(int nx, int ny, bool tiles);
+int sor64_max_tiles();
+cudaError_t launch_sor64(cudaStream_t s, const Sor64Plan& p, const Sor64Args& a, const Sor64Tiles& t, Sor64Result* out);
+
 void launch_shift(cudaStream_t s, const Geo& g, double* phi, const DevScalars* sc);
 void launch_bmax(cudaStream_t s, const Geo& g, const double* b, unsigned long long* bits);
 void launch_fill_hash(cudaStream_t s, const Geo& g, double* x);

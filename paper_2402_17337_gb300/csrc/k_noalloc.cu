@@ -195,8 +195,38 @@ extern "C" int ibm_poisson_solve_noalloc(int nx, int ny, const double* xf, const
   double* ref = scratch + COEF + 1;
   const int m = check_every > 0 ? check_every : 8;
   const int maxs = max_sweeps > 0 ? max_sweeps : 1000000;
+  // a grid that one cluster holds: sweeps and checks on the device (the result
+  // in the scratch behind the gauge value)
+  const ibm::Sor64Plan plan = ibm::sor64_plan(nx, ny, false);
+  if (plan.kind == ibm::Sor64Plan::CLUSTER) {
+    ibm::Sor64Result* out = (ibm::Sor64Result*)(scratch + COEF + 2);
+    for (int done = 0;;) {
+      const ibm::Sor64Args a{nx, ny, nx, 0, g.pE, g.pW, g.pN, g.pS, phi_dev, b_dev, nullptr, omega, tol, m, maxs - done, 8192};
+      ibm::Sor64Result r{};
+      cudaError_t e = ibm::launch_sor64(s, plan, a, ibm::Sor64Tiles{}, out);
+      if (e != cudaSuccess) return cuda_fail("the launch of the sweeps", e);
+      e = cudaMemcpyAsync(&r, out, sizeof r, cudaMemcpyDeviceToHost, s);
+      if (e != cudaSuccess) return cuda_fail("cudaMemcpyAsync of the result", e);
+      e = cudaStreamSynchronize(s);
+      if (e != cudaSuccess) return cuda_fail("the sweeps (cudaStreamSynchronize)", e);
+      double v;
+      std::memcpy(&v, &r.bits, sizeof v);
+      if (sweeps) *sweeps = done + r.checked;
+      if (res) *res = v;
+      done += r.sweeps;
+      if (r.status == ibm::SOR64_DIVERGED) {
+        ibm::set_last_error("ibm_poisson_solve_noalloc: residual is not finite");
+        return IBM_E_DIVERGED;
+      }
+      if (r.status == ibm::SOR64_NOCONV) {
+        ibm::set_last_error("ibm_poisson_solve_noalloc: max_sweeps reached before the tolerance");
+        return IBM_E_NOCONV;
+      }
+      if (r.status == ibm::SOR64_OK) break;
+    }
+  }
   dim3 blk(32, 8), grd_res((nx + 31) / 32, (ny + 7) / 8), grd_half(((nx + 1) / 2 + 31) / 32, (ny + 7) / 8);
-  for (int it = 0;; ++it) {
+  for (int it = 0; plan.kind != ibm::Sor64Plan::CLUSTER; ++it) {
     if (it % m == 0) {
       unsigned long long bits = 0;
       cudaError_t e = cudaMemsetAsync(norm, 0, sizeof(unsigned long long), s);

@@ -1,0 +1,65 @@
+"""FP64 sweeps kept on chip (k_sor64.cu) against the oracle: one cluster, tiles
+over all SMs, and the sizes where a grid goes from one to the other; strips and
+tiles of a few rows, odd sizes, sweep caps between two checks.  The kernels and
+the oracle share their arithmetic, so sweep counts agree exactly; fields are
+compared at 1e-13 of their largest value, above the rounding that 8 operations
+an update could leave in 60 sweeps (8 x 60 x 1.1e-16)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2402_17337_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("nx,ny", [(5, 4), (9, 200), (64, 15), (33, 16), (17, 17), (128, 93), (129, 95), (41, 300),
+                                   (300, 41), (191, 129), (513, 257), (500, 500), (501, 501)])
+@pytest.mark.parametrize("m,cap", [(8, 60), (3, 20), (1, 2), (7, 49)])
+def test_sweeps_on_chip_match_oracle(nx, ny, m, cap):
+    import torch
+    from paper_2402_17337_gb300 import Solver, build
+    build.build()
+    kw = dict(x0=0.0, x1=2.0 + nx / ny, y0=0.0, y1=1.5, nx=nx, ny=ny, hmin=0.0, dt=1.0)
+    g, o = Solver(**kw), oracle.Sim(**kw)
+    b = W.random_field((ny, nx), seed=nx + 3 * ny)
+    b -= b.mean()
+    phi0 = W.random_field((ny, nx), seed=5, scale=0.1)
+    rc, phio, so, ro = o.poisson(b, phi0=phi0, tol=1e-300, check=m, maxs=cap)
+    bd, pd = torch.tensor(b, device="cuda"), torch.tensor(phi0, device="cuda")
+    torch.cuda.synchronize()
+    rg, sg, rr = g.poisson_solve(bd.data_ptr(), pd.data_ptr(), 1e-300, m, cap)
+    assert rc == rg == -3 and sg == cap // m * m
+    assert abs(rr - ro) <= 1e-10 * ro
+    assert np.abs(pd.cpu().numpy() - phio).max() <= 1e-13 * np.abs(phio).max()
+
+
+def test_two_streams_and_threads_solve_at_once():
+    """Cooperative launches of two contexts from two threads do not wait on each other for good."""
+    import threading
+
+    import torch
+    from paper_2402_17337_gb300 import Solver, build
+    build.build()
+    nx, ny = 384, 200
+    kw = dict(x0=0.0, x1=3.0, y0=0.0, y1=1.5, nx=nx, ny=ny, hmin=0.0, dt=1.0)
+    b = W.random_field((ny, nx), seed=1)
+    b -= b.mean()
+    out = {}
+
+    def work(k):
+        g = Solver(**kw)
+        bd = torch.tensor(b, device="cuda")
+        for _ in range(4):
+            pd = torch.zeros_like(bd)
+            torch.cuda.synchronize()
+            rc = g.poisson_solve(bd.data_ptr(), pd.data_ptr(), 1e-300, 8, 400)
+        out[k] = rc, pd.cpu().numpy()
+        g.close()
+
+    ts = [threading.Thread(target=work, args=(k,)) for k in range(3)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert all(out[k][0][0] == -3 and np.array_equal(out[k][1], out[0][1]) for k in range(3))
