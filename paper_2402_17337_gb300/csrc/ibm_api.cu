@@ -803,6 +803,7 @@ int read_norm(ibm_ctx* c, const unsigned long long* dev_bits, double* out) {
   CUDA_TRY(cudaMemcpyAsync(&c->sc_host->res_bits, dev_bits, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                            c->stream));
   CUDA_TRY(cudaStreamSynchronize(c->stream));
+  if (sor32_failed()) return fail(IBM_E_TIMEOUT, "a sweep kernel gave up a bounded wait");
   *out = bits_to_double(c->sc_host->res_bits);
   return IBM_OK;
 }
@@ -1341,6 +1342,9 @@ struct ibm_batch {
   Sor32Case *h_sor = nullptr, *d_sor = nullptr;  // tables A (e32 -> e32b) at [0, n), B (e32b -> e32) at [n, 2n)
   DcCase *h_dc = nullptr, *d_dc = nullptr;
   unsigned long long *h_bits = nullptr, *d_bits = nullptr;
+  // tensor maps of every case's sweep arrays (sweep form 11) and what they were made for
+  unsigned char *h_maps = nullptr, *d_maps = nullptr;
+  std::vector<std::pair<int, const float*>> maps_of;
   // whole-step batching: the case table, the first block of every case per
   // launch kind, the active-case tables of the velocity solves (one region
   // for the residual launch, one for the sweep launches) and the scalars
@@ -1376,9 +1380,9 @@ struct ibm_batch {
     if (d_sor) cudaFree(d_sor);
     if (d_dc) cudaFree(d_dc);
     if (d_bits) cudaFree(d_bits);
-    for (void* q : {(void*)h_cases, (void*)h_first, (void*)h_hres, (void*)h_hswp, (void*)h_rb})
+    for (void* q : {(void*)h_maps, (void*)h_cases, (void*)h_first, (void*)h_hres, (void*)h_hswp, (void*)h_rb})
       if (q) cudaFreeHost(q);
-    for (void* q : {(void*)d_cases, (void*)d_first, (void*)d_hres, (void*)d_hswp, (void*)d_rb})
+    for (void* q : {(void*)d_maps, (void*)d_cases, (void*)d_first, (void*)d_hres, (void*)d_hswp, (void*)d_rb})
       if (q) cudaFree(q);
     for (cudaEvent_t e : ev) cudaEventDestroy(e);
     if (ev_b) cudaEventDestroy(ev_b);
@@ -1399,14 +1403,29 @@ int batch_sor_tables(ibm_batch* B, int cfg, const std::vector<int>& act, int* ti
                      const std::vector<int>* pairs = nullptr) {
   const int n = (int)B->cs.size(), na = (int)act.size();
   int first = 0;
+  // maps of the shape and of the buffers each case has now (a case stepped alone may have swapped its two)
+  const size_t mb = sor32_maps_bytes();
+  bool remade = false;
+  B->maps_of.resize(n, {-1, nullptr});
+  for (int i : act) {
+    ibm_ctx* c = B->cs[i];
+    const std::pair<int, const float*> key{cfg, c->e32};
+    if (B->maps_of[i] == key) continue;
+    if (!sor32_case_maps(cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, B->h_maps + i * mb))
+      return fail(IBM_E_CUDA, "batch case %d: tensor maps of the sweep arrays", i);
+    B->maps_of[i] = key;
+    remade = true;
+  }
+  if (remade) CUDA_TRY(cudaMemcpyAsync(B->d_maps, B->h_maps, n * mb, cudaMemcpyHostToDevice, B->stream));
   for (int k = 0; k < na; ++k) {
     ibm_ctx* c = B->cs[act[k]];
     int tx = 0, ty = 0;
     sor32_tiles(cfg, c->geo32, &tx, &ty);
     const float om = (float)c->P.omega_p;
     const int np = pairs ? (*pairs)[k] : INT_MAX;
-    B->h_sor[k] = Sor32Case{c->geo32, c->e32, c->e32b, c->r32, c->invd32, om, first, tx, np};
-    B->h_sor[n + k] = Sor32Case{c->geo32, c->e32b, c->e32, c->r32, c->invd32, om, first, tx, np};
+    const void* maps = B->d_maps + act[k] * mb;
+    B->h_sor[k] = Sor32Case{c->geo32, c->e32, c->e32b, c->r32, c->invd32, om, first, tx, maps, 0, np};
+    B->h_sor[n + k] = Sor32Case{c->geo32, c->e32b, c->e32, c->r32, c->invd32, om, first, tx, maps, 1, np};
     first += tx * ty;
   }
   *tiles = first;
@@ -1545,6 +1564,7 @@ int batch_solve(ibm_batch* B, const std::vector<double>& thr, std::vector<ibm_st
                              B->stream));
     CUDA_TRY(cudaStreamSynchronize(B->stream));
     CUDA_TRY(cudaGetLastError());
+    if (sor32_failed()) return fail(IBM_E_TIMEOUT, "a sweep kernel gave up a bounded wait");
     if (timing) {
       float ms = 0.f;
       CUDA_TRY(cudaEventElapsedTime(&ms, B->t0, B->t1));
@@ -2405,6 +2425,8 @@ int ibm_batch_create(ibm_ctx* const* cases, int n, ibm_batch** out) {
   ok = ok && cudaMalloc((void**)&B->d_sor, 2 * n * sizeof(Sor32Case)) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&B->d_dc, n * sizeof(DcCase)) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&B->d_bits, n * sizeof(unsigned long long)) == cudaSuccess;
+  ok = ok && cudaMallocHost((void**)&B->h_maps, n * sor32_maps_bytes()) == cudaSuccess;
+  ok = ok && cudaMalloc((void**)&B->d_maps, n * sor32_maps_bytes()) == cudaSuccess;
   ok = ok && cudaMallocHost((void**)&B->h_cases, n * sizeof(StepCase)) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&B->d_cases, n * sizeof(StepCase)) == cudaSuccess;
   ok = ok && cudaMallocHost((void**)&B->h_first, BK_NUM * n * sizeof(int)) == cudaSuccess;

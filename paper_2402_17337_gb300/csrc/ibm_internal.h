@@ -231,6 +231,8 @@ struct Sor32Case {
   const float* invd;
   float omega;
   int first, tiles_x;  // first CTA of this case, tiles per row
+  const void* maps;    // form 11: tensor maps of e32, e32b, r32, invd32 (device memory)
+  int flip;            // form 11: which of the first two e_in is
   int pairs;           // launch pairs of this round for this case (a launch with pair index >= pairs skips it)
 };
 struct DcCase {
@@ -243,6 +245,12 @@ struct DcCase {
   float* r32;
   unsigned long long* res_bits;
 };
+// true once a sweep kernel has given up a bounded wait for a tile's copies
+bool sor32_failed();
+// form 11: a case's four tensor maps (Sor32Case::maps; host memory, then copied to the device, 64-byte aligned)
+size_t sor32_maps_bytes();
+bool sor32_case_maps(int cfg, const Geo32& g, const float* e, const float* eb, const float* r, const float* invd,
+                     void* out);
 void sor32_tiles(int cfg, const Geo32& g, int* tiles_x, int* tiles_y);
 cudaError_t sor32_batch_prepare(int cfg);
 // pdl: launch as a programmatic dependent of the previous kernel on the

@@ -16,6 +16,11 @@
 // update coefficients a = omega / d and b = -a r (formed from the
 // right-hand side and the reciprocal diagonal) in registers for the whole launch
 // and shared memory only carries the values the neighbours read.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
+#include <algorithm>
+#include <mutex>
 #include <type_traits>
 
 #include "ibm_internal.h"
@@ -786,6 +791,219 @@ __device__ __forceinline__ void sor32_tile_v9(const Geo32& g, const float* __res
   }
 }
 
+// Fifth form (11): the update of form 10 on tiles that arrive by TMA, in
+// persistent CTAs.  In form 10 each thread loads its own cells of r, 1/d and
+// e; its registers hold a few of those loads at a time, so a tile waits for
+// memory several times in a row: 7.6 k of the 18.2 k clocks of a tile on
+// 2048x1024, with L2 at 13 % of its rate.  Here one thread requests the whole
+// tile (12 B a cell, three tensor copies, zero-filled outside the grid) and
+// each thread picks its cells up from shared memory; a CTA takes several
+// tiles in turn and requests the next one as soon as it has picked up the
+// current one, so that all but the first load hide behind the sweeps.
+// (16-byte cp.async copies instead of TMA cost 3.8 k clocks a tile to issue.)
+// With an even number of rows per run the first row of every run is even, so
+// a row's parity is known at compile time and all warps run the same code;
+// the warps of odd runs alternate between two copies of it (522 against 700
+// clocks a half-sweep for 96 and 112 rows).
+template <int TY, int K, int NY>
+struct Sor32ShapeV11 {
+  static constexpr int LK = 64, HK = K / 2, TK = LK - 2 * HK, LY = TY + 2 * K;
+  static constexpr int RPT = LY / NY, T = 32 * NY;
+  static constexpr int edges = 2 * (NY + 2) * 2 * 32;  // float2: first and last row of every run
+  static constexpr int field = 2 * LY * 32;            // float2: one array of the tile, both colours
+  static constexpr size_t smem = sizeof(float2) * (edges + 3 * field) + 16;
+  static_assert(K % 8 == 0, "the tile's first packed column lies on a 16-byte boundary");
+  static_assert(TY % 2 == 0 && LY % NY == 0 && RPT >= 3, "whole runs with a row between their first and last");
+};
+
+__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+constexpr long long kSorWaitCycles = 4000000000ll;  // about 2 s at the SM clock
+
+// waits for the phase with the given parity of an mbarrier; false (and *err
+// set) if it has not completed within kSorWaitCycles
+__device__ __forceinline__ bool sor_wait(unsigned bar, unsigned parity, unsigned* err) {
+  long long t0 = 0;
+  for (;;) {
+    unsigned ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    const long long now = clock64();
+    if (!t0) t0 = now;
+    if (now - t0 > kSorWaitCycles) {
+      atomicOr_system(err, 1u);
+      return false;
+    }
+  }
+}
+// one array of a tile: box {64 packed columns, LY rows, 2 colours} at (k0, j0, 0)
+__device__ __forceinline__ void tma_field(void* dst, const CUtensorMap* map, int k0, int j0, unsigned bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+      "[%5];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(k0), "r"(j0), "r"(0), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void expect_bytes(unsigned bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+
+// shared memory of a form-11 CTA: edge rows, then r, 1/d and e of the tile, then the mbarrier
+template <class S>
+struct TileMem {
+  float2 *edge, *r, *d, *e;
+  unsigned bar;
+  __device__ __forceinline__ explicit TileMem(unsigned char* base) {
+    edge = reinterpret_cast<float2*>(base);
+    r = edge + S::edges;
+    d = r + S::field;
+    e = d + S::field;
+    bar = smem_u32(e + S::field);
+  }
+};
+
+// set-up of a CTA: zero edge rows around the runs, the mbarrier
+template <class S>
+__device__ __forceinline__ void setup_v11(const TileMem<S>& M, int NY) {
+  const int tid = threadIdx.y * 32 + threadIdx.x;
+  float2* se = M.edge;  // [2][NY + 2][2][32]
+  for (int t = tid; t < 2 * 2 * 2 * 32; t += S::T)
+    se[(((t >> 7) * (NY + 2) + ((t >> 6) & 1 ? NY + 1 : 0)) * 2 + ((t >> 5) & 1)) * 32 + (t & 31)] =
+        make_float2(0.f, 0.f);
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(M.bar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+}
+
+// One tile whose arrays have been requested under the mbarrier phase `parity`;
+// next() is called by one thread once the tile has been picked up from shared
+// memory (it requests the next one).  False if the wait gave up.
+template <int TY, int K, int NY, class Next>
+__device__ __forceinline__ bool sor32_tile_v11(const Geo32& g, float* __restrict__ e_out, float omega, int zero_init,
+                                               int k0, int j0, const TileMem<Sor32ShapeV11<TY, K, NY>>& M,
+                                               unsigned parity, unsigned* err, Next next) {
+  using S = Sor32ShapeV11<TY, K, NY>;
+  constexpr int HK = S::HK, TK = S::TK, LY = S::LY, RPT = S::RPT;
+  constexpr unsigned FULL = 0xffffffffu;
+  float2(*se)[NY + 2][2][32] = reinterpret_cast<float2(*)[NY + 2][2][32]>(M.edge);  // run w at [w + 1]
+  const int nx = g.nx, ny = g.ny, pk = g.pk;
+  const int tx = threadIdx.x, ty = threadIdx.y, ly0 = ty * RPT;
+  const float omc = 1.f - omega;
+  const int kp = k0 + 2 * tx;  // first packed column of the pair; rows hold pk (even) entries
+  const bool pair_ok = kp >= 0 && kp < pk;
+  float ev[2][RPT][2], av[2][RPT][2], bv[2][RPT][2], cE[2][2], cW[2][2], cN[RPT], cS[RPT];
+#pragma unroll
+  for (int m = 0; m < 2; ++m) {  // cE[m][s]: the cell at i = 2k + s
+    const int k = kp + m;
+    cE[m][0] = pair_ok ? g.cE0[k] : 0.f;
+    cE[m][1] = pair_ok ? g.cE1[k] : 0.f;
+    cW[m][0] = pair_ok ? g.cW0[k] : 0.f;
+    cW[m][1] = pair_ok ? g.cW1[k] : 0.f;
+  }
+#pragma unroll
+  for (int q = 0; q < RPT; ++q) {
+    const int j = j0 + ly0 + q;
+    const bool rowok = j >= 0 && j < ny;
+    cN[q] = rowok ? g.pN[j] : 0.f;
+    cS[q] = rowok ? g.pS[j] : 0.f;
+  }
+  const bool late = !sor_wait(M.bar, parity, err);
+  if (__syncthreads_or(late)) return false;  // and every warp is past the edge rows of the tile before
+#pragma unroll
+  for (int q = 0; q < RPT; ++q)
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      // entries beyond the grid are zero, in the arrays' padding too: a = 0, b = -0, and a cell that starts at
+      // zero stays there
+      const int o = (c * LY + ly0 + q) * 32 + tx;
+      const float2 rr = M.r[o], dd = M.d[o];
+      sor_ab(omega, rr.x, dd.x, av[c][q][0], bv[c][q][0]);
+      sor_ab(omega, rr.y, dd.y, av[c][q][1], bv[c][q][1]);
+      const float2 x = zero_init ? make_float2(0.f, 0.f) : M.e[o];
+      ev[c][q][0] = x.x;
+      ev[c][q][1] = x.y;
+      if (q == 0) se[c][ty + 1][0][tx] = x;
+      if (q == RPT - 1) se[c][ty + 1][1][tx] = x;
+    }
+  __syncthreads();
+  if (tx == 0 && ty == 0) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the reads above before the next copies' writes
+    next();
+  }
+  __syncwarp();
+  // row q of colour c in a run whose first row has parity P
+  auto row = [&](auto colour, auto parity_, int q) {
+    constexpr int c = decltype(colour)::value, oc = c ^ 1;
+    const int s = (c + q + decltype(parity_)::value) & 1;
+    float xo[2];  // the neighbour across the packed column
+    if (s) {
+      xo[0] = ev[oc][q][1];
+      xo[1] = __shfl_down_sync(FULL, ev[oc][q][0], 1);
+    } else {
+      xo[0] = __shfl_up_sync(FULL, ev[oc][q][1], 1);
+      xo[1] = ev[oc][q][0];
+    }
+    float2 nN = make_float2(0.f, 0.f), nS = make_float2(0.f, 0.f);
+    if (q == RPT - 1) nN = se[oc][ty + 2][0][tx];
+    if (q == 0) nS = se[oc][ty][1][tx];
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      const float xN = q < RPT - 1 ? ev[oc][q < RPT - 1 ? q + 1 : q][m] : (m ? nN.y : nN.x);
+      const float xS = q > 0 ? ev[oc][q > 0 ? q - 1 : q][m] : (m ? nS.y : nS.x);
+      ev[c][q][m] = sor_update(cN[q], xN, cS[q], xS, s ? cW[m][1] : cE[m][0], ev[oc][q][m], s ? cE[m][1] : cW[m][0],
+                               xo[m], av[c][q][m], bv[c][q][m], omc, ev[c][q][m]);
+    }
+    if (q == 0) se[c][ty + 1][0][tx] = make_float2(ev[c][q][0], ev[c][q][1]);
+    if (q == RPT - 1) se[c][ty + 1][1][tx] = make_float2(ev[c][q][0], ev[c][q][1]);
+  };
+  // the barrier between the rows inside each run and its edge rows, as in form 10
+  auto half = [&](auto colour, auto parity_) {
+#pragma unroll
+    for (int q = 1; q < RPT - 1; ++q) row(colour, parity_, q);
+    __syncthreads();
+    row(colour, parity_, 0);
+    row(colour, parity_, RPT - 1);
+  };
+  using Zero = std::integral_constant<int, 0>;
+  using One = std::integral_constant<int, 1>;
+  const bool odd = RPT % 2 != 0 && (ty & 1) != 0;  // j0 is even
+#pragma unroll 1
+  for (int h = 0; h < K; h += 2) {
+    if (odd) {
+      if constexpr (RPT % 2 != 0) {
+        half(Zero{}, One{});
+        half(One{}, One{});
+      }
+    } else {
+      half(Zero{}, Zero{});
+      half(One{}, Zero{});
+    }
+  }
+  if (2 * tx >= HK && 2 * tx < HK + TK && pair_ok) {
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+      const int ly = ly0 + q, j = j0 + ly;
+      if (ly < K || ly >= K + TY || j >= ny) continue;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int s = (c + j) & 1;
+        float* dst = e_out + (size_t)(c * ny + j) * pk + kp;
+        if (2 * (kp + 1) + s < nx)
+          *reinterpret_cast<float2*>(dst) = make_float2(ev[c][q][0], ev[c][q][1]);
+        else if (2 * kp + s < nx)
+          dst[0] = ev[c][q][0];
+      }
+    }
+  }
+  return true;
+}
+
 // A tile shape: rows per tile, half-sweeps per launch, thread rows, form
 // (3: sor32_tile; 4: sor32_tile_v4 with a and b in shared memory; 5: with
 // a and b in registers; 6, 7: sor32_tile_v6 likewise; 8: as 7 with the
@@ -798,8 +1016,9 @@ struct Cfg {
   static constexpr int HK = (K + 1) / 2, TK = 64 - 2 * HK;
   static constexpr size_t smem =
       std::conditional_t<V == 3, Sor32Shape<TY, K, NY>,
-                         std::conditional_t<(V >= 9), Sor32ShapeV9<TY, K, NY>,
-                                            Sor32ShapeV4<TY, K, NY, V == 5 || V >= 7>>>::smem;
+                         std::conditional_t<V == 11, Sor32ShapeV11<TY, K, NY>,
+                                            std::conditional_t<(V >= 9), Sor32ShapeV9<TY, K, NY>,
+                                                               Sor32ShapeV4<TY, K, NY, V == 5 || V >= 7>>>>::smem;
 };
 
 template <class C>
@@ -861,6 +1080,153 @@ __global__ void __launch_bounds__(32 * C::NY, C::MINB)
   tile<C>(c.g, c.e_in, c.e_out, c.r, c.invd, c.omega, zero_init, t % c.tiles_x, t / c.tiles_x, smem);
 }
 
+// Form 11: CTA b takes tiles b, b + gridDim.x, ... of the grid (nbx tiles a
+// row).  The first tile's r and 1/d are requested before the dependency wait
+// on the argument given in sor32_tile_v6 (TMA reads through L2); e, which the
+// previous launch wrote, after it.
+template <class C>
+__global__ void __launch_bounds__(32 * C::NY, C::MINB)
+    k_sor32_tma(const __grid_constant__ CUtensorMap me, const __grid_constant__ CUtensorMap mr,
+                const __grid_constant__ CUtensorMap md, const Geo32 g, float* __restrict__ e_out, float omega,
+                int zero_init, int nbx, int ntiles, unsigned* __restrict__ err) {
+  using S = Sor32ShapeV11<C::TY, C::K, C::NY>;
+  extern __shared__ __align__(1024) unsigned char smem_tile[];
+  const TileMem<S> M(smem_tile);
+  const bool lead = threadIdx.x == 0 && threadIdx.y == 0;
+  setup_v11<S>(M, C::NY);
+  constexpr unsigned bytes = sizeof(float2) * S::field;
+  auto fetch_rd = [&](int t) {
+    const int k0 = t % nbx * S::TK - S::HK, j0 = t / nbx * C::TY - C::K;
+    expect_bytes(M.bar, zero_init ? 2 * bytes : 3 * bytes);
+    tma_field(M.r, &mr, k0, j0, M.bar);
+    tma_field(M.d, &md, k0, j0, M.bar);
+  };
+  auto fetch_e = [&](int t) {
+    tma_field(M.e, &me, t % nbx * S::TK - S::HK, t / nbx * C::TY - C::K, M.bar);
+  };
+  int t = blockIdx.x;
+  if (!zero_init && lead) fetch_rd(t);
+  griddep_wait();
+  griddep_release();
+  if (lead) {
+    if (zero_init)
+      fetch_rd(t);
+    else
+      fetch_e(t);
+  }
+  for (unsigned n = 0; t < ntiles; ++n) {
+    const int k0 = t % nbx * S::TK - S::HK, j0 = t / nbx * C::TY - C::K;
+    t += gridDim.x;
+    auto next = [&] {
+      if (t >= ntiles) return;
+      fetch_rd(t);
+      if (!zero_init) fetch_e(t);
+    };
+    if (!sor32_tile_v11<C::TY, C::K, C::NY>(g, e_out, omega, zero_init, k0, j0, M, n & 1u, err, next)) return;
+  }
+}
+
+// Batched form of it: the tiles of many cases in one list (CTA b takes tiles
+// b, b + gridDim.x, ...; a case's tiles are [first, first + count)).
+template <class C>
+__global__ void __launch_bounds__(32 * C::NY, C::MINB)
+    k_sor32_tma_batch(const Sor32Case* __restrict__ cases, int ncases, int ntiles, int zero_init, int q,
+                      unsigned* __restrict__ err) {
+  using S = Sor32ShapeV11<C::TY, C::K, C::NY>;
+  extern __shared__ __align__(1024) unsigned char smem_tile[];
+  __shared__ Sor32Case slot[2];  // descriptors of the current and the next tile's case
+  __shared__ int tile_no[2];     // and their tiles (ntiles: none)
+  const TileMem<S> M(smem_tile);
+  const bool lead = threadIdx.x == 0 && threadIdx.y == 0;
+  setup_v11<S>(M, C::NY);
+  griddep_wait();  // the descriptor tables are rewritten between rounds
+  griddep_release();
+  constexpr unsigned bytes = sizeof(float2) * S::field;
+  // one thread: the first tile at or after t of a case with sweeps left in this round, its descriptor into slot[w],
+  // its copies on their way
+  auto request = [&](int t, int w) {
+    for (; t < ntiles; t += gridDim.x) {
+      int lo = 0, hi = ncases - 1;
+      while (lo < hi) {  // last case with first <= t
+        const int mid = (lo + hi + 1) >> 1;
+        if (cases[mid].first <= t) lo = mid; else hi = mid - 1;
+      }
+      const Sor32Case& c = cases[lo];
+      if (q >= c.pairs) continue;
+      slot[w] = c;
+      const int u = t - c.first, k0 = u % c.tiles_x * S::TK - S::HK, j0 = u / c.tiles_x * C::TY - C::K;
+      const CUtensorMap* m = reinterpret_cast<const CUtensorMap*>(c.maps);
+      expect_bytes(M.bar, zero_init ? 2 * bytes : 3 * bytes);
+      tma_field(M.r, m + 2, k0, j0, M.bar);
+      tma_field(M.d, m + 3, k0, j0, M.bar);
+      if (!zero_init) tma_field(M.e, m + c.flip, k0, j0, M.bar);
+      break;
+    }
+    tile_no[w] = t < ntiles ? t : ntiles;
+  };
+  if (lead) request(blockIdx.x, 0);
+  __syncthreads();
+  for (unsigned n = 0;; ++n) {
+    const int w = n & 1, t = tile_no[w];
+    if (t >= ntiles) return;
+    const Sor32Case& c = slot[w];
+    const int u = t - c.first, k0 = u % c.tiles_x * S::TK - S::HK, j0 = u / c.tiles_x * C::TY - C::K;
+    auto next = [&] { request(t + gridDim.x, w ^ 1); };
+    // next() runs before the tile's half-sweeps, whose barriers make slot[w ^ 1] visible
+    if (!sor32_tile_v11<C::TY, C::K, C::NY>(c.g, c.e_out, c.omega, zero_init, k0, j0, M, n & 1u, err, next)) return;
+  }
+}
+
+// a flag the form-11 kernels set when a wait gives up; mapped host memory, so
+// the host reads it without a device synchronisation
+unsigned* sor_error_flag(unsigned** dev) {
+  static unsigned *host = nullptr, *devp = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    void *h = nullptr, *d = nullptr;
+    if (cudaHostAlloc(&h, sizeof(unsigned), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) return;
+    host = static_cast<unsigned*>(h);
+    *host = 0u;
+    if (cudaHostGetDevicePointer(&d, h, 0) == cudaSuccess) devp = static_cast<unsigned*>(d);
+  });
+  *dev = devp;
+  return host;
+}
+
+// nothing was launched for want of a tensor map or of the flag: reported as a failed wait is
+bool g_no_maps = false;
+void sor_no_maps() { g_no_maps = true; }
+
+// tensor map of a colour-split array [2][ny][pk] with boxes of 64 columns, rows rows, both colours
+bool tile_map(CUtensorMap* m, const Geo32& g, const float* p, int rows) {
+  static PFN_cuTensorMapEncodeTiled_v12000 enc = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      enc = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
+  });
+  if (!enc) return false;
+  const cuuint64_t dims[3] = {(cuuint64_t)g.pk, (cuuint64_t)g.ny, 2};
+  const cuuint64_t strides[2] = {(cuuint64_t)g.pk * 4, (cuuint64_t)g.pk * 4 * g.ny};
+  const cuuint32_t box[3] = {64, (cuuint32_t)rows, 2}, one[3] = {1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(p), dims, strides, box, one,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+int sm_count() {
+  static const int n = [] {
+    int d = 0, v = 0;
+    cudaGetDevice(&d);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, d);
+    return v;
+  }();
+  return n;
+}
+
 // Tile shapes the autotuner chooses from.
 struct Sor32Config {
   int TY, K, NY, V;
@@ -874,9 +1240,15 @@ struct Sor32Config {
 // any stream capture
 template <class C>
 cudaError_t prepare_shape() {
+  if constexpr (C::V == 11) {
+    cudaError_t e = cudaFuncSetAttribute(k_sor32_tma<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_sor32_tma_batch<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem);
+  } else {
   cudaError_t e = cudaFuncSetAttribute(k_sor32_rb<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_sor32_rb_batch<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem);
+  }
 }
 
 template <class C>
@@ -889,10 +1261,6 @@ void launch_shape(cudaStream_t s, const Geo32& g, const float* e_in, float* e_ou
   }
   const int ncol = (g.nx + 1) / 2;
   dim3 grd((ncol + C::TK - 1) / C::TK, (g.ny + C::TY - 1) / C::TY);
-  if (!pdl) {
-    k_sor32_rb<C><<<grd, dim3(32, C::NY), C::smem, s>>>(g, e_in, e_out, r, invd, omega, zero_init);
-    return;
-  }
   cudaLaunchConfig_t lc{};
   lc.gridDim = grd;
   lc.blockDim = dim3(32, C::NY);
@@ -902,18 +1270,28 @@ void launch_shape(cudaStream_t s, const Geo32& g, const float* e_in, float* e_ou
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = at;
-  lc.numAttrs = 1;
-  cudaLaunchKernelEx(&lc, k_sor32_rb<C>, g, e_in, e_out, r, invd, omega, zero_init);
+  lc.numAttrs = pdl ? 1 : 0;
+  if constexpr (C::V == 11) {
+    const int ntiles = (int)(grd.x * grd.y);
+    lc.gridDim = dim3(std::min(ntiles, sm_count() * C::MINB));
+    CUtensorMap me, mr, md;
+    unsigned* err = nullptr;
+    sor_error_flag(&err);
+    constexpr int LY = C::TY + 2 * C::K;
+    if (!err || !tile_map(&me, g, e_in, LY) || !tile_map(&mr, g, r, LY) || !tile_map(&md, g, invd, LY)) {
+      sor_no_maps();
+      return;
+    }
+    cudaLaunchKernelEx(&lc, k_sor32_tma<C>, me, mr, md, g, e_out, omega, zero_init, (int)grd.x, ntiles, err);
+  } else {
+    cudaLaunchKernelEx(&lc, k_sor32_rb<C>, g, e_in, e_out, r, invd, omega, zero_init);
+  }
 }
 
 template <class C>
 void launch_shape_batch(cudaStream_t s, const Sor32Case* cases, int ncases, int total_tiles, int zero_init,
                         int pdl, int q) {
   if (total_tiles <= 0) return;
-  if (!pdl) {
-    k_sor32_rb_batch<C><<<total_tiles, dim3(32, C::NY), C::smem, s>>>(cases, ncases, zero_init, q);
-    return;
-  }
   cudaLaunchConfig_t lc{};
   lc.gridDim = dim3(total_tiles);
   lc.blockDim = dim3(32, C::NY);
@@ -923,8 +1301,19 @@ void launch_shape_batch(cudaStream_t s, const Sor32Case* cases, int ncases, int 
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = at;
-  lc.numAttrs = 1;
-  cudaLaunchKernelEx(&lc, k_sor32_rb_batch<C>, cases, ncases, zero_init, q);
+  lc.numAttrs = pdl ? 1 : 0;
+  if constexpr (C::V == 11) {
+    unsigned* err = nullptr;
+    sor_error_flag(&err);
+    if (!err) {
+      sor_no_maps();
+      return;
+    }
+    lc.gridDim = dim3(std::min(total_tiles, sm_count() * C::MINB));
+    cudaLaunchKernelEx(&lc, k_sor32_tma_batch<C>, cases, ncases, total_tiles, zero_init, q, err);
+  } else {
+    cudaLaunchKernelEx(&lc, k_sor32_rb_batch<C>, cases, ncases, zero_init, q);
+  }
 }
 
 template <class C>
@@ -951,7 +1340,9 @@ const Sor32Config kConfigs[] = {
     shape<Cfg<96, 16, 16, 6, 1>>(), shape<Cfg<64, 16, 16, 7, 1>>(), shape<Cfg<80, 16, 16, 7, 1>>(),
     shape<Cfg<64, 16, 16, 8, 1>>(), shape<Cfg<80, 16, 16, 8, 1>>(), shape<Cfg<80, 16, 16, 9, 1>>(),
     shape<Cfg<80, 16, 16, 10, 1>>(), shape<Cfg<64, 16, 16, 10, 1>>(), shape<Cfg<48, 8, 16, 10, 1>>(),
-    shape<Cfg<32, 8, 8, 10, 2>>(),
+    shape<Cfg<32, 8, 8, 10, 2>>(), shape<Cfg<88, 16, 12, 11, 1>>(), shape<Cfg<80, 16, 8, 11, 1>>(),
+    shape<Cfg<64, 16, 16, 11, 1>>(), shape<Cfg<32, 16, 16, 11, 1>>(), shape<Cfg<48, 24, 16, 11, 1>>(),
+    shape<Cfg<32, 24, 16, 11, 1>>(), shape<Cfg<32, 8, 16, 11, 1>>(),
 };
 constexpr int kNumConfigs = sizeof(kConfigs) / sizeof(kConfigs[0]);
 
@@ -990,6 +1381,24 @@ cudaError_t sor32_batch_prepare(int cfg) { return kConfigs[cfg].prepare(); }
 void launch_sor32_batch(cudaStream_t s, int cfg, const Sor32Case* cases_dev, int ncases, int total_tiles,
                         int zero_init, int pdl, int q) {
   kConfigs[cfg].launch_batch(s, cases_dev, ncases, total_tiles, zero_init, pdl, q);
+}
+
+bool sor32_failed() {
+  unsigned* dev = nullptr;
+  const unsigned* host = sor_error_flag(&dev);
+  return g_no_maps || (host && *(volatile const unsigned*)host != 0u);
+}
+
+size_t sor32_maps_bytes() { return 4 * sizeof(CUtensorMap); }
+
+bool sor32_case_maps(int cfg, const Geo32& g, const float* e, const float* eb, const float* r, const float* invd,
+                     void* out) {
+  const Sor32Config& c = kConfigs[cfg];
+  if (c.V != 11) return true;
+  CUtensorMap* m = static_cast<CUtensorMap*>(out);
+  const int rows = c.TY + 2 * c.K;
+  return tile_map(m, g, e, rows) && tile_map(m + 1, g, eb, rows) && tile_map(m + 2, g, r, rows) &&
+         tile_map(m + 3, g, invd, rows);
 }
 
 void launch_dc_residual_batch(cudaStream_t s, const DcCase* cases_dev, int ncases, int total_blocks) {

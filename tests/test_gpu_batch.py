@@ -180,3 +180,29 @@ def test_fused_batch_step_matches_single_contexts_bit_for_bit_before_the_pressur
         assert x["div_max"] <= c.div_tol * 1.001
         alone.close()
     B.close()
+
+
+@pytest.mark.parametrize("shape", range(37, 41))
+def test_batch_tiles_by_tma_match_the_tile_per_block_form_bit_for_bit(shape):
+    """The persistent sweep kernels (form 11) take the tiles of all cases in
+    one list, skipping cases whose sweeps of the round are done; with 16
+    half-sweeps a launch, as shape 33 (form 10, a tile per block), the rounds
+    are the same and so are the fields.  Grids of less than one tile up to
+    several, more tiles than SMs, an odd one; budgets on and off."""
+    from paper_2402_17337_gb300 import Batch, build
+    build.build()
+    cfgs = W.batch_small(3) + W.batch64()[:3]
+    cfgs[1].nx, cfgs[1].ny = 133, 67
+    out = []
+    for k in (33, shape):
+        ss = solvers(cfgs)
+        B = Batch(ss)
+        B.set_sor_shape(k)
+        B.step(1)
+        B.set_budgets(False)
+        B.step(1)
+        assert B.profile()["sor_shape"][1] == 16
+        out.append([s.get(f) for s in ss for f in ("u", "v", "p")])
+        B.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
