@@ -139,7 +139,8 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 
 // Geometry of one launch (host-computed).
 struct TcGeom {
-  int TW, R;           // pixels per tile row, rows per tile (TW R = 128)
+  int TW, R;           // pixels per tile row, rows per MMA (TW R = 128)
+  int RB;              // MMA rows a tile stacks (R = 1 only): RB accumulators from one halo box
   int copies, boxw;    // A boxes per channel group (1 or 3), pixels per box row
   int a_region;        // bytes of one A box in shared memory (padded to 128)
   int a_bytes, b_bytes, stage_bytes, tx_bytes, stages;
@@ -170,8 +171,8 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, vol
 template <bool RELU>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_conv3x3_tc(const __grid_constant__ CUtensorMap tmX, const bf16* __restrict__ wpk, const float* __restrict__ bias,
-                 bf16* __restrict__ Y, int ldy, int offy, float* __restrict__ yf, int H, int W, int Cout, TcGeom G,
-                 unsigned int* __restrict__ err) {
+                 bf16* __restrict__ Y, int ldy, int offy, float* __restrict__ yf, ConvAlso also, int H, int W, int Cout,
+                 TcGeom G, unsigned int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bar_full[TC_STAGES_MAX], bar_empty[TC_STAGES_MAX];
   __shared__ __align__(8) unsigned long long bar_tfull[2], bar_tempty[2];
@@ -216,7 +217,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     z = t % G.tiles_z;
     t /= G.tiles_z;
     x0 = (t % G.tiles_x) * G.TW;
-    y0 = (t / G.tiles_x) * G.R;
+    y0 = (t / G.tiles_x) * G.R * G.RB;
   };
 
   const int nc = G.nchunks, S = G.stages, nq = nmine * nc;
@@ -258,14 +259,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         if (!wait_or_abort(smem_u32(&bar_full[s]), (uint32_t)(q / S) & 1u, abort)) break;
         tc_fence_after();
         const uint32_t st = sbase + s * G.stage_bytes, d = tmem + (uint32_t)buf * half_cols;
+        for (int rb = 0; rb < G.RB; ++rb) {
 #pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-          const int dy = tap / 3, dx = tap % 3;
-          const uint32_t a =
-              G.copies == 1 ? st + (dy * G.boxw + dx) * 16 : st + dx * 2 * G.a_region + dy * G.TW * 16;
-          // B: [tap][8-row group of output channels][channel group][8 rows][16 bytes]
-          const uint32_t b = st + G.a_bytes + tap * G.NT * 32;
-          tc_mma(d, smem_desc(a, G.a_region, 128), smem_desc(b, 128, 256), idesc, (ch | tap) != 0);
+          for (int tap = 0; tap < 9; ++tap) {
+            const int dy = tap / 3, dx = tap % 3;
+            const uint32_t a =
+                G.copies == 1 ? st + ((rb + dy) * G.boxw + dx) * 16 : st + dx * 2 * G.a_region + dy * G.TW * 16;
+            // B: [tap][8-row group of output channels][channel group][8 rows][16 bytes]
+            const uint32_t b = st + G.a_bytes + tap * G.NT * 32;
+            tc_mma(d + (uint32_t)(rb * G.NT), smem_desc(a, G.a_region, 128), smem_desc(b, 128, 256), idesc,
+                   (ch | tap) != 0);
+          }
         }
         tc_commit(smem_u32(&bar_empty[s]));
         if (ch == nc - 1) tc_commit(smem_u32(&bar_tfull[buf]));
@@ -289,33 +293,75 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       tc_fence_after();
       int x0, y0, z;
       coords(li, x0, y0, z);
-      const int y = y0 + m / G.TW, x = x0 + m % G.TW, n0 = z * G.NT;
-      const bool valid = x < W && y < H;
-      const size_t p = (size_t)y * W + x;
-      for (int c0 = 0; c0 < G.NT; c0 += 16) {
-        float v[16];
-        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)buf * half_cols + (uint32_t)c0, v);
+      const int x = x0 + m % G.TW, n0 = z * G.NT;
+      for (int c0 = 0; c0 < G.NT && n0 + c0 < Cout; c0 += 16) {
         const int co = n0 + c0;
-        if (!valid || co >= Cout) continue;
+        float bv[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          float t = v[j] + (bias ? bias[co + j] : 0.f);
-          v[j] = RELU ? fmaxf(t, 0.f) : t;
-        }
-        uint4 o[2];
-        uint32_t* ow = reinterpret_cast<uint32_t*>(o);
+        for (int j = 0; j < 16; ++j) bv[j] = bias ? bias[co + j] : 0.f;
+        uint32_t below[8];  // the tile row before, for the pooling
+        for (int rb = 0; rb < G.RB; ++rb) {
+          const int y = y0 + m / G.TW + rb;
+          const bool valid = x < W && y < H;
+          const size_t p = (size_t)y * W + x;
+          float v[16];
+          tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)buf * half_cols + (uint32_t)(rb * G.NT + c0), v);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-          ow[j] = *reinterpret_cast<uint32_t*>(&h);
-        }
-        uint4* dst = reinterpret_cast<uint4*>(Y + p * ldy + offy + co);
-        dst[0] = o[0];
-        dst[1] = o[1];
-        if (yf) {
-          float4* f = reinterpret_cast<float4*>(yf + p * Cout + co);
+          for (int j = 0; j < 16; ++j) {
+            const float t = v[j] + bv[j];
+            v[j] = RELU ? fmaxf(t, 0.f) : t;
+          }
+          if (yf && valid && co == 0) yf[p] = v[0];
+          uint4 o[2];
+          uint32_t* ow = reinterpret_cast<uint32_t*>(o);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) f[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+          for (int j = 0; j < 8; ++j) {
+            __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+            ow[j] = *reinterpret_cast<uint32_t*>(&h);
+          }
+          if (Y && valid) {
+            uint4* dst = reinterpret_cast<uint4*>(Y + p * ldy + offy + co);
+            dst[0] = o[0];
+            dst[1] = o[1];
+          }
+          if (also.up && valid) {
+            // nearest 2x upsampling: the pixel's four copies
+            uint4* d0 = reinterpret_cast<uint4*>(also.up + ((size_t)(2 * y) * (2 * W) + 2 * x) * also.ldu + co);
+            uint4* d1 = reinterpret_cast<uint4*>(also.up + ((size_t)(2 * y) * (2 * W) + 2 * x + 1) * also.ldu + co);
+            const size_t row = (size_t)(2 * W) * also.ldu / 8;  // uint4 per image row
+            d0[0] = d1[0] = d0[row] = d1[row] = o[0];
+            d0[1] = d1[1] = d0[row + 1] = d1[row + 1] = o[1];
+          }
+          if (also.pool) {
+            if (rb & 1) {
+              // 2x2 average of the stored (BF16) values: lane pairs hold x and x + 1; the even lane takes
+              // channels 0-7, the odd lane 8-15 (W and H are even, so a pair is inside or outside as a whole)
+              const bool odd = lane & 1;
+              uint32_t lo[4], hi[4], oth_lo[4], oth_hi[4];
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                lo[j] = odd ? below[j + 4] : below[j];
+                hi[j] = odd ? ow[j + 4] : ow[j];
+                oth_lo[j] = __shfl_xor_sync(0xffffffffu, odd ? below[j] : below[j + 4], 1);
+                oth_hi[j] = __shfl_xor_sync(0xffffffffu, odd ? ow[j] : ow[j + 4], 1);
+              }
+              uint4 r;
+              uint32_t* rw = reinterpret_cast<uint32_t*>(&r);
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                auto f2 = [](uint32_t w) { return __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&w)); };
+                const float2 a = f2(odd ? oth_lo[j] : lo[j]), b = f2(odd ? lo[j] : oth_lo[j]);
+                const float2 c = f2(odd ? oth_hi[j] : hi[j]), d = f2(odd ? hi[j] : oth_hi[j]);
+                __nv_bfloat162 h = __floats2bfloat162_rn(0.25f * (a.x + b.x + c.x + d.x), 0.25f * (a.y + b.y + c.y + d.y));
+                rw[j] = *reinterpret_cast<uint32_t*>(&h);
+              }
+              if (valid)
+                *reinterpret_cast<uint4*>(also.pool + ((size_t)(y / 2) * (W / 2) + x / 2) * also.ldp + co + (odd ? 8 : 0)) = r;
+            } else {
+#pragma unroll
+              for (int j = 0; j < 8; ++j) below[j] = ow[j];
+            }
+          }
         }
       }
       tc_fence_before();
@@ -483,22 +529,37 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 // whose weights are w[Cin][9][Cout]: W'[co][tap][ci] = w[ci][8 - tap][co].
 // One launch packs every job (blockIdx.y = job).
 __global__ void k_pack_conv_weights(const PackJob* __restrict__ jobs) {
+  // a thread packs the 8 channels (16 bytes) of one output channel and tap: a
+  // 16-byte load and store, and 32-bit index arithmetic (one element a thread
+  // with 64-bit divisions took 28.8 us for the 32/64/128/128 network)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const PackJob J = jobs[blockIdx.y];
   const int Cin = J.cin, Cout = J.cout, NT = J.nt, nchunks = Cin / 16;
-  const long n = (long)J.ntiles * nchunks * 9 * NT * 16;
-  for (long k = blockIdx.x * (long)blockDim.x + threadIdx.x; k < n; k += (long)gridDim.x * blockDim.x) {
-    const int e = (int)(k & 7), row = (int)((k >> 3) & 7), g = (int)((k >> 6) & 1);
-    long r = k >> 7;
-    const int ngrp = (int)(r % (NT / 8));
+  const int n = J.ntiles * nchunks * 9 * NT * 2;
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+    const int row = k & 7, g = (k >> 3) & 1;
+    int r = k >> 4;
+    const int ngrp = r % (NT / 8);
     r /= NT / 8;
-    const int tap = (int)(r % 9);
+    const int tap = r % 9;
     r /= 9;
-    const int ch = (int)(r % nchunks), t = (int)(r / nchunks);
-    const int co = t * NT + ngrp * 8 + row, ci = ch * 16 + g * 8 + e;
-    bf16 v = __float2bfloat16_rn(0.f);
-    if (co < Cout)
-      v = J.flip ? J.w[((size_t)ci * 9 + (8 - tap)) * Cout + co] : J.w[((size_t)co * 9 + tap) * Cin + ci];
-    J.wpk[k] = v;
+    const int ch = r % nchunks, t = r / nchunks;
+    const int co = t * NT + ngrp * 8 + row, ci = ch * 16 + g * 8;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (co < Cout) {
+      if (!J.flip) {
+        v = *reinterpret_cast<const uint4*>(J.w + ((size_t)co * 9 + tap) * Cin + ci);
+      } else {
+        unsigned short h[8];
+        const unsigned short* w = reinterpret_cast<const unsigned short*>(J.w);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) h[e] = w[((size_t)(ci + e) * 9 + (8 - tap)) * Cout + co];
+        v = make_uint4(h[0] | (unsigned)h[1] << 16, h[2] | (unsigned)h[3] << 16, h[4] | (unsigned)h[5] << 16,
+                       h[6] | (unsigned)h[7] << 16);
+      }
+    }
+    reinterpret_cast<uint4*>(J.wpk)[k] = v;
   }
 }
 
@@ -585,8 +646,17 @@ PackJob pack_job(int Cin, int Cout, const bf16* w, bf16* wpk, bool flip) {
 }
 
 void pack_conv_weights(cudaStream_t s, const PackJob* jobs_dev, int njobs, long max_elems) {
-  long b = (max_elems + 255) / 256;
-  k_pack_conv_weights<<<dim3((unsigned)(b > 1024 ? 1024 : b), (unsigned)njobs), 256, 0, s>>>(jobs_dev);
+  const long b = (max_elems / 8 + 255) / 256;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3((unsigned)(b > 256 ? 256 : (b < 1 ? 1 : b)), (unsigned)njobs);
+  lc.blockDim = dim3(256);
+  lc.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  cudaLaunchKernelEx(&lc, k_pack_conv_weights, jobs_dev);
 }
 
 int conv3x3_wgrad(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* Gd, int ldg, int offg, const bf16* X,
@@ -685,7 +755,7 @@ bool conv_tc_failed() {
 }
 
 int conv3x3(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* X, int ldx, int offx, const bf16* wpk,
-            const float* bias, bf16* Y, int ldy, int offy, bool relu, float* yf) {
+            const float* bias, bf16* Y, int ldy, int offy, bool relu, float* yf, ConvAlso also, bool* pooled) {
   if (Cin % 16 || Cout % 16 || ldx % 8 || offx % 8 || ldy % 8 || offy % 8) {
     set_last_error("convolution channel counts and slices must be multiples of 16 and 8");
     return -1;
@@ -702,19 +772,36 @@ int conv3x3(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* X, int 
   G.R = TC_M / G.TW;
   G.copies = G.R == 1 ? 1 : 3;
   G.boxw = G.R == 1 ? G.TW + 2 : G.TW;
-  const int rows = G.R + 2;
+  G.NT = conv_tile_channels(Cout);
+  // With one image row per MMA a tile stacks RB rows: one halo box of RB + 2
+  // rows serves RB accumulators, where RB tiles would load 3 RB rows.  TMA
+  // moves these boxes 16 bytes (a pixel's 8 channels) at a time, which is
+  // what bounds the narrow layers: 16 -> 16 channels on 512x1024, 25.6 us with
+  // RB = 1, 16.8 us with 4 (8 leaves too few loads in flight: 1 CTA an SM).
+  // The accumulators (two sets) stay within 256 columns, and a layer keeps a
+  // tile for every SM.
+  G.RB = 1;
+  if (G.R == 1)
+    for (int rb = 4; rb > 1 && G.RB == 1; rb /= 2)
+      if (rb * G.NT <= 128 && (long)((W + TC_M - 1) / TC_M) * ((H + rb - 1) / rb) >= 152) G.RB = rb;
+  // the pooling in the epilogue takes two rows of a tile
+  if (also.pool && G.R == 1 && G.RB == 1 && 2 * G.NT <= 256) G.RB = 2;
+  const bool pool = also.pool && G.R == 1 && G.RB % 2 == 0 && H % 2 == 0 && W % 2 == 0;
+  if (!pool) also.pool = nullptr;
+  if (pooled) *pooled = pool;
+  const int rows = G.R * G.RB + 2;
   G.a_region = (rows * G.boxw * 16 + 127) / 128 * 128;
   G.a_bytes = G.copies * 2 * G.a_region;
-  G.NT = conv_tile_channels(Cout);
   G.b_bytes = 9 * G.NT * 32;
   G.stage_bytes = (G.a_bytes + G.b_bytes + 1023) / 1024 * 1024;
   G.tx_bytes = G.copies * 2 * rows * G.boxw * 16 + G.b_bytes;
-  G.tmem_cols = pow2_at_least(2 * G.NT < 64 ? 64 : 2 * G.NT);  // two accumulators, each at least 32 columns
+  // two sets of RB accumulators, each set at least 32 columns
+  G.tmem_cols = pow2_at_least(2 * G.RB * G.NT < 64 ? 64 : 2 * G.RB * G.NT);
   G.nchunks = Cin / 16;
   G.stages = 3 * G.stage_bytes + 1024 <= TC_SMEM_MAX ? 3 : 2;
   G.tiles_x = (W + G.TW - 1) / G.TW;
   G.tiles_z = (Cout + G.NT - 1) / G.NT;
-  G.ntiles = G.tiles_x * ((H + G.R - 1) / G.R) * G.tiles_z;
+  G.ntiles = G.tiles_x * ((H + G.R * G.RB - 1) / (G.R * G.RB)) * G.tiles_z;
   // dynamic shared memory: the stages plus alignment slack, at least
   // tmem_min_smem
   int smem = G.stages * G.stage_bytes + 1024;
@@ -766,7 +853,7 @@ int conv3x3(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* X, int 
   at[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = at;
   lc.numAttrs = 1;
-  if (cudaLaunchKernelEx(&lc, kern, map, wpk, bias, Y, ldy, offy, yf, H, W, Cout, G, err_dev) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&lc, kern, map, wpk, bias, Y, ldy, offy, yf, also, H, W, Cout, G, err_dev) != cudaSuccess) {
     set_last_error("convolution launch failed");
     return -1;
   }

@@ -885,8 +885,8 @@ __device__ __forceinline__ void setup_v11(const TileMem<S>& M, int NY) {
 // next() is called by one thread once the tile has been picked up from shared
 // memory (it requests the next one).  False if the wait gave up.
 template <int TY, int K, int NY, class Next>
-__device__ __forceinline__ bool sor32_tile_v11(const Geo32& g, float* __restrict__ e_out, float omega, int zero_init,
-                                               int k0, int j0, const TileMem<Sor32ShapeV11<TY, K, NY>>& M,
+__device__ __forceinline__ bool sor32_tile_v11(const Geo32& g, float* __restrict__ e_out, float omega, float omc,
+                                               int zero_init, int k0, int j0, const TileMem<Sor32ShapeV11<TY, K, NY>>& M,
                                                unsigned parity, unsigned* err, Next next) {
   using S = Sor32ShapeV11<TY, K, NY>;
   constexpr int HK = S::HK, TK = S::TK, LY = S::LY, RPT = S::RPT;
@@ -894,7 +894,6 @@ __device__ __forceinline__ bool sor32_tile_v11(const Geo32& g, float* __restrict
   float2(*se)[NY + 2][2][32] = reinterpret_cast<float2(*)[NY + 2][2][32]>(M.edge);  // run w at [w + 1]
   const int nx = g.nx, ny = g.ny, pk = g.pk;
   const int tx = threadIdx.x, ty = threadIdx.y, ly0 = ty * RPT;
-  const float omc = 1.f - omega;
   const int kp = k0 + 2 * tx;  // first packed column of the pair; rows hold pk (even) entries
   const bool pair_ok = kp >= 0 && kp < pk;
   float ev[2][RPT][2], av[2][RPT][2], bv[2][RPT][2], cE[2][2], cW[2][2], cN[RPT], cS[RPT];
@@ -1088,7 +1087,7 @@ template <class C>
 __global__ void __launch_bounds__(32 * C::NY, C::MINB)
     k_sor32_tma(const __grid_constant__ CUtensorMap me, const __grid_constant__ CUtensorMap mr,
                 const __grid_constant__ CUtensorMap md, const Geo32 g, float* __restrict__ e_out, float omega,
-                int zero_init, int nbx, int ntiles, unsigned* __restrict__ err) {
+                float omc, int zero_init, int nbx, int ntiles, unsigned* __restrict__ err) {
   using S = Sor32ShapeV11<C::TY, C::K, C::NY>;
   extern __shared__ __align__(1024) unsigned char smem_tile[];
   const TileMem<S> M(smem_tile);
@@ -1122,7 +1121,7 @@ __global__ void __launch_bounds__(32 * C::NY, C::MINB)
       fetch_rd(t);
       if (!zero_init) fetch_e(t);
     };
-    if (!sor32_tile_v11<C::TY, C::K, C::NY>(g, e_out, omega, zero_init, k0, j0, M, n & 1u, err, next)) return;
+    if (!sor32_tile_v11<C::TY, C::K, C::NY>(g, e_out, omega, omc, zero_init, k0, j0, M, n & 1u, err, next)) return;
   }
 }
 
@@ -1173,7 +1172,7 @@ __global__ void __launch_bounds__(32 * C::NY, C::MINB)
     const int u = t - c.first, k0 = u % c.tiles_x * S::TK - S::HK, j0 = u / c.tiles_x * C::TY - C::K;
     auto next = [&] { request(t + gridDim.x, w ^ 1); };
     // next() runs before the tile's half-sweeps, whose barriers make slot[w ^ 1] visible
-    if (!sor32_tile_v11<C::TY, C::K, C::NY>(c.g, c.e_out, c.omega, zero_init, k0, j0, M, n & 1u, err, next)) return;
+    if (!sor32_tile_v11<C::TY, C::K, C::NY>(c.g, c.e_out, c.omega, 1.f - c.omega, zero_init, k0, j0, M, n & 1u, err, next)) return;
   }
 }
 
@@ -1282,7 +1281,7 @@ void launch_shape(cudaStream_t s, const Geo32& g, const float* e_in, float* e_ou
       sor_no_maps();
       return;
     }
-    cudaLaunchKernelEx(&lc, k_sor32_tma<C>, me, mr, md, g, e_out, omega, zero_init, (int)grd.x, ntiles, err);
+    cudaLaunchKernelEx(&lc, k_sor32_tma<C>, me, mr, md, g, e_out, omega, 1.f - omega, zero_init, (int)grd.x, ntiles, err);
   } else {
     cudaLaunchKernelEx(&lc, k_sor32_rb<C>, g, e_in, e_out, r, invd, omega, zero_init);
   }

@@ -9,12 +9,23 @@ namespace nn {
 
 using bf16 = __nv_bfloat16;
 
+// What a convolution writes besides its output: its 2x2 average (pool, ldp
+// channels a pixel) and its nearest 2x upsampling (up, ldu channels a pixel).
+struct ConvAlso {
+  bf16* pool = nullptr;
+  int ldp = 0;
+  bf16* up = nullptr;
+  int ldu = 0;
+};
 // Y = act(conv3x3(X, W) + bias), zero padding, on the tcgen05 tensor cores
 // (k_conv_tc.cu); Cin, Cout % 16 == 0, ldx, offx, ldy, offy % 8 == 0; wpk:
-// the weights packed by pack_conv_weights; yf: optional dense FP32 copy of the
-// output [H][W][Cout].  Returns 0, or -1 with ibm_last_error set.
+// the weights packed by pack_conv_weights; Y may be null (only the other
+// outputs are wanted); yf: optional FP32 copy of output channel 0, [H][W].
+// *pooled: whether also.pool was written (a layer of narrow tiles cannot; the
+// caller then pools).  Returns 0, or -1 with ibm_last_error set.
 int conv3x3(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* X, int ldx, int offx, const bf16* wpk,
-            const float* bias, bf16* Y, int ldy, int offy, bool relu, float* yf);
+            const float* bias, bf16* Y, int ldy, int offy, bool relu, float* yf, ConvAlso also = ConvAlso{},
+            bool* pooled = nullptr);
 // elements of the packed weights of a convolution with Cin inputs and Cout
 // outputs, and the packing of w[Cout][9][Cin] (flip: of the data-gradient
 // operator of a layer with weights w[Cin][9][Cout], W'[co][tap][ci] =
@@ -35,14 +46,13 @@ bool conv_tc_failed();
 // cores (k_conv_tc.cu); Cout <= 128; returns 0, or -1 with ibm_last_error set
 int conv3x3_wgrad(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* G, int ldg, int offg, const bf16* X,
                    int ldx, int offx, float* dW);
-void relu_grad(cudaStream_t s, long npix, int C, bf16* G, int ldg, int offg, const bf16* Y, int ldy, int offy);
 void avgpool(cudaStream_t s, int H, int W, int C, const bf16* X, int ldx, int offx, bf16* Y, int ldy, int offy);
 void avgpool_grad(cudaStream_t s, int H, int W, int C, const bf16* dY, int ldy, int offy, bf16* dX, int ldx, int offx,
                   bool acc);
-void upsample(cudaStream_t s, int H, int W, int C, const bf16* X, int ldx, int offx, bf16* Y, int ldy, int offy);
 void upsample_grad(cudaStream_t s, int H, int W, int C, const bf16* dY, int ldy, int offy, bf16* dX, int ldx, int offx,
                    bool acc);
-void bias_grad(cudaStream_t s, long npix, int C, const bf16* G, int ldg, int offg, float* db);
+void relu_bias_grad(cudaStream_t s, long npix, int C, bf16* G, int ldg, int offg, const bf16* Y, int ldy, int offy,
+                    float* db);
 void mse(cudaStream_t s, long npix, const float* out, int ldo, const float* target, const float* mask, float inv_count,
          bf16* dout, int ldd, double* loss);
 void adam(cudaStream_t s, long n, float* w, const float* g, float* m, float* v, bf16* wb, float lr, float b1, float b2,

@@ -135,7 +135,7 @@ int ensure_acts(ibm_unet* n, int H, int W) {
   B(&n->ge3, px3, w[3]);
   B(&n->out, px0, 16);
   B(&n->gout, px0, 16);
-  rc |= dalloc(n, (void**)&n->outf, px0 * 16 * sizeof(float));
+  rc |= dalloc(n, (void**)&n->outf, px0 * sizeof(float));
   if (rc) return IBM_E_CUDA;
   n->H = H;
   n->W = W;
@@ -197,35 +197,50 @@ void ensure_packed(ibm_unet* n, cudaStream_t s) {
   n->wdirty = false;
 }
 
-int forward(ibm_unet* n, cudaStream_t s) {
+// outp: FP32 output [H][W]; train: keep every activation the backward pass reads
+int forward(ibm_unet* n, cudaStream_t s, float* outp, bool train) {
   const int* w = n->w;
   std::vector<Edge> E = edges(n);
   ensure_packed(n, s);
   int rc = 0;
-  auto run = [&](const Edge& e) {
+  auto run = [&](const Edge& e, ConvAlso also = ConvAlso{}, bool keep = true) {
     const Conv& c = n->conv[e.conv];
     Level& L = n->lv[level_of(n, e.x)];
-    rc |= conv3x3(s, L.H, L.W, c.cin, c.cout, e.x.p, e.x.ld, e.x.off, n->wpk + c.pk, n->pw + c.b, e.y.p, e.y.ld,
-                  e.y.off, c.relu, e.conv == 14 ? n->outf : nullptr);
+    bool pooled = false;
+    rc |= conv3x3(s, L.H, L.W, c.cin, c.cout, e.x.p, e.x.ld, e.x.off, n->wpk + c.pk, n->pw + c.b,
+                  keep ? e.y.p : nullptr, e.y.ld, e.y.off, c.relu, e.conv == 14 ? outp : nullptr, also, &pooled);
+    return pooled;
+  };
+  // each level's output is upsampled into the concatenation above it by the convolution that makes it
+  auto up_of = [&](int l) {
+    ConvAlso a;
+    a.up = n->lv[l].cat;
+    a.ldu = n->lv[l].cup + w[l];
+    return a;
   };
   // encoder
   for (int l = 0; l < 4; ++l) {
-    if (l > 0) {
-      Level& P = n->lv[l - 1];
-      avgpool(s, P.H, P.W, w[l - 1], P.cat, P.cup + w[l - 1], P.cup, n->lv[l].in, w[l - 1], 0);
-    }
     run(E[2 * l]);
-    run(E[2 * l + 1]);
+    if (l == 3) {
+      run(E[7], up_of(2), train);
+      break;
+    }
+    ConvAlso a;
+    a.pool = n->lv[l + 1].in;
+    a.ldp = w[l];
+    Level& L = n->lv[l];
+    if (!run(E[2 * l + 1], a))
+      avgpool(s, L.H, L.W, w[l], L.cat, L.cup + w[l], L.cup, n->lv[l + 1].in, w[l], 0);
   }
   // decoder
   for (int l = 2, k = 8; l >= 0; --l, k += 2) {
-    Level& L = n->lv[l];
-    const bf16* src = l == 2 ? n->e3 : n->lv[l + 1].d;
-    upsample(s, L.H, L.W, L.cup, src, L.cup, 0, L.cat, L.cup + w[l], 0);
     run(E[k]);
-    run(E[k + 1]);
+    if (l > 0)
+      run(E[k + 1], up_of(l - 1), train);
+    else
+      run(E[k + 1]);
   }
-  run(E[14]);
+  run(E[14], ConvAlso{}, false);
   return rc;
 }
 
@@ -236,9 +251,8 @@ int conv_backward(ibm_unet* n, const Edge& e, cudaStream_t s, bool need_dx) {
   Level& L = n->lv[level_of(n, e.x)];
   Act gy = grad_of(n, e.y), gx = grad_of(n, e.x);
   const long npix = (long)L.H * L.W;
-  if (c.relu) relu_grad(s, npix, c.cout, gy.p, gy.ld, gy.off, e.y.p, e.y.ld, e.y.off);
+  relu_bias_grad(s, npix, c.cout, gy.p, gy.ld, gy.off, c.relu ? e.y.p : nullptr, e.y.ld, e.y.off, n->grad + c.b);
   if (conv3x3_wgrad(s, L.H, L.W, c.cin, c.cout, gy.p, gy.ld, gy.off, e.x.p, e.x.ld, e.x.off, n->grad + c.w)) return -1;
-  bias_grad(s, npix, c.cout, gy.p, gy.ld, gy.off, n->grad + c.b);
   if (need_dx)
     return conv3x3(s, L.H, L.W, c.cout, c.cin, gy.p, gy.ld, gy.off, n->wpkf + c.pkf, nullptr, gx.p, gx.ld, gx.off,
                    false, nullptr);
@@ -382,9 +396,9 @@ int ibm_unet_grads(const ibm_unet* n, float* host, long long count) {
 }  // extern "C"
 
 namespace ibm {
-// kernels one forward pass launches: input packing, 15 convolutions, 3
-// poolings, 3 upsamplings
-int unet_forward_launches() { return 1 + 15 + 3 + 3; }
+// kernels one forward pass launches: input packing and 15 convolutions (a
+// level narrower than 128 pixels pools in a kernel of its own)
+int unet_forward_launches() { return 1 + 15; }
 }  // namespace ibm
 
 extern "C" {
@@ -397,9 +411,7 @@ int ibm_unet_forward(ibm_unet* n, const float* feat, int H, int W, float* out, v
   if (rc) return rc;
   if (conv_tc_failed()) return ufail(IBM_E_TIMEOUT, "a U-Net convolution gave up a bounded wait earlier");
   pack_input(s, (long)H * W, 4, 16, feat, n->lv[0].in);
-  if (forward(n, s)) return IBM_E_CUDA;
-  UCUDA(cudaMemcpy2DAsync(out, sizeof(float), n->outf, 16 * sizeof(float), sizeof(float), (size_t)H * W,
-                          cudaMemcpyDeviceToDevice, s));
+  if (forward(n, s, out, false)) return IBM_E_CUDA;
   UCUDA(cudaGetLastError());
   return IBM_OK;
 }
@@ -412,11 +424,11 @@ int ibm_unet_train_step(ibm_unet* n, const float* feat, const float* target, int
   int rc = ensure_acts(n, H, W);
   if (rc) return rc;
   pack_input(s, (long)H * W, 4, 16, feat, n->lv[0].in);
-  if (forward(n, s)) return IBM_E_CUDA;
+  if (forward(n, s, n->outf, true)) return IBM_E_CUDA;
   UCUDA(cudaMemsetAsync(n->grad, 0, n->nparam * 4, s));
   UCUDA(cudaMemsetAsync(n->loss_d, 0, 8, s));
   const long npix = (long)H * W;
-  mse(s, npix, n->outf, 16, target, nullptr, 1.f / (float)npix, n->gout, 16, n->loss_d);
+  mse(s, npix, n->outf, 1, target, nullptr, 1.f / (float)npix, n->gout, 16, n->loss_d);
   if (backward(n, s)) return IBM_E_CUDA;
   if (apply) {
     n->adam_t += 1;
