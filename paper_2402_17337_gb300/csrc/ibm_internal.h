@@ -272,27 +272,32 @@ struct MgLevel {
   const float* invd;     // reciprocal diagonal
   int cur;               // buffer holding the current correction
 };
-int mg_coarse_max();
-constexpr int kTailLevels = 8, kTailCells = 5632;  // 44 KB of shared memory: a larger level costs one CTA more than its launches
-struct MgTail {             // the small levels, run by one CTA (k_mg_tail)
-  MgLevel lv[kTailLevels];  // lv[0] = first tail level, its r from global memory
-  int off[kTailLevels];     // offsets of each level's cells in shared memory
-  int n;                    // number of tail levels (the last is solved by SOR)
+// the small levels, run by one CTA (k_mg_low)
+constexpr int kLowLevels = 12, kLowSmem = 200 * 1024;
+struct MgLowLevel {
+  int nx, ny, pk;
+  int off, coff;   // first float in shared memory, and in the constants
+  const float* r;  // (the first level's is read)
+};
+struct MgLow {
+  MgLowLevel lv[kLowLevels];  // lv[0]: its r from global memory
+  int n, smem;                // levels, bytes of shared memory
+  int nzero, nconst;          // floats that start at zero; floats of constants behind them
+  // per level: pE, pW, wx, ax, ox (nx each; ox as integers), pN, pS, wy, ay, oy (ny each), invd [ny][nx]
+  const float* consts;
   float omega_c;
   int sweeps_c;
 };
-cudaError_t prepare_mg_tail();  // dynamic shared memory limit, once, outside graph capture
-void launch_mg_tail(cudaStream_t s, const MgTail& T, float* e_top);
+bool mg_low_layout(MgLow& T);
+void launch_mg_low(cudaStream_t s, const MgLow& T, float* e_top);
 size_t fcg_scalars_bytes();  // device scalars of the FCG iteration (zero-initialised)
 void launch_mg_restrict(cudaStream_t s, const MgLevel& F, const float* ef, const MgLevel& C);
 void launch_mg_prolong(cudaStream_t s, const MgLevel& C, const float* ec, const MgLevel& F, float* ef);
-void launch_mg_coarse(cudaStream_t s, const MgLevel& L, float* e_out, float omega, int sweeps);
 int sor32_find_shape(int rows_per_tile, int half_sweeps, int form);
 void launch_fcg_dot(cudaStream_t s, const MgLevel& L, const float* dxv, const float* dyv, const float* z,
                     const float* q, void* sc);
-void launch_fcg_dir(cudaStream_t s, const MgLevel& L, const float* z, float* p, const void* sc, int first);
-void launch_fcg_apply(cudaStream_t s, const MgLevel& L, const float* dxv, const float* dyv, const float* p,
-                      const float* r, float* q, void* sc);
+void launch_fcg_apply(cudaStream_t s, const MgLevel& L, const float* dxv, const float* dyv, const float* z,
+                      const float* p_old, float* p, const float* r, float* q, void* sc, int first);
 void launch_fcg_update(cudaStream_t s, const MgLevel& L, const float* p, const float* q, float* x, float* r,
                        const void* sc);
 

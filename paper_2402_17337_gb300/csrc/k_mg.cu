@@ -22,197 +22,352 @@
 // Smoothing is red-black Gauss-Seidel by the FP32 tile kernel of k_mixed.cu;
 // the coarsest level (a few dozen cells) is solved by red-black SOR inside
 // one CTA.  All arrays use the colour-split layout rb_at of the FP32 sweeps.
+#include <algorithm>
+#include <cstdint>
+#include <mutex>
+
 #include "ibm_internal.h"
 
 namespace ibm {
 
 namespace {
 
-__device__ inline float level_res(const MgLevel& L, const float* __restrict__ e, int i, int j) {
-  const int nx = L.g.nx, ny = L.g.ny, pk = L.g.pk;
-  const float x = e[rb_at(i, j, ny, pk)];
-  const float xE = i < nx - 1 ? e[rb_at(i + 1, j, ny, pk)] : x;
-  const float xW = i > 0 ? e[rb_at(i - 1, j, ny, pk)] : x;
-  const float xN = j < ny - 1 ? e[rb_at(i, j + 1, ny, pk)] : x;
-  const float xS = j > 0 ? e[rb_at(i, j - 1, ny, pk)] : x;
-  float Le = L.pE[i] * (xE - x);
-  Le = fmaf(L.pW[i], xW - x, Le);
-  Le = fmaf(L.g.pN[j], xN - x, Le);
-  Le = fmaf(L.g.pS[j], xS - x, Le);
-  return L.r[rb_at(i, j, ny, pk)] - Le;
+// Every kernel of a cycle is a programmatic dependent launch: it waits for the
+// one before it and then lets the next one be scheduled (direct launches; a
+// graph per iteration, as the cycle ran before, left about 100 us of a
+// 360 us iteration on 2048x1024 between kernels).
+__device__ __forceinline__ void pdl_enter() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... KArgs, typename... Args>
+void launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = grid;
+  lc.blockDim = block;
+  lc.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  cudaLaunchKernelEx(&lc, k, static_cast<KArgs>(args)...);
 }
 
-// one thread per coarse cell: residual of its (up to four) children, restricted
+// One thread per coarse cell: residual of its (up to four) children,
+// restricted.  Packed column I of the fine level holds the children's columns
+// 2I and 2I + 1, one of each colour in each row, so the cells and their W and
+// E neighbours are entries I - 1, I and I + 1 of the two colour rows: of the
+// fine correction a warp reads whole lines (per-cell index arithmetic and its
+// loads took 14.0 us for 2048x1024).
 __global__ void k_mg_restrict(const MgLevel F, const float* __restrict__ ef, MgLevel C) {
+  pdl_enter();
   const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
   if (I >= C.g.nx || J >= C.g.ny) return;
+  const int nx = F.g.nx, ny = F.g.ny, pk = F.g.pk, i0 = 2 * I;
+  const bool two = i0 + 1 < nx;
+  // row j: cells 2I (colour j & 1) and 2I + 1 (the other colour)
+  auto at2 = [&](const float* p, int j) {
+    const size_t a = ((size_t)(j & 1) * ny + j) * pk + I, b = ((size_t)((j & 1) ^ 1) * ny + j) * pk + I;
+    return make_float2(p[a], two ? p[b] : 0.f);
+  };
   float acc = 0.f;
+  const float2 zero = make_float2(0.f, 0.f);
+  const int j0 = 2 * J;
+  float2 s = j0 > 0 ? at2(ef, j0 - 1) : zero, x = at2(ef, j0), n;
+#pragma unroll
   for (int b = 0; b < 2; ++b) {
-    const int j = 2 * J + b;
-    if (j >= F.g.ny) break;
-    float row = 0.f;
-    for (int a = 0; a < 2; ++a) {
-      const int i = 2 * I + a;
-      if (i >= F.g.nx) break;
-      row = fmaf(F.wx[i], level_res(F, ef, i, j), row);
+    const int j = j0 + b;
+    if (j >= ny) break;
+    n = j + 1 < ny ? at2(ef, j + 1) : zero;
+    // W of 2I: cell 2I - 1, the other colour at packed column I - 1; E of 2I + 1: cell 2I + 2, at I + 1
+    const float w = I > 0 ? ef[((size_t)((j & 1) ^ 1) * ny + j) * pk + I - 1] : 0.f;
+    const float e = i0 + 2 < nx ? ef[((size_t)(j & 1) * ny + j) * pk + I + 1] : 0.f;
+    const float2 r = at2(F.r, j);
+    const float cN = F.g.pN[j], cS = F.g.pS[j];
+    // a neighbour outside the grid has coefficient zero
+    float L0 = F.pE[i0] * (x.y - x.x);
+    L0 = fmaf(F.pW[i0], w - x.x, L0);
+    L0 = fmaf(cN, n.x - x.x, L0);
+    L0 = fmaf(cS, s.x - x.x, L0);
+    float row = F.wx[i0] * (r.x - L0);
+    if (two) {
+      float L1 = F.pE[i0 + 1] * (e - x.y);
+      L1 = fmaf(F.pW[i0 + 1], x.x - x.y, L1);
+      L1 = fmaf(cN, n.y - x.y, L1);
+      L1 = fmaf(cS, s.y - x.y, L1);
+      row = fmaf(F.wx[i0 + 1], r.y - L1, row);
     }
     acc = fmaf(F.wy[j], row, acc);
+    s = x;
+    x = n;
   }
   C.r[rb_at(I, J, C.g.ny, C.g.pk)] = acc;
 }
 
-// one thread per fine cell: parent I = i/2 and neighbour I + ox_i (ox_i in
+// One thread per coarse column I and fine row j: the fine cells 2I and 2I + 1.
+// Fine cell i takes parent i / 2 and its neighbour i / 2 + ox_i (ox_i in
 // {-1, 0, +1}, 0 at the boundary) with weight ax_i on the neighbour, the same
-// in y
+// in y.
 __global__ void k_mg_prolong(const MgLevel C, const float* __restrict__ ec, MgLevel F, float* __restrict__ ef) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= F.g.nx || j >= F.g.ny) return;
-  const int I = i >> 1, J = j >> 1, I2 = I + F.ox[i], J2 = J + F.oy[j];
-  const float ax = F.ax[i], ay = F.ay[j];
-  const int ny = C.g.ny, pk = C.g.pk;
-  const float e00 = ec[rb_at(I, J, ny, pk)], e10 = ec[rb_at(I2, J, ny, pk)];
-  const float e01 = ec[rb_at(I, J2, ny, pk)], e11 = ec[rb_at(I2, J2, ny, pk)];
-  const float lo = fmaf(ax, e10 - e00, e00), hi = fmaf(ax, e11 - e01, e01);
-  ef[rb_at(i, j, F.g.ny, F.g.pk)] += fmaf(ay, hi - lo, lo);
-}
-
-// coarsest level: red-black SOR from e = 0 in shared memory, one CTA
-constexpr int kCoarseMax = 1024;  // cells the coarsest level may hold
-
-__global__ void __launch_bounds__(1024) k_mg_coarse(MgLevel L, float* __restrict__ e_out, float omega, int sweeps) {
-  __shared__ float se[kCoarseMax], sr[kCoarseMax], sd[kCoarseMax];
-  const int nx = L.g.nx, ny = L.g.ny, n = nx * ny;
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    const int i = t % nx, j = t / nx;
-    const size_t o = rb_at(i, j, ny, L.g.pk);
-    se[t] = 0.f;
-    sr[t] = L.r[o];
-    sd[t] = L.invd[o];
-  }
-  __syncthreads();
-  for (int s = 0; s < sweeps; ++s)
-    for (int c = 0; c < 2; ++c) {
-      for (int t = threadIdx.x; t < n; t += blockDim.x) {
-        const int i = t % nx, j = t / nx;
-        if (((i + j) & 1) != c) continue;
-        const float xE = i < nx - 1 ? se[t + 1] : 0.f, xW = i > 0 ? se[t - 1] : 0.f;
-        const float xN = j < ny - 1 ? se[t + nx] : 0.f, xS = j > 0 ? se[t - nx] : 0.f;
-        float sum = L.pE[i] * xE;
-        sum = fmaf(L.pW[i], xW, sum);
-        sum = fmaf(L.g.pN[j], xN, sum);
-        sum = fmaf(L.g.pS[j], xS, sum);
-        const float gs = (sum - sr[t]) * sd[t];
-        se[t] = fmaf(omega, gs - se[t], se[t]);
-      }
-      __syncthreads();
-    }
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    const int i = t % nx, j = t / nx;
-    e_out[rb_at(i, j, ny, L.g.pk)] = se[t];
+  pdl_enter();
+  const int I = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (I >= C.g.nx || j >= F.g.ny) return;
+  const int J = j >> 1, J2 = J + F.oy[j], ny = C.g.ny, pk = C.g.pk;
+  const float ay = F.ay[j];
+  const float e00 = ec[rb_at(I, J, ny, pk)], e01 = ec[rb_at(I, J2, ny, pk)];
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const int i = 2 * I + a;
+    if (i >= F.g.nx) break;
+    const int I2 = I + F.ox[i];
+    const float ax = F.ax[i];
+    const float e10 = ec[rb_at(I2, J, ny, pk)], e11 = ec[rb_at(I2, J2, ny, pk)];
+    const float lo = fmaf(ax, e10 - e00, e00), hi = fmaf(ax, e11 - e01, e01);
+    ef[((size_t)((i + j) & 1) * F.g.ny + j) * F.g.pk + I] += fmaf(ay, hi - lo, lo);
   }
 }
 
 inline dim3 grid_for(int nx, int ny) { return dim3((nx + 31) / 32, (ny + 7) / 8); }
 
-// ---- the small levels of the hierarchy in one CTA: the V-cycle below a
-// level whose cells (with all coarser levels) fit in shared memory runs in a
-// single launch instead of four launches per level, each of which would be
-// mostly launch latency.  Same operations as the per-level kernels: two
-// red-black Gauss-Seidel sweeps before and after, residual and restriction,
-// bilinear prolongation, SOR on the coarsest level; corrections from zero.
-__device__ inline float tail_sum(const MgLevel& L, const float* e, int i, int j) {
-  const int nx = L.g.nx, ny = L.g.ny, t = j * nx + i;
-  const float xE = i < nx - 1 ? e[t + 1] : 0.f, xW = i > 0 ? e[t - 1] : 0.f;
-  const float xN = j < ny - 1 ? e[t + nx] : 0.f, xS = j > 0 ? e[t - nx] : 0.f;
-  float sum = L.pE[i] * xE;
-  sum = fmaf(L.pW[i], xW, sum);
-  sum = fmaf(L.g.pN[j], xN, sum);
-  sum = fmaf(L.g.pS[j], xS, sum);
-  return sum;
+// ---- the small levels of the hierarchy in one launch of one CTA
+//
+// Below some 9000 cells a level's four launches (smoothing twice,
+// restriction, prolongation) are latency; from there down the whole V-cycle
+// runs in one CTA.  Same operations as the per-level kernels: two red-black
+// Gauss-Seidel sweeps before and after, residual and restriction, bilinear
+// prolongation, SOR on the coarsest level; corrections from zero.  What binds
+// is the chain of half-sweeps (about 100 of them, each a barrier and a few
+// shared-memory loads), so a thread keeps the coefficients, right-hand sides
+// and reciprocal diagonals of its cells in registers over a level's
+// half-sweeps, corrections lie in shared memory inside a border of zeros (no
+// tests at the boundary), and the coarsest level, at most 64 cells, runs in
+// one warp.  Everything that does not change between cycles (coefficients,
+// transfer weights, reciprocal diagonals of all levels) comes in one copy at
+// the start.  (Reading it from global memory on every use, the levels below
+// 128x64 alone took 49.8 us; a cluster of 16 CTAs with strips of rows and a
+// cluster barrier per half-sweep took 68 us from 256x128 down.)
+constexpr int kLowThreads = 1024;
+constexpr int kLowRows = 4;  // cells of one colour a thread owns at most
+
+struct LowCells {  // a thread's cells of one level: column pair k, rows g, g + G, ...
+  int k, g, G;
+  float cE[2], cW[2];                                     // per colour: the cell's column is fixed, G being even
+  float cN[kLowRows], cS[kLowRows];
+  float r[2][kLowRows], d[2][kLowRows];
+};
+
+// e[j + 1][i + 1] of a level, rows nx + 2 apart
+__device__ __forceinline__ float* low_e(const MgLow& T, float* sm, int l) { return sm + T.lv[l].off; }
+__device__ __forceinline__ float* low_r(const MgLow& T, float* sm, int l) {
+  return sm + T.lv[l].off + (T.lv[l].ny + 2) * (T.lv[l].nx + 2);
 }
 
-__device__ inline void tail_relax(const MgLevel& L, float* e, const float* r, float omega, int sweeps) {
-  const int nx = L.g.nx, n = nx * L.g.ny;
-  for (int s = 0; s < sweeps; ++s)
-    for (int c = 0; c < 2; ++c) {
-      for (int t = threadIdx.x; t < n; t += blockDim.x) {
-        const int i = t % nx, j = t / nx;
-        if (((i + j) & 1) != c) continue;
-        const float gs = (tail_sum(L, e, i, j) - r[t]) * L.invd[rb_at(i, j, L.g.ny, L.g.pk)];
-        e[t] = fmaf(omega, gs - e[t], e[t]);
-      }
-      __syncthreads();
-    }
-}
-
-__global__ void __launch_bounds__(1024) k_mg_tail(const MgTail T, float* __restrict__ e_top) {
-  extern __shared__ float tail_smem[];
-  float* se = tail_smem;               // corrections of all tail levels
-  float* sr = tail_smem + kTailCells;  // right-hand sides
-  const MgLevel& top = T.lv[0];
-  for (int t = threadIdx.x; t < top.g.nx * top.g.ny; t += blockDim.x) {
-    const int i = t % top.g.nx, j = t / top.g.nx;
-    sr[t] = top.r[rb_at(i, j, top.g.ny, top.g.pk)];
+// the constants of a level in shared memory, in the order mg_low_consts packs them
+struct LowConst {
+  const float *pE, *pW, *wx, *ax, *ox, *pN, *pS, *wy, *ay, *oy, *invd;
+  __device__ __forceinline__ LowConst(const MgLowLevel& A, const float* base) {
+    const float* p = base + A.coff;
+    pE = p;
+    pW = p + A.nx;
+    wx = p + 2 * A.nx;
+    ax = p + 3 * A.nx;
+    ox = p + 4 * A.nx;
+    p += 5 * A.nx;
+    pN = p;
+    pS = p + A.ny;
+    wy = p + 2 * A.ny;
+    ay = p + 3 * A.ny;
+    oy = p + 4 * A.ny;
+    invd = p + 5 * A.ny;
   }
-  for (int l = 0; l < T.n; ++l) {
-    const MgLevel& A = T.lv[l];
-    float *e = se + T.off[l], *r = sr + T.off[l];
-    const int n = A.g.nx * A.g.ny;
-    for (int t = threadIdx.x; t < n; t += blockDim.x) e[t] = 0.f;
-    __syncthreads();
-    if (l == T.n - 1) {
-      tail_relax(A, e, r, T.omega_c, T.sweeps_c);
-      break;
+};
+
+__device__ __forceinline__ void low_load(const MgLowLevel& A, const LowConst& K, const float* r, LowCells& c) {
+  const int nx = A.nx, ny = A.ny, w2 = (nx + 1) / 2;
+  c.g = threadIdx.x / w2;
+  c.k = threadIdx.x - c.g * w2;
+  c.G = (kLowThreads / w2) & ~1;
+  if (c.g >= c.G) c.g = ny;  // no cells
+#pragma unroll
+  for (int m = 0; m < kLowRows; ++m) {
+    const int j = c.g + c.G * m;
+    const bool in = j < ny;
+    c.cN[m] = in ? K.pN[j] : 0.f;
+    c.cS[m] = in ? K.pS[j] : 0.f;
+#pragma unroll
+    for (int col = 0; col < 2; ++col) {
+      const int i = 2 * c.k + ((col + c.g) & 1);
+      const bool cell = in && i < nx;
+      if (m == 0) {
+        c.cE[col] = cell ? K.pE[i] : 0.f;
+        c.cW[col] = cell ? K.pW[i] : 0.f;
+      }
+      c.r[col][m] = cell ? r[j * nx + i] : 0.f;
+      c.d[col][m] = cell ? K.invd[j * nx + i] : 0.f;
     }
-    tail_relax(A, e, r, 1.0f, 2);
-    const MgLevel& C = T.lv[l + 1];
-    float* rc = sr + T.off[l + 1];
-    for (int t = threadIdx.x; t < C.g.nx * C.g.ny; t += blockDim.x) {
-      const int I = t % C.g.nx, J = t / C.g.nx;
+  }
+}
+
+// two red-black Gauss-Seidel sweeps
+__device__ __forceinline__ void low_relax(const MgLowLevel& A, float* e, const LowCells& c) {
+  const int nx = A.nx, P = nx + 2;
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    const int col = h & 1, i = 2 * c.k + ((col + c.g) & 1);
+#pragma unroll
+    for (int m = 0; m < kLowRows; ++m) {
+      const int j = c.g + c.G * m;
+      if (j < A.ny && i < nx) {
+        float* p = e + (j + 1) * P + i + 1;
+        float sum = c.cE[col] * p[1];
+        sum = fmaf(c.cW[col], p[-1], sum);
+        sum = fmaf(c.cN[m], p[P], sum);
+        sum = fmaf(c.cS[m], p[-P], sum);
+        const float gs = (sum - c.r[col][m]) * c.d[col][m];
+        p[0] = fmaf(1.0f, gs - p[0], p[0]);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+__global__ void __launch_bounds__(kLowThreads, 1) k_mg_low(const __grid_constant__ MgLow T, float* __restrict__ e_top) {
+  extern __shared__ float low_smem[];
+  const int tid = threadIdx.x;
+  // the constants, before the wait (nothing writes them after set-up), and zero corrections
+  float* konst = low_smem + T.nzero;
+  for (int t = tid; t < T.nconst / 4; t += kLowThreads)
+    reinterpret_cast<float4*>(konst)[t] = reinterpret_cast<const float4*>(T.consts)[t];
+  for (int t = tid; t < T.nzero / 4; t += kLowThreads)
+    reinterpret_cast<float4*>(low_smem)[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  __syncthreads();
+  const MgLowLevel& top = T.lv[0];
+  {
+    float* r = low_r(T, low_smem, 0);
+    for (int t = tid; t < top.nx * top.ny; t += kLowThreads) {
+      const int j = t / top.nx, i = t - j * top.nx;
+      r[t] = top.r[rb_at(i, j, top.ny, top.pk)];
+    }
+  }
+  __syncthreads();
+  const int last = T.n - 1;
+  LowCells c;
+  for (int l = 0; l < last; ++l) {
+    const MgLowLevel &A = T.lv[l], &C = T.lv[l + 1];
+    float *e = low_e(T, low_smem, l), *r = low_r(T, low_smem, l), *rc = low_r(T, low_smem, l + 1);
+    const LowConst K(A, konst);
+    low_load(A, K, r, c);
+    low_relax(A, e, c);
+    const int P = A.nx + 2;
+    for (int t = tid; t < C.nx * C.ny; t += kLowThreads) {
+      const int J = t / C.nx, I = t - J * C.nx;
       float acc = 0.f;
+#pragma unroll
       for (int b = 0; b < 2; ++b) {
         const int j = 2 * J + b;
-        if (j >= A.g.ny) break;
+        if (j >= A.ny) break;
         float row = 0.f;
+#pragma unroll
         for (int a = 0; a < 2; ++a) {
           const int i = 2 * I + a;
-          if (i >= A.g.nx) break;
-          const int u = j * A.g.nx + i;
-          const float x = e[u];
-          const float xE = i < A.g.nx - 1 ? e[u + 1] : x, xW = i > 0 ? e[u - 1] : x;
-          const float xN = j < A.g.ny - 1 ? e[u + A.g.nx] : x, xS = j > 0 ? e[u - A.g.nx] : x;
-          float Le = A.pE[i] * (xE - x);
-          Le = fmaf(A.pW[i], xW - x, Le);
-          Le = fmaf(A.g.pN[j], xN - x, Le);
-          Le = fmaf(A.g.pS[j], xS - x, Le);
-          row = fmaf(A.wx[i], r[u] - Le, row);
+          if (i >= A.nx) break;
+          const float* p = e + (j + 1) * P + i + 1;
+          const float x = p[0];
+          float Le = K.pE[i] * (p[1] - x);
+          Le = fmaf(K.pW[i], p[-1] - x, Le);
+          Le = fmaf(K.pN[j], p[P] - x, Le);
+          Le = fmaf(K.pS[j], p[-P] - x, Le);
+          row = fmaf(K.wx[i], r[j * A.nx + i] - Le, row);
         }
-        acc = fmaf(A.wy[j], row, acc);
+        acc = fmaf(K.wy[j], row, acc);
       }
       rc[t] = acc;
     }
     __syncthreads();
   }
-  for (int l = T.n - 2; l >= 0; --l) {
-    const MgLevel& A = T.lv[l];
-    const MgLevel& C = T.lv[l + 1];
-    float *e = se + T.off[l], *r = sr + T.off[l];
-    const float* ec = se + T.off[l + 1];
-    for (int t = threadIdx.x; t < A.g.nx * A.g.ny; t += blockDim.x) {
-      const int i = t % A.g.nx, j = t / A.g.nx;
-      const int I = i >> 1, J = j >> 1, I2 = I + A.ox[i], J2 = J + A.oy[j];
-      const float ax = A.ax[i], ay = A.ay[j];
-      const float e00 = ec[J * C.g.nx + I], e10 = ec[J * C.g.nx + I2];
-      const float e01 = ec[J2 * C.g.nx + I], e11 = ec[J2 * C.g.nx + I2];
-      const float lo = fmaf(ax, e10 - e00, e00), hi = fmaf(ax, e11 - e01, e01);
-      e[t] += fmaf(ay, hi - lo, lo);
+  {
+    // coarsest level: red-black SOR; a lane owns up to two cells of each colour (more than 64 cells: the whole CTA)
+    const MgLowLevel& Z = T.lv[last];
+    const LowConst K(Z, konst);
+    float *e = low_e(T, low_smem, last), *r = low_r(T, low_smem, last);
+    const int nx = Z.nx, ny = Z.ny, P = nx + 2, w2 = (nx + 1) / 2;
+    if (nx * ny <= 64) {
+      if (tid < 32) {
+        float aE[2][2], aW[2][2], aN[2][2], aS[2][2], rr[2][2], dd[2][2];
+        float* p[2][2];
+#pragma unroll
+        for (int col = 0; col < 2; ++col)
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const int t = tid + 32 * q, j = t / w2, i = 2 * (t - j * w2) + ((col + j) & 1);
+            const bool in = j < ny && i < nx;
+            p[col][q] = in ? e + (j + 1) * P + i + 1 : nullptr;
+            aE[col][q] = in ? K.pE[i] : 0.f;
+            aW[col][q] = in ? K.pW[i] : 0.f;
+            aN[col][q] = in ? K.pN[j] : 0.f;
+            aS[col][q] = in ? K.pS[j] : 0.f;
+            rr[col][q] = in ? r[j * nx + i] : 0.f;
+            dd[col][q] = in ? K.invd[j * nx + i] : 0.f;
+          }
+        for (int s = 0; s < T.sweeps_c; ++s)
+#pragma unroll
+          for (int col = 0; col < 2; ++col) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+              if (float* x = p[col][q]) {
+                float sum = aE[col][q] * x[1];
+                sum = fmaf(aW[col][q], x[-1], sum);
+                sum = fmaf(aN[col][q], x[P], sum);
+                sum = fmaf(aS[col][q], x[-P], sum);
+                const float gs = (sum - rr[col][q]) * dd[col][q];
+                x[0] = fmaf(T.omega_c, gs - x[0], x[0]);
+              }
+            __syncwarp();
+          }
+      }
+    } else {
+      for (int h = 0; h < 2 * T.sweeps_c; ++h) {
+        for (int t = tid; t < ny * w2; t += kLowThreads) {
+          const int j = t / w2, i = 2 * (t - j * w2) + ((h + j) & 1);
+          if (i >= nx) continue;
+          float* x = e + (j + 1) * P + i + 1;
+          float sum = K.pE[i] * x[1];
+          sum = fmaf(K.pW[i], x[-1], sum);
+          sum = fmaf(K.pN[j], x[P], sum);
+          sum = fmaf(K.pS[j], x[-P], sum);
+          const float gs = (sum - r[j * nx + i]) * K.invd[j * nx + i];
+          x[0] = fmaf(T.omega_c, gs - x[0], x[0]);
+        }
+        __syncthreads();
+      }
     }
     __syncthreads();
-    tail_relax(A, e, r, 1.0f, 2);
   }
-  for (int t = threadIdx.x; t < top.g.nx * top.g.ny; t += blockDim.x) {
-    const int i = t % top.g.nx, j = t / top.g.nx;
-    e_top[rb_at(i, j, top.g.ny, top.g.pk)] = se[t];
+  for (int l = last - 1; l >= 0; --l) {
+    const MgLowLevel &A = T.lv[l], &C = T.lv[l + 1];
+    float *e = low_e(T, low_smem, l), *ec = low_e(T, low_smem, l + 1);
+    const LowConst K(A, konst);
+    low_load(A, K, low_r(T, low_smem, l), c);
+    const int P = A.nx + 2, PC = C.nx + 2;
+    for (int t = tid; t < A.nx * A.ny; t += kLowThreads) {
+      const int j = t / A.nx, i = t - j * A.nx;
+      const int I = (i >> 1) + 1, J = (j >> 1) + 1, I2 = I + __float_as_int(K.ox[i]), J2 = J + __float_as_int(K.oy[j]);
+      const float ax = K.ax[i], ay = K.ay[j];
+      const float e00 = ec[J * PC + I], e10 = ec[J * PC + I2];
+      const float e01 = ec[J2 * PC + I], e11 = ec[J2 * PC + I2];
+      const float lo = fmaf(ax, e10 - e00, e00), hi = fmaf(ax, e11 - e01, e01);
+      e[(j + 1) * P + i + 1] += fmaf(ay, hi - lo, lo);
+    }
+    __syncthreads();
+    low_relax(A, e, c);
+  }
+  const float* e = low_e(T, low_smem, 0);
+  for (int t = tid; t < top.nx * top.ny; t += kLowThreads) {
+    const int j = t / top.nx, i = t - j * top.nx;
+    e_top[rb_at(i, j, top.ny, top.pk)] = e[(j + 1) * (top.nx + 2) + i + 1];
   }
 }
 
@@ -282,6 +437,7 @@ constexpr int kReduceBlocks = 1216;  // 8 CTAs of 8 warps per SM: full occupancy
 // <z, q>; the last block sets beta = -<z, q> / <p, Lp> of the previous direction
 __global__ void k_fcg_dot(const MgLevel L, const float* __restrict__ dxv, const float* __restrict__ dyv,
                           const float* __restrict__ z, const float* __restrict__ q, FcgScalars* __restrict__ sc) {
+  pdl_enter();
   const int tx = (L.g.nx + 31) / 32, nt = tx * ((L.g.ny + 7) / 8);
   float v = 0.f;
   for (int t = blockIdx.x; t < nt; t += gridDim.x) {
@@ -300,19 +456,16 @@ __global__ void k_fcg_dot(const MgLevel L, const float* __restrict__ dxv, const 
   }
 }
 
-// p = z (first) or p = z + beta p
-__global__ void k_fcg_dir(const MgLevel L, const float* __restrict__ z, float* __restrict__ p,
-                          const FcgScalars* __restrict__ sc, int first) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= L.g.nx || j >= L.g.ny) return;
-  const size_t o = rb_at(i, j, L.g.ny, L.g.pk);
-  p[o] = first ? z[o] : fmaf(sc->beta, p[o], z[o]);
-}
-
-// q = L p, <p, q>, <p, r>; the last block sets alpha = <p, r> / <p, q>
+// p = z (first) or z + beta p_old, formed on the fly at the cell and its
+// neighbours (one pass instead of two), q = L p, <p, q>, <p, r>; the last block
+// sets alpha = <p, r> / <p, q>
+template <bool FIRST>
 __global__ void k_fcg_apply(const MgLevel L, const float* __restrict__ dxv, const float* __restrict__ dyv,
-                            const float* __restrict__ p, const float* __restrict__ r, float* __restrict__ q,
-                            FcgScalars* __restrict__ sc) {
+                            const float* __restrict__ z, const float* __restrict__ p_old, float* __restrict__ p,
+                            const float* __restrict__ r, float* __restrict__ q, FcgScalars* __restrict__ sc) {
+  pdl_enter();
+  const float beta = FIRST ? 0.f : sc->beta;
+  auto dir = [&](size_t o) { return FIRST ? z[o] : fmaf(beta, p_old[o], z[o]); };
   float vpq = 0.f, vpr = 0.f;
   const int nx = L.g.nx, ny = L.g.ny, pk = L.g.pk;
   const int tx = (nx + 31) / 32, nt = tx * ((ny + 7) / 8);
@@ -320,15 +473,16 @@ __global__ void k_fcg_apply(const MgLevel L, const float* __restrict__ dxv, cons
     const int i = (t % tx) * 32 + threadIdx.x, j = (t / tx) * 8 + threadIdx.y;
     if (i >= nx || j >= ny) continue;
     const size_t o = rb_at(i, j, ny, pk);
-    const float x = p[o];
-    const float xE = i < nx - 1 ? p[rb_at(i + 1, j, ny, pk)] : x;
-    const float xW = i > 0 ? p[rb_at(i - 1, j, ny, pk)] : x;
-    const float xN = j < ny - 1 ? p[rb_at(i, j + 1, ny, pk)] : x;
-    const float xS = j > 0 ? p[rb_at(i, j - 1, ny, pk)] : x;
+    const float x = dir(o);
+    const float xE = i < nx - 1 ? dir(rb_at(i + 1, j, ny, pk)) : x;
+    const float xW = i > 0 ? dir(rb_at(i - 1, j, ny, pk)) : x;
+    const float xN = j < ny - 1 ? dir(rb_at(i, j + 1, ny, pk)) : x;
+    const float xS = j > 0 ? dir(rb_at(i, j - 1, ny, pk)) : x;
     float Lp = L.pE[i] * (xE - x);
     Lp = fmaf(L.pW[i], xW - x, Lp);
     Lp = fmaf(L.g.pN[j], xN - x, Lp);
     Lp = fmaf(L.g.pS[j], xS - x, Lp);
+    p[o] = x;
     q[o] = Lp;
     const float Vx = dxv[i] * dyv[j] * x;
     vpq = fmaf(Vx, Lp, vpq);
@@ -346,15 +500,26 @@ __global__ void k_fcg_apply(const MgLevel L, const float* __restrict__ dxv, cons
   }
 }
 
-// x += alpha p; r -= alpha q
-__global__ void k_fcg_update(const MgLevel L, const float* __restrict__ p, const float* __restrict__ q,
-                             float* __restrict__ x, float* __restrict__ r, const FcgScalars* __restrict__ sc) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= L.g.nx || j >= L.g.ny) return;
-  const size_t o = rb_at(i, j, L.g.ny, L.g.pk);
+// x += alpha p; r -= alpha q, over the arrays as they lie (4 entries a thread;
+// their padding is zero and stays zero)
+__global__ void k_fcg_update(int n4, const float4* __restrict__ p, const float4* __restrict__ q,
+                             float4* __restrict__ x, float4* __restrict__ r, const FcgScalars* __restrict__ sc) {
+  pdl_enter();
   const float alpha = sc->alpha;
-  x[o] = fmaf(alpha, p[o], x[o]);
-  r[o] = fmaf(-alpha, q[o], r[o]);
+  for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < n4; o += gridDim.x * blockDim.x) {
+    const float4 pp = p[o], qq = q[o];
+    float4 xx = x[o], rr = r[o];
+    xx.x = fmaf(alpha, pp.x, xx.x);
+    xx.y = fmaf(alpha, pp.y, xx.y);
+    xx.z = fmaf(alpha, pp.z, xx.z);
+    xx.w = fmaf(alpha, pp.w, xx.w);
+    rr.x = fmaf(-alpha, qq.x, rr.x);
+    rr.y = fmaf(-alpha, qq.y, rr.y);
+    rr.z = fmaf(-alpha, qq.z, rr.z);
+    rr.w = fmaf(-alpha, qq.w, rr.w);
+    x[o] = xx;
+    r[o] = rr;
+  }
 }
 
 }  // namespace
@@ -368,42 +533,64 @@ inline int reduce_blocks(const MgLevel& L) {
 
 void launch_fcg_dot(cudaStream_t s, const MgLevel& L, const float* dxv, const float* dyv, const float* z,
                     const float* q, void* sc) {
-  k_fcg_dot<<<reduce_blocks(L), dim3(32, 8), 0, s>>>(L, dxv, dyv, z, q, (FcgScalars*)sc);
+  launch_pdl(k_fcg_dot, dim3(reduce_blocks(L)), dim3(32, 8), s, L, dxv, dyv, z, q, (FcgScalars*)sc);
 }
-void launch_fcg_dir(cudaStream_t s, const MgLevel& L, const float* z, float* p, const void* sc, int first) {
-  k_fcg_dir<<<grid_for(L.g.nx, L.g.ny), dim3(32, 8), 0, s>>>(L, z, p, (const FcgScalars*)sc, first);
-}
-void launch_fcg_apply(cudaStream_t s, const MgLevel& L, const float* dxv, const float* dyv, const float* p,
-                      const float* r, float* q, void* sc) {
-  k_fcg_apply<<<reduce_blocks(L), dim3(32, 8), 0, s>>>(L, dxv, dyv, p, r, q, (FcgScalars*)sc);
+void launch_fcg_apply(cudaStream_t s, const MgLevel& L, const float* dxv, const float* dyv, const float* z,
+                      const float* p_old, float* p, const float* r, float* q, void* sc, int first) {
+  launch_pdl(first ? k_fcg_apply<true> : k_fcg_apply<false>, dim3(reduce_blocks(L)), dim3(32, 8), s, L, dxv, dyv, z,
+             p_old, p, r, q, (FcgScalars*)sc);
 }
 void launch_fcg_update(cudaStream_t s, const MgLevel& L, const float* p, const float* q, float* x, float* r,
                        const void* sc) {
-  k_fcg_update<<<grid_for(L.g.nx, L.g.ny), dim3(32, 8), 0, s>>>(L, p, q, x, r, (const FcgScalars*)sc);
+  const int n4 = 2 * L.g.ny * (L.g.pk / 4), blocks = (n4 + 255) / 256;
+  launch_pdl(k_fcg_update, dim3(blocks < 2432 ? blocks : 2432), dim3(256), s, n4, (const float4*)p, (const float4*)q,
+             (float4*)x, (float4*)r, (const FcgScalars*)sc);
 }
 
-int mg_coarse_max() { return kCoarseMax; }
-
-cudaError_t prepare_mg_tail() {
-  return cudaFuncSetAttribute(k_mg_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(2 * kTailCells * sizeof(float)));
+// Fills T's shared-memory offsets for its n levels (nx, ny of lv set, finest
+// first); false if the levels do not fit the CTA (threads or shared memory).
+bool mg_low_layout(MgLow& T) {
+  static bool ok = false;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    ok = cudaFuncSetAttribute(k_mg_low, cudaFuncAttributeMaxDynamicSharedMemorySize, kLowSmem) == cudaSuccess;
+  });
+  long off = 0, coff = 0;
+  for (int l = 0; l < T.n; ++l) {
+    MgLowLevel& A = T.lv[l];
+    const int w2 = (A.nx + 1) / 2, G = (kLowThreads / w2) & ~1;
+    if (l < T.n - 1 && (G < 2 || A.ny > G * kLowRows)) return false;
+    A.off = (int)off;
+    off += (long)(A.ny + 2) * (A.nx + 2) + (long)A.ny * A.nx;
+    A.coff = (int)coff;
+    coff += 5l * (A.nx + A.ny) + (long)A.nx * A.ny;
+  }
+  T.nzero = (int)((off + 3) / 4 * 4);
+  T.nconst = (int)((coff + 3) / 4 * 4);
+  T.smem = (T.nzero + T.nconst) * (int)sizeof(float);
+  return ok && ((off + coff) * (long)sizeof(float) + 64) <= kLowSmem;
 }
 
-void launch_mg_tail(cudaStream_t s, const MgTail& T, float* e_top) {
-  k_mg_tail<<<1, 1024, 2 * kTailCells * sizeof(float), s>>>(T, e_top);
+void launch_mg_low(cudaStream_t s, const MgLow& T, float* e_top) {
+  cudaLaunchConfig_t lc{};
+  cudaLaunchAttribute at[1];
+  lc.gridDim = dim3(1);
+  lc.blockDim = dim3(kLowThreads);
+  lc.dynamicSmemBytes = T.smem;
+  lc.stream = s;
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  cudaLaunchKernelEx(&lc, k_mg_low, T, e_top);
 }
 
 void launch_mg_restrict(cudaStream_t s, const MgLevel& F, const float* ef, const MgLevel& C) {
-  k_mg_restrict<<<grid_for(C.g.nx, C.g.ny), dim3(32, 8), 0, s>>>(F, ef, C);
+  launch_pdl(k_mg_restrict, grid_for(C.g.nx, C.g.ny), dim3(32, 8), s, F, ef, C);
 }
 
 void launch_mg_prolong(cudaStream_t s, const MgLevel& C, const float* ec, const MgLevel& F, float* ef) {
-  k_mg_prolong<<<grid_for(F.g.nx, F.g.ny), dim3(32, 8), 0, s>>>(C, ec, F, ef);
-}
-
-void launch_mg_coarse(cudaStream_t s, const MgLevel& L, float* e_out, float omega, int sweeps) {
-  const int n = L.g.nx * L.g.ny, threads = n >= 1024 ? 1024 : (n + 31) / 32 * 32;  // few warps: cheap barriers
-  k_mg_coarse<<<1, threads, 0, s>>>(L, e_out, omega, sweeps);
+  launch_pdl(k_mg_prolong, grid_for(C.g.nx, F.g.ny), dim3(32, 8), s, C, ec, F, ef);
 }
 
 }  // namespace ibm

@@ -182,7 +182,7 @@ def test_fused_batch_step_matches_single_contexts_bit_for_bit_before_the_pressur
     B.close()
 
 
-@pytest.mark.parametrize("shape", range(37, 41))
+@pytest.mark.parametrize("shape", range(37, 42))
 def test_batch_tiles_by_tma_match_the_tile_per_block_form_bit_for_bit(shape):
     """The persistent sweep kernels (form 11) take the tiles of all cases in
     one list, skipping cases whose sweeps of the round are done; with 16
