@@ -159,6 +159,7 @@ struct ibm_ctx {
   // FP64 sweeps kept on chip (precision 0)
   Sor64Plan sor64;
   Sor64Tiles sor64_tiles{};
+  size_t sor64_bytes = 0;  // of its norms and words
   Sor64Result *sor64_res = nullptr, *sor64_host = nullptr;  // device; pinned, behind sc_host
   // history
   double *cl_d = nullptr, *cd_d = nullptr;
@@ -788,12 +789,17 @@ int read_norm(ibm_ctx* c, const unsigned long long* dev_bits, double* out) {
 
 // The sweeps and checks of solve_poisson on the device (k_sor64.cu); the host
 // waits once per launch of up to kChunk64 sweeps.
-constexpr int kChunk64 = 8192;
+constexpr int kChunk64 = 8192;  // two exchanges or checks a sweep at most: well below kSor64Numbers
 int solve_poisson_chip(ibm_ctx* c, double thr, int m, int maxs, int* sweeps, double* res) {
   const Geo& g = c->geo;
-  Sor64Tiles t = c->sor64_tiles;
-  t.phi2 = c->phi2;
   for (int done = 0;;) {
+    // exchange numbers are used once; when they run out the buffers are cleared
+    if (c->sor64.kind == Sor64Plan::TILES && c->sor64_tiles.first > UINT_MAX - 2 * kSor64Numbers) {
+      CUDA_TRY(cudaMemsetAsync(c->sor64_tiles.norms, 0, c->sor64_bytes, c->stream));
+      c->sor64_tiles.first = 0;
+    }
+    const Sor64Tiles t = c->sor64_tiles;
+    c->sor64_tiles.first += kSor64Numbers;
     const Sor64Args a{g.nx, g.ny, g.pitch, at(0, 0, g.pitch), g.pE, g.pW, g.pN, g.pS, c->phi, c->b, c->invd_p,
                       c->P.omega_p, thr, m, maxs - done, kChunk64};
     if (c->profiling) CUDA_TRY(cudaEventRecord(c->ev0, c->stream));
@@ -1937,13 +1943,16 @@ int ibm_create_grid(const ibm_grid_params* params, ibm_ctx** out) {
   if (!rc && P.precision == 0) {
     c->sor64 = sor64_plan(P.nx, P.ny, true);
     if (c->sor64.kind != Sor64Plan::NONE) {
-      // one block: two norms and two flags per tile, the result
-      const size_t nt = sor64_max_tiles();
+      // one block: the result, the norms' slots, the exchange words
+      const size_t nt = c->sor64.kind == Sor64Plan::TILES ? sor64_max_tiles() : 0;
+      const size_t words = nt ? 4 * (size_t)P.nx * P.ny : 0;
       unsigned char* blk = nullptr;
-      rc |= c->alloc(&blk, 24 * nt + sizeof(Sor64Result));
-      c->sor64_tiles.norms = (unsigned long long*)blk;
-      c->sor64_tiles.flags = (unsigned*)(blk + 16 * nt);
-      c->sor64_res = (Sor64Result*)(blk + 24 * nt);
+      c->sor64_bytes = 32 * nt + 8 * words;
+      rc |= c->alloc(&blk, 32 + c->sor64_bytes);
+      c->sor64_res = (Sor64Result*)blk;
+      c->sor64_tiles.norms = (unsigned long long*)(blk + 32);
+      c->sor64_tiles.words = c->sor64_tiles.norms + 4 * nt;
+      c->sor64_tiles.stride = words / 2;
       c->sor64_host = (Sor64Result*)(c->sc_host + 1);
     }
   }

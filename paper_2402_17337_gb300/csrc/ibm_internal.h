@@ -133,10 +133,13 @@ struct Sor64Args {
 };
 struct Sor64Tiles {
   int nbx, nby, K;
-  double* phi2;                // a second pitched field (exchanges alternate between it and phi)
-  unsigned* flags;             // 2 per tile
-  unsigned long long* norms;   // 2 per tile
+  unsigned long long* words;   // 2 buffers of 2 words per cell
+  size_t stride;               // words of one buffer
+  unsigned long long* norms;   // 4 words per tile
+  unsigned first;              // exchanges are numbered from first + 1; no number is used twice on the buffers
 };
+// exchange numbers one launch may use
+constexpr unsigned kSor64Numbers = 1u << 16;
 enum { SOR64_MORE = 0, SOR64_OK, SOR64_NOCONV, SOR64_DIVERGED };
 struct Sor64Result {
   unsigned long long bits;  // norm of the last check

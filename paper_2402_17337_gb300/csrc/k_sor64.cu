@@ -20,6 +20,7 @@
 // launch (about 2.3 us) and, every check, a host wait (about 15 us).
 #include <cstdint>
 #include <mutex>
+#include <type_traits>
 
 #include "ibm_internal.h"
 
@@ -90,18 +91,22 @@ constexpr int CL_CPT = 2;        // cells of one colour a thread owns at most
 constexpr size_t CL_SMEM = 100 * 1024;
 // Which kernel a grid takes (us per sweep, checks every 8 sweeps included;
 // the launch-per-half-sweep kernels of k_sor.cu in brackets):
-//   70x45    cluster 1.8 [10.4], tiles 2.7
-//   133x67   cluster 2.6 [10.7], tiles 3.1
-//   192x128  cluster 4.8, tiles 3.7 [10]
-//   512x256  tiles 6.5 [10.1]
-//   1024x512 tiles 14.0 [10.3]
+//   70x45    cluster 1.8 [10.4], tiles 2.1
+//   100x60   cluster 2.1, tiles 2.2
+//   133x67   cluster 2.6 [10.7], tiles 2.3
+//   192x128  cluster 4.8, tiles 2.7 [10]
+//   512x256  tiles 5.1 [10.1]
+//   700x350  tiles 7.3 [10.2]
+//   1024x512 tiles 12 [10.3]
 // so one cluster up to kClusterCells, tiles up to kTilesCells, and above
-// that the kernels of k_sor.cu, whose launches are then long enough.
-constexpr long kClusterCells = 12000, kTilesCells = 250000;
+// that the kernels of k_sor.cu, whose launches are then long enough.  A
+// half-sweep's floor is its chain of eight dependent FP64 instructions, about
+// 160 clocks each, and a barrier: 0.9 us.
+constexpr long kClusterCells = 7500, kTilesCells = 300000;
 // Model of the tiles' time that picks their shape, in clocks, fitted to those
 // measurements: one exchange, one half-sweep's barrier and latency, and 32
-// updates (128 of FP64 issue, the rest index arithmetic and shared memory).
-constexpr double kExchange = 7000.0, kHalf = 1300.0, kWarpUpdate = 200.0;
+// updates (128 of FP64 issue, the rest shared memory).
+constexpr double kExchange = 1500.0, kHalf = 1500.0, kWarpUpdate = 190.0;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
@@ -224,145 +229,164 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_sor64_cluster(Sor64Args A, So
 
 // ------------------------------------------------- tiles over all SMs
 
-constexpr int TL_THREADS = 512;
+constexpr int TL_THREADS = 640;
+constexpr int TL_CPT = 2;  // cells of one colour a thread owns at most
 
-__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 constexpr long long kWaitCycles = 2000000000ll;  // about 1 s at the SM clock
-// waits until *p has reached v; false after kWaitCycles
-__device__ __forceinline__ bool wait_flag(const unsigned* p, unsigned v) {
-  if ((int)(ld_acquire(p) - v) >= 0) return true;
+
+// A double with its exchange number: two 8-byte words {half, number}, each
+// written and read whole, so a reader that sees the number in both has the
+// value and needs no flag or fence (a fence here waits for every store of the
+// SM: with data, fence and flag 512x256 took 6.4 us a sweep, with this 5.1).
+__device__ __forceinline__ void post(unsigned long long* p, unsigned long long v, unsigned no) {
+  const unsigned long long lo = (v & 0xffffffffull) | ((unsigned long long)no << 32);
+  const unsigned long long hi = (v >> 32) | ((unsigned long long)no << 32);
+  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(lo), "l"(hi) : "memory");
+}
+__device__ __forceinline__ bool peek(const unsigned long long* p, unsigned no, unsigned long long& v) {
+  unsigned long long lo, hi;
+  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
+  v = (lo & 0xffffffffull) | (hi << 32);
+  return (unsigned)(lo >> 32) == no && (unsigned)(hi >> 32) == no;
+}
+// waits for exchange number no at p; false after kWaitCycles
+__device__ __forceinline__ bool fetch(const unsigned long long* p, unsigned no, unsigned long long& v) {
+  if (peek(p, no, v)) return true;
   const long long t0 = clock64();
-  while ((int)(ld_acquire(p) - v) < 0)
+  while (!peek(p, no, v))
     if (clock64() - t0 > kWaitCycles) return false;
   return true;
 }
 
-// CTA b owns tile (b % nbx, b / nbx) of the grid.  Shared memory holds phi, b
-// and the reciprocal diagonal of the tile and a halo of K cells, and the 1-D
-// coefficients.  Half-sweep h = 1 .. K after an exchange updates the tile and
-// K - h cells round it (the halo shrinks by one cell each time), so the tile
-// is exact after K half-sweeps; then each CTA publishes the K cells along its
-// edges in one of two buffers (phi2 and phi in turn), raises its flag, waits
-// for its neighbours' flags and refreshes its halo.  A buffer is written
-// again two exchanges later, after the neighbours' flags of the exchange in
-// between, which they raise after having read it.  All CTAs are resident at
-// once (cooperative launch); a wait that lasts about a second gives up and
-// the launch reports it.
+// Cell u of the perimeter of the w x h rectangle at (x, y), walked from its
+// corner (x, y) along the bottom row, the right column, the top row and the
+// left column; consecutive cells alternate in colour.
+__device__ __forceinline__ void perimeter(int x, int y, int w, int h, int u, int& i, int& j) {
+  if (u < w) {
+    i = x + u;
+    j = y;
+  } else if ((u -= w) < h - 1) {
+    i = x + w - 1;
+    j = y + 1 + u;
+  } else if ((u -= h - 1) < w - 1) {
+    i = x + w - 2 - u;
+    j = y + h - 1;
+  } else {
+    u -= w - 1;
+    i = x;
+    j = y + h - 2 - u;
+  }
+}
+
+// CTA b owns tile (b % nbx, b / nbx) of the grid.  Shared memory holds phi of
+// the tile and a halo of K cells.  Half-sweep h = 1 .. K after an exchange
+// updates the tile and K - h cells round it, so the tile is exact after K
+// half-sweeps; then each CTA posts the K cells along its edges and picks up
+// its halo from its neighbours' posts (two buffers in turn: a buffer is
+// written again two exchanges later, after the neighbours' posts of the
+// exchange in between, which they make after having read it).  The cells of a
+// colour are listed tile first, then ring by ring outwards, so those of
+// half-sweep h are the first of the list; a thread keeps the coefficients, b
+// and the reciprocal diagonal of its TL_CPT entries in registers.  All CTAs
+// are resident at once (cooperative launch); a wait that lasts about a second
+// gives up and the launch reports it.
 __global__ void __launch_bounds__(TL_THREADS, 1) k_sor64_tiles(Sor64Args A, Sor64Tiles T, Sor64Result* __restrict__ out) {
   extern __shared__ __align__(16) double sm64[];
   __shared__ unsigned long long wmax[TL_THREADS / 32];
   const int nx = A.nx, ny = A.ny, K = T.K, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int bx = blockIdx.x % T.nbx, by = blockIdx.x / T.nbx, nb = T.nbx * T.nby;
-  const int x0 = (int)((long)nx * bx / T.nbx), x1 = (int)((long)nx * (bx + 1) / T.nbx);
-  const int y0 = (int)((long)ny * by / T.nby), y1 = (int)((long)ny * (by + 1) / T.nby);
-  const int X0 = x0 - K, Y0 = y0 - K, RW = x1 - x0 + 2 * K, RH = y1 - y0 + 2 * K;  // region with its halo
-  const int P = RW + 2;                                                         // one spare column on each side
-  double* ph = sm64;                  // [RH + 2][P]
-  double* sb = ph + (RH + 2) * P;     // [RH][RW]
-  double* sd = sb + RH * RW;          // [RH][RW]
-  double* cE = sd + RH * RW;          // [RW]
-  double* cW = cE + RW;
-  double* cN = cW + RW;               // [RH]
-  double* cS = cN + RH;
-  for (int t = tid; t < (RH + 2) * P; t += TL_THREADS) {
-    const int r = t / P, i = X0 + (t - r * P) - 1, j = Y0 + r - 1;
-    const bool in = i >= 0 && i < nx && j >= 0 && j < ny && i >= X0 && i < X0 + RW && j >= Y0 && j < Y0 + RH;
+  const int x0 = (int)((long)nx * bx / T.nbx), x1 = (int)((long)nx * (bx + 1) / T.nbx), w = x1 - x0;
+  const int y0 = (int)((long)ny * by / T.nby), y1 = (int)((long)ny * (by + 1) / T.nby), h = y1 - y0;
+  const int X0 = x0 - K, Y0 = y0 - K, P = w + 2 * K, RH = h + 2 * K;  // region with its halo
+  double* ph = sm64;  // [RH][P]
+  for (int t = tid; t < RH * P; t += TL_THREADS) {
+    const int r = t / P, i = X0 + (t - r * P), j = Y0 + r;
+    const bool in = i >= 0 && i < nx && j >= 0 && j < ny;
     ph[t] = in ? __ldcg(A.phi + A.off + (size_t)j * A.pitch + i) : 0.0;
   }
-  for (int t = tid; t < RH * RW; t += TL_THREADS) {
-    const int r = t / RW, i = X0 + (t - r * RW), j = Y0 + r;
-    const bool in = i >= 0 && i < nx && j >= 0 && j < ny;
-    const size_t o = A.off + (size_t)j * A.pitch + i;
-    sb[t] = in ? A.b[o] : 0.0;
-    sd[t] = in ? A.invd[o] : 0.0;
-  }
-  for (int t = tid; t < RW; t += TL_THREADS) {
-    const int i = X0 + t;
-    const bool in = i >= 0 && i < nx;
-    cE[t] = in ? A.pE[i] : 0.0;
-    cW[t] = in ? A.pW[i] : 0.0;
-  }
-  for (int t = tid; t < RH; t += TL_THREADS) {
-    const int j = Y0 + t;
-    const bool in = j >= 0 && j < ny;
-    cN[t] = in ? A.pN[j] : 0.0;
-    cS[t] = in ? A.pS[j] : 0.0;
-  }
-  // the neighbour this thread waits for in an exchange (the first 8 threads), -1: none
-  int nbr = -1;
-  if (tid < 8) {
-    const int q = tid < 4 ? tid : tid + 1;  // 3 x 3 neighbourhood without its centre
-    const int ax = bx + q % 3 - 1, ay = by + q / 3 - 1;
-    if (ax >= 0 && ax < T.nbx && ay >= 0 && ay < T.nby) nbr = ay * T.nbx + ax;
-  }
+  const int w2 = (w + 1) / 2, n_own = h * w2;
+  double aE[2][TL_CPT], aW[2][TL_CPT], aN[2][TL_CPT], aS[2][TL_CPT], bb[2][TL_CPT], dd[2][TL_CPT];
+  int pos[2][TL_CPT];  // index into ph, 0: no cell
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+#pragma unroll
+    for (int k = 0; k < TL_CPT; ++k) {
+      int t = tid + k * TL_THREADS, i, j;
+      bool in = true;
+      if (t < n_own) {
+        const int r = t / w2;
+        j = y0 + r;
+        i = x0 + 2 * (t - r * w2) + ((c + x0 + j) & 1);
+        in = i < x1;
+      } else {
+        t -= n_own;
+        int q = 1;
+        while (q < K && t >= w + h + 4 * q - 2) t -= w + h + 4 * q++ - 2;
+        in = q < K;
+        perimeter(x0 - q, y0 - q, w + 2 * q, h + 2 * q, 2 * t + ((c + x0 + y0) & 1), i, j);
+      }
+      in = in && i >= 0 && i < nx && j >= 0 && j < ny;
+      aE[c][k] = in ? A.pE[i] : 0.0;
+      aW[c][k] = in ? A.pW[i] : 0.0;
+      aN[c][k] = in ? A.pN[j] : 0.0;
+      aS[c][k] = in ? A.pS[j] : 0.0;
+      const size_t o = A.off + (size_t)j * A.pitch + i;
+      bb[c][k] = in ? A.b[o] : 0.0;
+      dd[c][k] = in ? A.invd[o] : 0.0;
+      pos[c][k] = in ? (j - Y0) * P + i - X0 : 0;
+    }
   __syncthreads();
-  unsigned epoch = 0, checks = 0;
+  unsigned no = T.first;  // number of the last exchange or check
+  unsigned exchanges = 0, checks = 0;  // each alternates between its two buffers
   bool dead = false;
   // refreshes the halo; false if a neighbour did not come
   auto exchange = [&]() {
-    double* buf = (epoch & 1) ? A.phi : T.phi2;
-    ++epoch;
-    const int w = x1 - x0, h = y1 - y0;
-    // the K cells along each edge of the tile (all of it if the tile is narrower than 2 K)
-    for (int t = tid; t < w * h; t += TL_THREADS) {
-      const int r = t / w, q = t - r * w;
-      if (r < K || r >= h - K || q < K || q >= w - K)
-        __stcg(buf + A.off + (size_t)(y0 + r) * A.pitch + x0 + q, ph[(r + K + 1) * P + q + K + 1]);
-    }
-    __syncthreads();
-    if (tid == 0) {
-      __threadfence();
-      st_release(T.flags + blockIdx.x, epoch);
+    ++no;
+    unsigned long long* buf = T.words + ((exchanges++ & 1) ? T.stride : 0);
+    // the K outermost rings of the tile (all of it if it is narrower), then the K rings round it
+    const int rings = min(K, (min(w, h) + 1) / 2);
+    int total = 0;
+    for (int q = 0; q < rings; ++q) {
+      const int ww = w - 2 * q, hh = h - 2 * q, n = ww > 1 && hh > 1 ? 2 * (ww + hh) - 4 : ww * hh;
+      for (int u = tid - total % TL_THREADS < 0 ? tid - total % TL_THREADS + TL_THREADS : tid - total % TL_THREADS; u < n;
+           u += TL_THREADS) {
+        int i, j;
+        if (ww > 1 && hh > 1) {
+          perimeter(x0 + q, y0 + q, ww, hh, u, i, j);
+        } else {
+          i = x0 + q + (ww > 1 ? u : 0);
+          j = y0 + q + (ww > 1 ? 0 : u);
+        }
+        post(buf + 2 * ((size_t)j * nx + i), (unsigned long long)__double_as_longlong(ph[(j - Y0) * P + i - X0]), no);
+      }
+      total += n;
     }
     bool late = false;
-    if (nbr >= 0) late = !wait_flag(T.flags + nbr, epoch);
-    if (__syncthreads_or(late)) return false;
-    const int top = K * RW, mid = h * 2 * K;  // halo cells: K rows below, K rows above, K columns on both sides
-    for (int t = tid; t < 2 * top + mid; t += TL_THREADS) {
-      int r, q;
-      if (t < 2 * top) {
-        r = t / RW;
-        q = t - r * RW;
-        if (r >= K) r += h;
-      } else {
-        const int u = t - 2 * top;
-        r = u / (2 * K);
-        q = u - r * 2 * K;
-        r += K;
-        if (q >= K) q += w;
+    total = 0;
+    for (int q = 1; q <= K; ++q) {
+      const int n = 2 * (w + h) + 8 * q - 4;
+      for (int u = tid - total % TL_THREADS < 0 ? tid - total % TL_THREADS + TL_THREADS : tid - total % TL_THREADS;
+           u < n && !late; u += TL_THREADS) {
+        int i, j;
+        perimeter(x0 - q, y0 - q, w + 2 * q, h + 2 * q, u, i, j);
+        if (i < 0 || i >= nx || j < 0 || j >= ny) continue;
+        unsigned long long v;
+        late = !fetch(buf + 2 * ((size_t)j * nx + i), no, v);
+        ph[(j - Y0) * P + i - X0] = __longlong_as_double((long long)v);
       }
-      const int i = X0 + q, j = Y0 + r;
-      if (i >= 0 && i < nx && j >= 0 && j < ny)
-        ph[(r + 1) * P + q + 1] = __ldcg(buf + A.off + (size_t)j * A.pitch + i);
+      total += n;
     }
-    __syncthreads();
-    return true;
+    return !__syncthreads_or(late);
   };
-  // half-sweep of colour c over the region without its outer h cells
-  auto half = [&](int c, int h) {
-    const int w = RW - 2 * h, hh = RH - 2 * h, w2 = (w + 1) / 2, n = hh * w2;
-    const int dr = TL_THREADS / w2, dk = TL_THREADS - dr * w2;
-    int r = tid / w2, k = tid - r * w2;
-    for (int t = tid; t < n; t += TL_THREADS) {
-      const int rr = h + r, q = h + 2 * k + ((c + Y0 + rr + X0 + h) & 1);
-      if (q < RW - h) {
-        const int p = (rr + 1) * P + q + 1, o = rr * RW + q;
-        ph[p] = sor64(cE[q], cW[q], cN[rr], cS[rr], ph[p + 1], ph[p - 1], ph[p + P], ph[p - P], sb[o], sd[o], A.omega,
-                      ph[p]);
-      }
-      r += dr;
-      k += dk;
-      if (k >= w2) {
-        k -= w2;
-        ++r;
-      }
+  // half-sweep hs of colour C after an exchange: the first n cells of the list
+  auto half = [&](auto colour, int n) {
+    constexpr int c = decltype(colour)::value;
+#pragma unroll
+    for (int k = 0; k < TL_CPT; ++k) {
+      const int p = pos[c][k];
+      if (p && tid + k * TL_THREADS < n)
+        ph[p] = sor64(aE[c][k], aW[c][k], aN[c][k], aS[c][k], ph[p + 1], ph[p - 1], ph[p + P], ph[p - P], bb[c][k],
+                      dd[c][k], A.omega, ph[p]);
     }
     __syncthreads();
   };
@@ -375,32 +399,32 @@ __global__ void __launch_bounds__(TL_THREADS, 1) k_sor64_tiles(Sor64Args A, Sor6
         fresh = K;
       }
       unsigned long long v = 0ull;
-      const int w = x1 - x0, n = w * (y1 - y0);
-      for (int t = tid; t < n; t += TL_THREADS) {
-        const int r = t / w, q = t - r * w + K, rr = r + K, p = (rr + 1) * P + q + 1;
-        const unsigned long long b = abs_bits(res64(cE[q], cW[q], cN[rr], cS[rr], ph[p + 1], ph[p - 1], ph[p + P],
-                                                    ph[p - P], sb[rr * RW + q], ph[p]));
-        v = b > v ? b : v;
-      }
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int k = 0; k < TL_CPT; ++k) {
+          const int p = pos[c][k];
+          if (!p || tid + k * TL_THREADS >= n_own) continue;
+          const unsigned long long b = abs_bits(res64(aE[c][k], aW[c][k], aN[c][k], aS[c][k], ph[p + 1], ph[p - 1],
+                                                      ph[p + P], ph[p - P], bb[c][k], ph[p]));
+          v = b > v ? b : v;
+        }
       v = warp_max(v);
       if (lane == 0) wmax[warp] = v;
       __syncthreads();
-      // the CTA's norm to its slot of this check's bank, then every CTA reads every slot
-      unsigned long long* slots = T.norms + (checks & 1) * nb;
-      ++checks;
+      // the CTA's norm to its slot, then every CTA reads every slot
+      ++no;
+      // (a slot is written again two checks later: every CTA has read it before it posts to the check in between)
+      unsigned long long* slots = T.norms + ((checks++ & 1) ? 2 * nb : 0);
       if (warp == 0) {
         v = warp_max(lane < TL_THREADS / 32 ? wmax[lane] : 0ull);
-        if (lane == 0) {
-          __stcg(slots + blockIdx.x, v);
-          __threadfence();
-          st_release(T.flags + nb + blockIdx.x, checks);
-        }
+        if (lane == 0) post(slots + 2 * blockIdx.x, v, no);
       }
       v = 0ull;
       bool late = false;
-      for (int t = tid; t < nb; t += TL_THREADS) {
-        if (!wait_flag(T.flags + nb + t, checks)) { late = true; break; }
-        const unsigned long long b = __ldcg(slots + t);
+      for (int t = tid; t < nb && !late; t += TL_THREADS) {
+        unsigned long long b;
+        late = !fetch(slots + 2 * t, no, b);
         v = b > v ? b : v;
       }
       v = warp_max(v);
@@ -420,28 +444,17 @@ __global__ void __launch_bounds__(TL_THREADS, 1) k_sor64_tiles(Sor64Args A, Sor6
       if (!exchange()) { dead = true; break; }
       fresh = K;
     }
-    half(0, K - fresh + 1);
-    half(1, K - fresh + 2);
+    // rings 1 .. fresh - 1, then fresh - 2: (w + h + 4 q - 2) cells of a colour in ring q
+    auto cells = [&](int q) { return n_own + q * (w + h - 2) + 2 * q * (q + 1); };
+    half(std::integral_constant<int, 0>{}, cells(fresh - 1));
+    half(std::integral_constant<int, 1>{}, cells(fresh - 2));
     fresh -= 2;
     ++L.s;
   }
-  const int w = x1 - x0, n = w * (y1 - y0);
-  if (!dead && L.s != L.last) {
-    // an exchange may have followed the last check: every CTA has read its
-    // halo from phi before any of them writes its whole tile there
-    ++checks;
-    if (tid == 0) {
-      __threadfence();
-      st_release(T.flags + nb + blockIdx.x, checks);
-    }
-    for (int t = tid; t < nb; t += TL_THREADS)
-      if (!wait_flag(T.flags + nb + t, checks)) dead = true;
-    dead = __syncthreads_or(dead);
-  }
   if (!dead)
-    for (int t = tid; t < n; t += TL_THREADS) {
+    for (int t = tid; t < w * h; t += TL_THREADS) {
       const int r = t / w, q = t - r * w;
-      A.phi[A.off + (size_t)(y0 + r) * A.pitch + x0 + q] = ph[(r + K + 1) * P + q + K + 1];
+      A.phi[A.off + (size_t)(y0 + r) * A.pitch + x0 + q] = ph[(r + K) * P + q + K];
     }
   if (dead && tid == 0) atomicOr(&out->late, 1);
   if (blockIdx.x == 0 && tid == 0) {
@@ -496,9 +509,12 @@ const Sor64Dev& sor64_device() {
   return dev[d];
 }
 
-size_t tiles_smem(int w, int h, int K) {
-  const size_t RW = w + 2 * K, RH = h + 2 * K;
-  return sizeof(double) * ((RH + 2) * (RW + 2) + 2 * RH * RW + 2 * RW + 2 * RH);
+size_t tiles_smem(int w, int h, int K) { return sizeof(double) * (size_t)(w + 2 * K) * (h + 2 * K); }
+
+// entries of a colour's list: the tile and K - 1 rings
+long tiles_list(int w, int h, int K) {
+  const int q = K - 1;
+  return (long)h * ((w + 1) / 2) + (long)q * (w + h - 2) + 2l * q * (q + 1);
 }
 
 }  // namespace
@@ -528,13 +544,9 @@ Sor64Plan sor64_plan(int nx, int ny, bool tiles) {
       if (nby < 1) continue;
       const int w = (nx + nbx - 1) / nbx, h = (ny + nby - 1) / nby;
       const size_t smem = tiles_smem(w, h, K);
-      if (smem > (size_t)d.smem) continue;
+      if (smem > (size_t)d.smem || tiles_list(w, h, K) > TL_THREADS * TL_CPT) continue;
       double t = kExchange;
-      for (int q = 1; q <= K; ++q) {
-        const double n = (double)((w + 2 * (K - q) + 1) / 2) * (h + 2 * (K - q));
-        const double warps = n / 32;
-        t += kWarpUpdate * warps + kHalf;
-      }
+      for (int q = 1; q <= K; ++q) t += kWarpUpdate * (tiles_list(w, h, q) / 32.0) + kHalf;
       t /= K;
       if (p.kind == Sor64Plan::NONE || t < best) {
         best = t;
@@ -571,8 +583,6 @@ cudaError_t launch_sor64(cudaStream_t s, const Sor64Plan& p, const Sor64Args& a,
   tt.nbx = p.nbx;
   tt.nby = p.nby;
   tt.K = p.K;
-  e = cudaMemsetAsync(tt.flags, 0, 2 * sizeof(unsigned) * p.nbx * p.nby, s);
-  if (e != cudaSuccess) return e;
   Sor64Args aa = a;
   void* args[] = {&aa, &tt, &out};
   return cudaLaunchCooperativeKernel((const void*)k_sor64_tiles, dim3(p.nbx * p.nby), dim3(TL_THREADS), args, p.smem, s);

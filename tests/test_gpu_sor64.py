@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("nx,ny", [(5, 4), (9, 200), (64, 15), (33, 16), (17, 17), (128, 93), (129, 95), (41, 300),
-                                   (300, 41), (191, 129), (513, 257), (500, 500), (501, 501)])
+                                   (300, 41), (191, 129), (513, 257), (500, 500), (547, 548), (548, 549), (75, 100), (76, 100)])
 @pytest.mark.parametrize("m,cap", [(8, 60), (3, 20), (1, 2), (7, 49)])
 def test_sweeps_on_chip_match_oracle(nx, ny, m, cap):
     import torch
