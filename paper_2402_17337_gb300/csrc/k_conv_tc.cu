@@ -4,23 +4,23 @@
 //
 // The convolution is an implicit GEMM.  One CTA computes a tile of M = 128
 // output pixels (R image rows of TW pixels, R TW = 128) times NT output
-// channels; K runs over the 9 taps and the input channels, 16 channels (one
-// K = 16 MMA) per tap and chunk.  Operands use the K-major layout without
-// swizzling, whose unit is the core matrix: 8 rows (pixels, or output
-// channels) of 16 bytes (8 channels) stored contiguously.
+// channels; K runs over the input channels in chunks of KC (64, 32 or 16) and
+// over the 9 taps, one MMA per tap and 16 channels.
 //
 //   A (pixels x channels): the input halo tile is loaded by TMA from a 3-D
-//   tensor map over the activation view (channels, x, y), one box of 8
-//   channels per channel group, so shared memory holds [row][pixel][8 ch],
-//   16 bytes per pixel.  A tap's operand is a window of that tile: with one
-//   image row per tile (R = 1) the box spans TW + 2 pixels and a tap's
-//   shift (dy, dx) moves the descriptor's start by dy rows and dx pixels
-//   (16 bytes each); with R > 1 rows a pixel shift would wrap between rows,
-//   so three boxes are loaded, each already shifted by its dx, and a tap
-//   moves the start by dy rows only.  Out-of-image pixels are zero-filled by
-//   the TMA unit, which is the convolution's zero padding.
+//     tensor map over the activation view (channels, x, y), one box of KC
+//     channels, so shared memory holds [row][pixel][KC], 2 KC bytes a pixel
+//     with the swizzle of that width (K-major).  A tap's operand is a window of
+//     that tile: with one image row per tile (R = 1) the box spans TW + 2
+//     pixels and a tap's shift (dy, dx) moves the descriptor's start by dy
+//     rows and dx pixels (the swizzle acts on the address, so a window may
+//     start at any pixel); with R > 1 rows a pixel shift would wrap between
+//     rows, so three boxes are loaded, each already shifted by its dx, and a
+//     tap moves the start by dy rows only.  Out-of-image pixels are
+//     zero-filled by the TMA unit, which is the convolution's zero padding.
 //   B (output channels x channels): weights pre-packed (k_pack_conv_weights)
-//   into the exact shared-memory image of a chunk, copied by one bulk copy.
+//     as shared-memory images without swizzling (core matrices of 8 rows x 16
+//     bytes), copied by bulk copies.
 //
 // Consecutive convolutions are programmatic dependent launches (the next
 // kernel's set-up overlaps the previous one's tail).  The CTAs are
@@ -102,26 +102,49 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// shared-memory matrix descriptor, K-major without swizzling: start address,
-// leading byte offset (between the two core matrices of a K = 16 slice),
-// stride byte offset (between 8-row groups), descriptor version 1
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
+// Shared-memory matrix descriptors as two words (descriptor version 1).  Low
+// word: start address / 16, leading byte offset (core matrices of a K = 16
+// slice without swizzling; unused with it); high word: stride byte offset
+// (between 8-row groups), version, swizzle.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) { return (addr >> 4) | (lbo >> 4) << 16; }
+__device__ __forceinline__ uint32_t desc_hi(uint32_t sbo) { return (sbo >> 4) | 1u << 14; }
+// A K-major operand whose rows are row_bytes = 32, 64 or 128 wide with the
+// swizzle of that width, 8-row groups contiguous.  The swizzle acts on the
+// address, so a window may start at any row of the pattern and a K = 16 slice
+// 32 bytes further along the row.
+__device__ __forceinline__ uint32_t desc_hi_swizzled(uint32_t row_bytes) {
+  return desc_hi(8 * row_bytes) | (row_bytes == 128 ? 2u : (row_bytes == 64 ? 4u : 6u)) << 29;
 }
 // instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
 // K-major, N = n, M = 128
 __device__ __forceinline__ uint32_t instr_desc(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24);
 }
-__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+// One thread of the warp, chosen so that the compiler knows the branch holds
+// one thread and keeps the operands of the instructions below in uniform
+// registers.  A 128 x N x 16 MMA reads 4 KB + 32 N bytes of shared memory and
+// takes that over 128 bytes/clock: 40 clocks at N = 16, 48 at 64, 65 at 128
+// issued this way (58 and more from a thread picked by its lane number).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+// Descriptors come as low and high words; the loops below add to the low one.
+__device__ __forceinline__ void tc_mma(uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                       uint32_t idesc, uint32_t acc) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %6, 0;\n"
+      " mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n" ::"r"(d),
+      "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(acc)
       : "memory");
 }
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 // 16 consecutive FP32 columns of this warp's 32 lanes
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
@@ -141,9 +164,10 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 struct TcGeom {
   int TW, R;           // pixels per tile row, rows per MMA (TW R = 128)
   int RB;              // MMA rows a tile stacks (R = 1 only): RB accumulators from one halo box
-  int copies, boxw;    // A boxes per channel group (1 or 3), pixels per box row
-  int a_region;        // bytes of one A box in shared memory (padded to 128)
-  int a_bytes, b_bytes, stage_bytes, tx_bytes, stages;
+  int KC;              // input channels per chunk: 64, 32 or 16
+  int copies, boxw;    // A boxes per chunk (1 or 3), pixels per box row
+  int a_region;        // bytes of one A box in shared memory (padded to 1024)
+  int a_bytes, a_tx, stage_bytes, stages;  // a_tx: bytes the A boxes of a chunk bring
   int NT, tmem_cols, nchunks;
   int tiles_x, tiles_z, ntiles;  // tiles: TW-pixel columns x R-row bands x NT-channel groups
 };
@@ -201,6 +225,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (threadIdx.x == 128) prefetch_map(&tmX);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -212,6 +237,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   // then the next launch may be scheduled.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // the biases, once per CTA (they come from a previous kernel when training); read after the first accumulator wait
+  float* sb = reinterpret_cast<float*>(smem_raw + (sbase - smem_u32(smem_raw)) + G.stages * G.stage_bytes);
+  if (warp < 4) {
+    for (int k = threadIdx.x; k < Cout; k += 128) sb[k] = bias ? bias[k] : 0.f;
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+  }
   auto coords = [&](int li, int& x0, int& y0, int& z) {
     int t = (int)blockIdx.x + li * (int)gridDim.x;
     z = t % G.tiles_z;
@@ -226,7 +257,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     // pairs q = li nc + ch; a stage is reloaded once the MMAs that read it
     // have completed (empty barrier, committed by the MMA thread)
     if (lane == 0) {
-      const size_t wchunk = (size_t)2 * 9 * G.NT * 8;  // bf16 elements of one chunk's weights
       int issued = 0;
       for (int q = 0; q < nq; ++q) {
         const int li = q / nc, ch = q % nc, s = q % S;
@@ -234,12 +264,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         int x0, y0, z;
         coords(li, x0, y0, z);
         const uint32_t st = sbase + s * G.stage_bytes, bar = smem_u32(&bar_full[s]);
-        mbar_expect_tx(bar, G.tx_bytes);
+        // this tile's output channels of the packed weights: NT of them, fewer in the last tile
+        const int n0 = z * G.NT, nt = Cout - n0 < G.NT ? Cout - n0 : G.NT, k16 = G.KC / 16;
+        mbar_expect_tx(bar, G.a_tx + k16 * 9 * nt * 32);
         for (int cp = 0; cp < G.copies; ++cp)
-          for (int g = 0; g < 2; ++g)
-            tma_load_3d(st + (cp * 2 + g) * G.a_region, &tmX, ch * 16 + g * 8, G.copies == 1 ? x0 - 1 : x0 + cp - 1,
-                        y0 - 1, bar);
-        bulk_load(st + G.a_bytes, wpk + ((size_t)z * nc + ch) * wchunk, G.b_bytes, bar);
+          tma_load_3d(st + cp * G.a_region, &tmX, ch * G.KC, x0 + cp - 1, y0 - 1, bar);
+        const bf16* w = wpk + (size_t)ch * k16 * 9 * Cout * 16 + (size_t)n0 * 16;
+        if (nt == Cout)
+          bulk_load(st + G.a_bytes, w, k16 * 9 * nt * 32, bar);
+        else
+          for (int t = 0; t < 9 * k16; ++t)
+            bulk_load(st + G.a_bytes + t * G.NT * 32, w + (size_t)t * Cout * 16, nt * 32, bar);
         issued = q + 1;
       }
       if (*abort && issued > 0)  // the last load issued has landed (bounded) before the CTA may exit
@@ -248,36 +283,56 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     __syncwarp();
   } else if (warp == 5) {
     // MMA issuer: never waits for its own MMAs, only for data (full) and for
-    // the epilogue to have drained an accumulator (tempty)
-    if (lane == 0) {
-      const uint32_t idesc = instr_desc(G.NT);
-      int done = 0;
-      for (int q = 0; q < nq; ++q) {
-        const int li = q / nc, ch = q % nc, s = q % S, buf = li & 1;
-        if (ch == 0 && li >= 2 && !wait_or_abort(smem_u32(&bar_tempty[buf]), (uint32_t)((li >> 1) - 1) & 1u, abort))
-          break;
-        if (!wait_or_abort(smem_u32(&bar_full[s]), (uint32_t)(q / S) & 1u, abort)) break;
-        tc_fence_after();
-        const uint32_t st = sbase + s * G.stage_bytes, d = tmem + (uint32_t)buf * half_cols;
-        for (int rb = 0; rb < G.RB; ++rb) {
+    // the epilogue to have drained an accumulator (tempty).  An MMA costs this
+    // thread two additions: building each descriptor took 105 clocks an MMA,
+    // more than twice what the tensor cores need.
+    if (elect_one()) {
+      const uint32_t idesc = instr_desc(G.NT), row = (uint32_t)G.KC * 2;  // row: bytes of a pixel
+      const uint32_t a_hi = desc_hi_swizzled(row), b_hi = desc_hi(256), b_step = (uint32_t)G.NT * 2;
+      uint32_t a_tap[9];
 #pragma unroll
-          for (int tap = 0; tap < 9; ++tap) {
-            const int dy = tap / 3, dx = tap % 3;
-            const uint32_t a =
-                G.copies == 1 ? st + ((rb + dy) * G.boxw + dx) * 16 : st + dx * 2 * G.a_region + dy * G.TW * 16;
-            // B: [tap][8-row group of output channels][channel group][8 rows][16 bytes]
-            const uint32_t b = st + G.a_bytes + tap * G.NT * 32;
-            tc_mma(d + (uint32_t)(rb * G.NT), smem_desc(a, G.a_region, 128), smem_desc(b, 128, 256), idesc,
-                   (ch | tap) != 0);
+      for (int tap = 0; tap < 9; ++tap)
+        a_tap[tap] = (G.copies == 1 ? (uint32_t)((tap / 3) * G.boxw + tap % 3) * row
+                                    : (uint32_t)(tap % 3 * G.a_region) + (uint32_t)(tap / 3 * G.TW) * row) >> 4;
+      int s = 0, last = -1;
+      uint32_t phase = 0;
+      bool ok = true;
+      for (int li = 0; li < nmine && ok; ++li) {
+        const int buf = li & 1;
+        const uint32_t d = tmem + (uint32_t)buf * half_cols;
+        if (li >= 2) ok = wait_or_abort(smem_u32(&bar_tempty[buf]), (uint32_t)((li >> 1) - 1) & 1u, abort);
+        for (int ch = 0; ch < nc; ++ch) {
+          ok = ok && wait_or_abort(smem_u32(&bar_full[s]), phase, abort);
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t st = sbase + s * G.stage_bytes;
+          uint32_t ar = desc_lo(st, 0);
+          // B: [K = 16 slice][tap][8-row group of output channels][channel group][8 rows][16 bytes]
+          const uint32_t b0 = desc_lo(st + G.a_bytes, 128);
+          for (int rb = 0; rb < G.RB; ++rb) {
+            uint32_t b = b0, ak = ar;
+            for (int k = 0; k < G.KC / 16; ++k) {
+#pragma unroll
+              for (int tap = 0; tap < 9; ++tap) {
+                tc_mma(d + (uint32_t)(rb * G.NT), ak + a_tap[tap], a_hi, b, b_hi, idesc, (uint32_t)(ch | k | tap));
+                b += b_step;
+              }
+              ak += 2;
+            }
+            ar += (uint32_t)G.boxw * row >> 4;
+          }
+          tc_commit(smem_u32(&bar_empty[s]));
+          if (ch == nc - 1) tc_commit(smem_u32(&bar_tfull[buf]));
+          last = s;
+          if (++s == S) {
+            s = 0;
+            phase ^= 1u;
           }
         }
-        tc_commit(smem_u32(&bar_empty[s]));
-        if (ch == nc - 1) tc_commit(smem_u32(&bar_tfull[buf]));
-        done = q + 1;
       }
       if (*abort) {
         // the MMAs issued have completed (bounded) before the accumulators are freed
-        if (done > 0) mbar_wait(smem_u32(&bar_empty[(done - 1) % S]), (uint32_t)((done - 1) / S) & 1u);
+        if (last >= 0) mbar_wait(smem_u32(&bar_empty[last]), last < s ? phase : phase ^ 1u);
         atomicOr_system(err, 1u);
       }
     }
@@ -298,7 +353,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const int co = n0 + c0;
         float bv[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) bv[j] = bias ? bias[co + j] : 0.f;
+        for (int j = 0; j < 16; ++j) bv[j] = sb[co + j];
         uint32_t below[8];  // the tile row before, for the pooling
         for (int rb = 0; rb < G.RB; ++rb) {
           const int y = y0 + m / G.TW + rb;
@@ -442,6 +497,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (threadIdx.x == 128) {
+    prefetch_map(&tmG);
+    prefetch_map(&tmX);
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -467,22 +526,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
     __syncwarp();
   } else if (warp == 5) {
-    if (lane == 0) {
-      // both operands MN-major (transpose bits), N = NT, M = 128
+    // both operands MN-major (transpose bits), N = NT, M = 128
+    if (elect_one()) {
       const uint32_t idesc = instr_desc(G.NT) | (1u << 15) | (1u << 16);
+      const uint32_t a_hi = desc_hi(G.a_region), b_hi = desc_hi(G.b_region);
       int done = 0;
       for (int q = 0; q < nq; ++q) {
         const int s = q % S;
         if (!wait_or_abort(smem_u32(&bar_full[s]), (uint32_t)(q / S) & 1u, abort)) break;
         tc_fence_after();
         const uint32_t st = sbase + s * G.stage_bytes;
+        uint32_t a = desc_lo(st, 128), b = desc_lo(st + G.a_bytes, 128);
         for (int ks = 0; ks < G.P / 16; ++ks) {
-          const uint64_t a = smem_desc(st + ks * 256, 128, G.a_region);
 #pragma unroll
-          for (int t = 0; t < 3; ++t) {
-            const uint64_t b = smem_desc(st + G.a_bytes + (ks * 16 + t) * 16, 128, G.b_region);
-            tc_mma(tmem + (uint32_t)(t * G.NT), a, b, idesc, (q | ks) != 0);
-          }
+          for (int t = 0; t < 3; ++t)
+            tc_mma(tmem + (uint32_t)(t * G.NT), a, a_hi, b + t, b_hi, idesc, (uint32_t)(q | ks));
+          a += 16;
+          b += 16;
         }
         tc_commit(smem_u32(&bar_empty[s]));
         done = q + 1;
@@ -521,10 +581,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 }
 
 // Packed weights of a convolution with Cin input and Cout output channels:
-// for output-channel tile t (NT channels) and input-channel chunk ch (16
-// channels), the chunk's shared-memory image
-//   [tap 9][8-row group NT/8][channel group 2][row 8][8 channels]
-// of W'[co][tap][ci], zero for co >= Cout.  W' is the layer's weights
+// for each 16 input channels the shared-memory image
+//   [tap 9][8-row group Cout/8][channel group 2][row 8][8 channels]
+// of W'[co][tap][ci]; a tile of output channels is a contiguous piece of each
+// tap.  W' is the layer's weights
 // w[Cout][9][Cin]; with flip it is the data-gradient operator of a layer
 // whose weights are w[Cin][9][Cout]: W'[co][tap][ci] = w[ci][8 - tap][co].
 // One launch packs every job (blockIdx.y = job).
@@ -535,29 +595,24 @@ __global__ void k_pack_conv_weights(const PackJob* __restrict__ jobs) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const PackJob J = jobs[blockIdx.y];
-  const int Cin = J.cin, Cout = J.cout, NT = J.nt, nchunks = Cin / 16;
-  const int n = J.ntiles * nchunks * 9 * NT * 2;
+  const int Cin = J.cin, Cout = J.cout, n = Cin / 16 * 9 * Cout * 2;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int row = k & 7, g = (k >> 3) & 1;
     int r = k >> 4;
-    const int ngrp = r % (NT / 8);
-    r /= NT / 8;
-    const int tap = r % 9;
-    r /= 9;
-    const int ch = r % nchunks, t = r / nchunks;
-    const int co = t * NT + ngrp * 8 + row, ci = ch * 16 + g * 8;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (co < Cout) {
-      if (!J.flip) {
-        v = *reinterpret_cast<const uint4*>(J.w + ((size_t)co * 9 + tap) * Cin + ci);
-      } else {
-        unsigned short h[8];
-        const unsigned short* w = reinterpret_cast<const unsigned short*>(J.w);
+    const int ngrp = r % (Cout / 8);
+    r /= Cout / 8;
+    const int tap = r % 9, ch = r / 9;
+    const int co = ngrp * 8 + row, ci = ch * 16 + g * 8;
+    uint4 v;
+    if (!J.flip) {
+      v = *reinterpret_cast<const uint4*>(J.w + ((size_t)co * 9 + tap) * Cin + ci);
+    } else {
+      unsigned short h[8];
+      const unsigned short* w = reinterpret_cast<const unsigned short*>(J.w);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) h[e] = w[((size_t)(ci + e) * 9 + (8 - tap)) * Cout + co];
-        v = make_uint4(h[0] | (unsigned)h[1] << 16, h[2] | (unsigned)h[3] << 16, h[4] | (unsigned)h[5] << 16,
-                       h[6] | (unsigned)h[7] << 16);
-      }
+      for (int e = 0; e < 8; ++e) h[e] = w[((size_t)(ci + e) * 9 + (8 - tap)) * Cout + co];
+      v = make_uint4(h[0] | (unsigned)h[1] << 16, h[2] | (unsigned)h[3] << 16, h[4] | (unsigned)h[5] << 16,
+                     h[6] | (unsigned)h[7] << 16);
     }
     reinterpret_cast<uint4*>(J.wpk)[k] = v;
   }
@@ -626,23 +681,10 @@ int pow2_at_least(int v) {
 
 }  // namespace
 
-int conv_tile_channels(int Cout) { return Cout <= 128 ? Cout : 128; }
-
-size_t packed_conv_weights(int Cin, int Cout) {
-  const int NT = conv_tile_channels(Cout), ntiles = (Cout + NT - 1) / NT;
-  return (size_t)ntiles * NT * 9 * Cin;
-}
+size_t packed_conv_weights(int Cin, int Cout) { return (size_t)Cout * 9 * Cin; }
 
 PackJob pack_job(int Cin, int Cout, const bf16* w, bf16* wpk, bool flip) {
-  PackJob j{};
-  j.cin = Cin;
-  j.cout = Cout;
-  j.nt = conv_tile_channels(Cout);
-  j.ntiles = (Cout + j.nt - 1) / j.nt;
-  j.flip = flip ? 1 : 0;
-  j.w = w;
-  j.wpk = wpk;
-  return j;
+  return PackJob{Cin, Cout, flip ? 1 : 0, w, wpk};
 }
 
 void pack_conv_weights(cudaStream_t s, const PackJob* jobs_dev, int njobs, long max_elems) {
@@ -772,39 +814,50 @@ int conv3x3(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* X, int 
   G.R = TC_M / G.TW;
   G.copies = G.R == 1 ? 1 : 3;
   G.boxw = G.R == 1 ? G.TW + 2 : G.TW;
-  G.NT = conv_tile_channels(Cout);
+  G.tiles_x = (W + G.TW - 1) / G.TW;
+  // Output channels per tile: all of them up to 128, halved (not below 32)
+  // while the tiles are fewer than half the SMs.  A halving doubles the CTAs
+  // and the loads of A: the forward pass of the 32/64/128/128 network on
+  // 256x512 takes 170 us with a quarter of the SMs as the line, 163 with half,
+  // 168 with all.
+  G.NT = Cout <= 128 ? Cout : 128;
+  while (G.NT >= 64 && G.NT % 32 == 0 && (long)G.tiles_x * ((H + G.R - 1) / G.R) * ((Cout + G.NT - 1) / G.NT) < 76)
+    G.NT /= 2;
+  G.tiles_z = (Cout + G.NT - 1) / G.NT;
   // With one image row per MMA a tile stacks RB rows: one halo box of RB + 2
-  // rows serves RB accumulators, where RB tiles would load 3 RB rows.  TMA
-  // moves these boxes 16 bytes (a pixel's 8 channels) at a time, which is
-  // what bounds the narrow layers: 16 -> 16 channels on 512x1024, 25.6 us with
-  // RB = 1, 16.8 us with 4 (8 leaves too few loads in flight: 1 CTA an SM).
-  // The accumulators (two sets) stay within 256 columns, and a layer keeps a
-  // tile for every SM.
+  // rows serves RB accumulators, where RB tiles would load 3 RB rows, and the
+  // weights of a chunk are loaded once.  RB NT <= 64: the forward pass of
+  // 16/32/32/48 on 512x1024 takes 196 us with 32, 172 with 64, 176 with 128.
+  // A layer keeps a tile for every SM.
   G.RB = 1;
   if (G.R == 1)
     for (int rb = 4; rb > 1 && G.RB == 1; rb /= 2)
-      if (rb * G.NT <= 128 && (long)((W + TC_M - 1) / TC_M) * ((H + rb - 1) / rb) >= 152) G.RB = rb;
+      if (rb * G.NT <= 64 && (long)G.tiles_x * G.tiles_z * ((H + rb - 1) / rb) >= 152) G.RB = rb;
   // the pooling in the epilogue takes two rows of a tile
   if (also.pool && G.R == 1 && G.RB == 1 && 2 * G.NT <= 256) G.RB = 2;
   const bool pool = also.pool && G.R == 1 && G.RB % 2 == 0 && H % 2 == 0 && W % 2 == 0;
   if (!pool) also.pool = nullptr;
   if (pooled) *pooled = pool;
-  const int rows = G.R * G.RB + 2;
-  G.a_region = (rows * G.boxw * 16 + 127) / 128 * 128;
-  G.a_bytes = G.copies * 2 * G.a_region;
-  G.b_bytes = 9 * G.NT * 32;
-  G.stage_bytes = (G.a_bytes + G.b_bytes + 1023) / 1024 * 1024;
-  G.tx_bytes = G.copies * 2 * rows * G.boxw * 16 + G.b_bytes;
+  // Channels per chunk: the most of which two stages fit.  A TMA box moves
+  // one contiguous run per pixel, so a chunk of 64 channels takes an eighth of
+  // the runs that 8-channel boxes take: 163 us for 32/64/128/128 on 256x512,
+  // against 180 with chunks of 16.
+  const int rows = G.R * G.RB + 2, smem_extra = 1024 + Cout * 4;  // alignment slack, biases
+  for (G.KC = 64;; G.KC /= 2) {
+    G.a_region = (rows * G.boxw * G.KC * 2 + 1023) / 1024 * 1024;
+    G.a_bytes = G.copies * G.a_region;
+    G.a_tx = G.copies * rows * G.boxw * G.KC * 2;
+    G.stage_bytes = (G.a_bytes + 9 * G.NT * G.KC * 2 + 1023) / 1024 * 1024;
+    if (G.KC == 16 || (Cin % G.KC == 0 && 2 * G.stage_bytes + smem_extra <= TC_SMEM_MAX)) break;
+  }
   // two sets of RB accumulators, each set at least 32 columns
   G.tmem_cols = pow2_at_least(2 * G.RB * G.NT < 64 ? 64 : 2 * G.RB * G.NT);
-  G.nchunks = Cin / 16;
-  G.stages = 3 * G.stage_bytes + 1024 <= TC_SMEM_MAX ? 3 : 2;
-  G.tiles_x = (W + G.TW - 1) / G.TW;
-  G.tiles_z = (Cout + G.NT - 1) / G.NT;
+  G.nchunks = Cin / G.KC;
+  G.stages = 3 * G.stage_bytes + smem_extra <= TC_SMEM_MAX ? 3 : 2;
   G.ntiles = G.tiles_x * ((H + G.R * G.RB - 1) / (G.R * G.RB)) * G.tiles_z;
-  // dynamic shared memory: the stages plus alignment slack, at least
+  // dynamic shared memory: the stages, alignment slack and biases, at least
   // tmem_min_smem
-  int smem = G.stages * G.stage_bytes + 1024;
+  int smem = G.stages * G.stage_bytes + smem_extra;
   const int smem_tmem = tmem_min_smem(G.tmem_cols);
   if (smem < smem_tmem) smem = smem_tmem;
   if (smem > TC_SMEM_MAX) {
@@ -814,10 +867,13 @@ int conv3x3(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* X, int 
   CUtensorMap map;
   cuuint64_t dims[3] = {(cuuint64_t)Cin, (cuuint64_t)W, (cuuint64_t)H};
   cuuint64_t strides[2] = {(cuuint64_t)ldx * 2, (cuuint64_t)W * ldx * 2};
-  cuuint32_t box[3] = {8, (cuuint32_t)G.boxw, (cuuint32_t)rows};
+  cuuint32_t box[3] = {(cuuint32_t)G.KC, (cuuint32_t)G.boxw, (cuuint32_t)rows};
+  const CUtensorMapSwizzle swz = G.KC == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+                                 : G.KC == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                              : CU_TENSOR_MAP_SWIZZLE_32B;
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult cr = enc(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<bf16*>(X + offx), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (cr != CUDA_SUCCESS) {
     set_last_error("cuTensorMapEncodeTiled rejected an activation view");

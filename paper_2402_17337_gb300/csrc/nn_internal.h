@@ -32,7 +32,7 @@ int conv3x3(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* X, int 
 // w[ci][8 - tap][co])
 size_t packed_conv_weights(int Cin, int Cout);
 struct PackJob {
-  int cin, cout, nt, ntiles, flip;
+  int cin, cout, flip;
   const bf16* w;
   bf16* wpk;
 };
