@@ -192,7 +192,11 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, vol
 // the sequence of (tile, chunk) pairs), lane 0 of warp 5 the MMAs.  Two accumulators in
 // tensor memory alternate between tiles, so the MMAs of a tile run while
 // the previous tile's epilogue reads the other one.
-template <bool RELU>
+// GRAD (a data gradient): the epilogue applies the ReLU mask of the layer that
+// made this convolution's input and sums that layer's bias gradient, a pass
+// over the gradient (139 of 1025 us of a training step at 256x512) less.
+enum ConvOut { OUT_PLAIN, OUT_RELU, OUT_GRAD };
+template <ConvOut OUT>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_conv3x3_tc(const __grid_constant__ CUtensorMap tmX, const bf16* __restrict__ wpk, const float* __restrict__ bias,
                  bf16* __restrict__ Y, int ldy, int offy, float* __restrict__ yf, ConvAlso also, int H, int W, int Cout,
@@ -237,7 +241,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   // then the next launch may be scheduled.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  // the biases, once per CTA (they come from a previous kernel when training); read after the first accumulator wait
+  // the biases, once per CTA (OUT_GRAD: the CTA's sums of the bias gradient)
   float* sb = reinterpret_cast<float*>(smem_raw + (sbase - smem_u32(smem_raw)) + G.stages * G.stage_bytes);
   if (warp < 4) {
     for (int k = threadIdx.x; k < Cout; k += 128) sb[k] = bias ? bias[k] : 0.f;
@@ -351,20 +355,26 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       const int x = x0 + m % G.TW, n0 = z * G.NT;
       for (int c0 = 0; c0 < G.NT && n0 + c0 < Cout; c0 += 16) {
         const int co = n0 + c0;
-        float bv[16];
+        float bv[16];  // OUT_GRAD: the pixel's sums over rb
 #pragma unroll
-        for (int j = 0; j < 16; ++j) bv[j] = sb[co + j];
+        for (int j = 0; j < 16; ++j) bv[j] = OUT == OUT_GRAD ? 0.f : sb[co + j];
         uint32_t below[8];  // the tile row before, for the pooling
         for (int rb = 0; rb < G.RB; ++rb) {
           const int y = y0 + m / G.TW + rb;
           const bool valid = x < W && y < H;
           const size_t p = (size_t)y * W + x;
+          uint4 mk[2] = {};
+          if (OUT == OUT_GRAD && valid) {
+            const uint4* src = reinterpret_cast<const uint4*>(also.act + p * also.lda + also.offa + co);
+            mk[0] = src[0];
+            mk[1] = src[1];
+          }
           float v[16];
           tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)buf * half_cols + (uint32_t)(rb * G.NT + c0), v);
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            const float t = v[j] + bv[j];
-            v[j] = RELU ? fmaxf(t, 0.f) : t;
+            if (OUT != OUT_GRAD) v[j] += bv[j];
+            if (OUT == OUT_RELU) v[j] = fmaxf(v[j], 0.f);
           }
           if (yf && valid && co == 0) yf[p] = v[0];
           uint4 o[2];
@@ -373,6 +383,19 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
           for (int j = 0; j < 8; ++j) {
             __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
             ow[j] = *reinterpret_cast<uint32_t*>(&h);
+          }
+          if (OUT == OUT_GRAD) {
+            // zero where the activation is not positive (mk is zero outside the image), then add to the sums
+            const uint32_t* mw = reinterpret_cast<const uint32_t*>(mk);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&mw[j]));
+              if (!(a.x > 0.f)) ow[j] &= 0xFFFF0000u;
+              if (!(a.y > 0.f)) ow[j] &= 0x0000FFFFu;
+              const float2 g = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&ow[j]));
+              bv[2 * j] += g.x;
+              bv[2 * j + 1] += g.y;
+            }
           }
           if (Y && valid) {
             uint4* dst = reinterpret_cast<uint4*>(Y + p * ldy + offy + co);
@@ -418,10 +441,30 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             }
           }
         }
+        if (OUT == OUT_GRAD) {
+          // sum over the warp's pixels: at each step a lane passes on half of its channels and adds the other
+          // lane's share of the half it keeps; lanes 2c and 2c + 1 end with channel c
+#pragma unroll
+          for (int w = 8; w >= 1; w /= 2) {
+            const bool up = lane & (2 * w);
+#pragma unroll
+            for (int j = 0; j < w; ++j) {
+              const float got = __shfl_xor_sync(0xffffffffu, up ? bv[j] : bv[j + w], 2 * w);
+              bv[j] = (up ? bv[j + w] : bv[j]) + got;
+            }
+          }
+          bv[0] += __shfl_xor_sync(0xffffffffu, bv[0], 1);
+          if (!(lane & 1)) atomicAdd(&sb[co + lane / 2], bv[0]);
+        }
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bar_tempty[buf]));
+    }
+    if (OUT == OUT_GRAD) {
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      for (int k = threadIdx.x; k < Cout; k += 128)
+        if (sb[k] != 0.f) atomicAdd(also.db + k, sb[k]);
     }
   }
   tc_fence_before();
@@ -881,7 +924,7 @@ int conv3x3(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* X, int 
   }
   if (first_use_on_device(0)) {
     // the largest shared-memory carveout, so that several CTAs fit on an SM
-    for (auto k : {k_conv3x3_tc<true>, k_conv3x3_tc<false>}) {
+    for (auto k : {k_conv3x3_tc<OUT_PLAIN>, k_conv3x3_tc<OUT_RELU>, k_conv3x3_tc<OUT_GRAD>}) {
       cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MAX);
       cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
     }
@@ -892,7 +935,7 @@ int conv3x3(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* X, int 
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  auto kern = relu ? k_conv3x3_tc<true> : k_conv3x3_tc<false>;
+  auto kern = also.act ? k_conv3x3_tc<OUT_GRAD> : (relu ? k_conv3x3_tc<OUT_RELU> : k_conv3x3_tc<OUT_PLAIN>);
   int per_sm = SM_SMEM / (smem + 2048);
   if (per_sm > 2048 / TC_THREADS) per_sm = 2048 / TC_THREADS;
   if (per_sm > 512 / G.tmem_cols) per_sm = 512 / G.tmem_cols;

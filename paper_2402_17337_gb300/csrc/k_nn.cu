@@ -94,80 +94,56 @@ __global__ void k_avgpool(int H, int W, int C, const bf16* __restrict__ X, int l
   }
 }
 
-// gradient of the average pool: dX[2y+a][2x+b][c] (+)= dY[y][x][c] / 4; one
-// thread per fine pixel and 8 channels
-__global__ void k_avgpool_grad(int H, int W, int C, const bf16* __restrict__ dY, int ldy, int offy,
-                               bf16* __restrict__ dX, int ldx, int offx, int accumulate) {
-  pdl_enter();
-  const int Gc = C / 8, n = H * W * Gc;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    const int c0 = (k % Gc) * 8, p = k / Gc, x = p % W, y = p / W;
-    float g[8], d[8];
-    bf16x8_to_float(*reinterpret_cast<const uint4*>(dY + ((size_t)(y / 2) * (W / 2) + x / 2) * ldy + offy + c0), g);
-    uint4* dp = reinterpret_cast<uint4*>(dX + (size_t)p * ldx + offx + c0);
-    if (accumulate) bf16x8_to_float(*dp, d);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float gj = 0.25f * g[j];
-      d[j] = accumulate ? d[j] + gj : gj;
-    }
-    *dp = bf16x8_to(d);
-  }
-}
-
-// gradient of the upsampling: dX[y][x][c] (+)= sum of the 2x2 block of dY;
-// one thread per coarse pixel and 8 channels
-__global__ void k_upsample_grad(int H, int W, int C, const bf16* __restrict__ dY, int ldy, int offy,
-                                bf16* __restrict__ dX, int ldx, int offx, int accumulate) {
-  pdl_enter();
-  const int H2 = H / 2, W2 = W / 2, Gc = C / 8, n = H2 * W2 * Gc;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    const int c0 = (k % Gc) * 8, p = k / Gc, x = p % W2, y = p / W2;
-    auto at = [&](int yy, int xx, float (&f)[8]) {
-      bf16x8_to_float(*reinterpret_cast<const uint4*>(dY + ((size_t)yy * W + xx) * ldy + offy + c0), f);
-    };
-    float a[8], b[8], c[8], e[8], d[8];
-    at(2 * y, 2 * x, a);
-    at(2 * y, 2 * x + 1, b);
-    at(2 * y + 1, 2 * x, c);
-    at(2 * y + 1, 2 * x + 1, e);
-    uint4* dp = reinterpret_cast<uint4*>(dX + (size_t)p * ldx + offx + c0);
-    if (accumulate) bf16x8_to_float(*dp, d);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float g = a[j] + b[j] + c[j] + e[j];
-      d[j] = accumulate ? d[j] + g : g;
-    }
-    *dp = bf16x8_to(d);
-  }
-}
-
-// Gradient through ReLU, in place (G[p][c] = 0 where Y[p][c] <= 0; Y null: no
-// ReLU), and the bias gradient db[c] += sum_p G[p][c], in one pass over G (two
-// passes cost 107 and 64 us of a 1.0 ms training step at 256x512).  A block
-// of 256 threads reads 256 / (C / 8) pixels at a time, each thread 8 channels
-// of one pixel (16 bytes), sums over its pixels, then the block sums its
-// threads' partials per channel in shared memory and adds them to db.
-__global__ void k_relu_bias_grad(long npix, int C, bf16* __restrict__ G, int ldg, int offg, const bf16* __restrict__ Y,
-                                 int ldy, int offy, float* __restrict__ db) {
+// The gradient of a ReLU output Y from the next level's gradient dY, through
+// the average pool (FROM_POOL: G[p] += dY[p / 2] / 4) or the upsampling
+// (FROM_UP: G[p] = the sum of the 2x2 block of dY), zeroed where Y <= 0, and
+// that layer's bias gradient db[c] += sum_p G[p][c], in one pass over G (as
+// two passes the six such layers of 32/64/128/128 at 256x512 took 30 and 52 us
+// of a training step).  A block of 256 threads takes 256 / (C / 8) pixels at
+// a time, each thread 8 channels of one pixel (16 bytes), sums over its
+// pixels, then the block sums its threads' partials per channel in shared
+// memory and adds them to db.  H, W: the size of G.
+enum GradFrom { FROM_POOL, FROM_UP };
+template <GradFrom FROM>
+__global__ void k_resize_relu_grad(int H, int W, int C, const bf16* __restrict__ dY, int ldy, bf16* __restrict__ G,
+                                   int ldg, int offg, const bf16* __restrict__ Y, int lda, int offa,
+                                   float* __restrict__ db) {
   __shared__ float part[256][9];  // [thread][8 channels], padded against bank conflicts
   pdl_enter();
-  const int Gc = C / 8, rows = blockDim.x / Gc;
+  const int Gc = C / 8, rows = blockDim.x / Gc, npix = H * W;
   const int g = threadIdx.x % Gc, r = threadIdx.x / Gc;
   float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   if (r < rows) {
-    for (long p = (long)blockIdx.x * rows + r; p < npix; p += (long)gridDim.x * rows) {
-      uint4* gp = reinterpret_cast<uint4*>(G + p * ldg + offg + 8 * g);
-      float v[8];
-      bf16x8_to_float(*gp, v);
-      if (Y) {
-        float y[8];
-        bf16x8_to_float(*reinterpret_cast<const uint4*>(Y + p * ldy + offy + 8 * g), y);
+    for (int p = blockIdx.x * rows + r; p < npix; p += gridDim.x * rows) {
+      const int x = p % W, y = p / W;
+      auto at = [&](size_t q, float (&f)[8]) {
+        bf16x8_to_float(*reinterpret_cast<const uint4*>(dY + q * ldy + 8 * g), f);
+      };
+      uint4* gp = reinterpret_cast<uint4*>(G + (size_t)p * ldg + offg + 8 * g);
+      float v[8], act[8];
+      bf16x8_to_float(*reinterpret_cast<const uint4*>(Y + (size_t)p * lda + offa + 8 * g), act);
+      if (FROM == FROM_POOL) {
+        float d[8];
+        bf16x8_to_float(*gp, v);
+        at((size_t)(y / 2) * (W / 2) + x / 2, d);
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (!(y[j] > 0.f)) v[j] = 0.f;
-        *gp = bf16x8_to(v);
+        for (int j = 0; j < 8; ++j) v[j] += 0.25f * d[j];
+      } else {
+        float a[8], b[8], c[8], d[8];
+        const size_t q = (size_t)(2 * y) * (2 * W) + 2 * x;
+        at(q, a);
+        at(q + 1, b);
+        at(q + 2 * W, c);
+        at(q + 2 * W + 1, d);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = a[j] + b[j] + c[j] + d[j];
       }
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (!(act[j] > 0.f)) v[j] = 0.f;
+      const uint4 o = bf16x8_to(v);
+      *gp = o;
+      bf16x8_to_float(o, v);
 #pragma unroll
       for (int j = 0; j < 8; ++j) acc[j] += v[j];
     }
@@ -185,24 +161,32 @@ __global__ void k_relu_bias_grad(long npix, int C, bf16* __restrict__ G, int ldg
   }
 }
 
-// loss = mean over masked pixels of (out[p][0] - target[p])^2 ; dOut = 2 (out - target) / count
+// loss = mean over masked pixels of (out[p][0] - target[p])^2 ; dOut = 2 (out - target) / count ; db += sum dOut
 __global__ void k_mse(long npix, const float* __restrict__ out, int ldo, const float* __restrict__ target,
                       const float* __restrict__ mask, float inv_count, bf16* __restrict__ dout, int ldd,
-                      double* __restrict__ loss) {
+                      double* __restrict__ loss, float* __restrict__ db) {
   pdl_enter();
   double s = 0.0;
+  float sb = 0.f;
   for (long p = blockIdx.x * (long)blockDim.x + threadIdx.x; p < npix; p += (long)gridDim.x * blockDim.x) {
     float m = mask ? mask[p] : 1.f;
     float d = (out[p * ldo] - target[p]) * m;
     s += (double)d * d;
     // channel 0 of the pixel's ldd (a multiple of 8) channels, the others zero: 16-byte stores
     __nv_bfloat162 h = __floats2bfloat162_rn(2.f * d * inv_count, 0.f);
+    sb += __low2float(h);
     uint4* o = reinterpret_cast<uint4*>(dout + p * ldd);
     o[0] = make_uint4(*reinterpret_cast<unsigned*>(&h), 0u, 0u, 0u);
     for (int c = 1; c < ldd / 8; ++c) o[c] = make_uint4(0u, 0u, 0u, 0u);
   }
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, s * inv_count);
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    sb += __shfl_xor_sync(0xffffffffu, sb, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(loss, s * inv_count);
+    atomicAdd(db, sb);
+  }
 }
 
 // Adam on FP32 master weights, BF16 copy for the kernels
@@ -256,25 +240,23 @@ inline int grid1(long n) {
 void avgpool(cudaStream_t s, int H, int W, int C, const bf16* X, int ldx, int offx, bf16* Y, int ldy, int offy) {
   launch_pdl(k_avgpool, grid1((long)H * W * C / 32), 256, s, H, W, C, X, ldx, offx, Y, ldy, offy);
 }
-void avgpool_grad(cudaStream_t s, int H, int W, int C, const bf16* dY, int ldy, int offy, bf16* dX, int ldx, int offx,
-                  bool acc) {
-  launch_pdl(k_avgpool_grad, grid1((long)H * W * C / 8), 256, s, H, W, C, dY, ldy, offy, dX, ldx, offx, acc ? 1 : 0);
+static int resize_grad_blocks(long npix, int C) {
+  const long rows = 256 / (C / 8), blocks = (npix + rows * 4 - 1) / (rows * 4);  // at least 4 pixels per thread
+  return (int)(blocks > 1216 ? 1216 : blocks);
 }
-void upsample_grad(cudaStream_t s, int H, int W, int C, const bf16* dY, int ldy, int offy, bf16* dX, int ldx, int offx,
-                   bool acc) {
-  launch_pdl(k_upsample_grad, grid1((long)H * W * C / 32), 256, s, H, W, C, dY, ldy, offy, dX, ldx, offx, acc ? 1 : 0);
+void avgpool_grad(cudaStream_t s, int H, int W, int C, const bf16* dY, int ldy, bf16* g, int ldg, int offg,
+                  const bf16* act, int lda, int offa, float* db) {
+  launch_pdl(k_resize_relu_grad<FROM_POOL>, resize_grad_blocks((long)H * W, C), 256, s, H, W, C, dY, ldy, g, ldg, offg,
+             act, lda, offa, db);
 }
-void relu_bias_grad(cudaStream_t s, long npix, int C, bf16* G, int ldg, int offg, const bf16* Y, int ldy, int offy,
-                    float* db) {
-  const long rows = 256 / (C / 8);
-  long blocks = (npix + rows * 4 - 1) / (rows * 4);  // at least 4 pixels per thread
-  if (blocks > 1216) blocks = 1216;
-  if (blocks < 1) blocks = 1;
-  launch_pdl(k_relu_bias_grad, (int)blocks, 256, s, npix, C, G, ldg, offg, Y, ldy, offy, db);
+void upsample_grad(cudaStream_t s, int H, int W, int C, const bf16* dY, int ldy, bf16* g, int ldg, const bf16* act,
+                   int lda, float* db) {
+  launch_pdl(k_resize_relu_grad<FROM_UP>, resize_grad_blocks((long)H * W / 4, C), 256, s, H / 2, W / 2, C, dY, ldy, g,
+             ldg, 0, act, lda, 0, db);
 }
 void mse(cudaStream_t s, long npix, const float* out, int ldo, const float* target, const float* mask, float inv_count,
-         bf16* dout, int ldd, double* loss) {
-  launch_pdl(k_mse, grid1(npix), 256, s, npix, out, ldo, target, mask, inv_count, dout, ldd, loss);
+         bf16* dout, int ldd, double* loss, float* db) {
+  launch_pdl(k_mse, grid1(npix), 256, s, npix, out, ldo, target, mask, inv_count, dout, ldd, loss, db);
 }
 void adam(cudaStream_t s, long n, float* w, const float* g, float* m, float* v, bf16* wb, float lr, float b1, float b2,
           float eps, float c1, float c2) {

@@ -11,11 +11,17 @@ using bf16 = __nv_bfloat16;
 
 // What a convolution writes besides its output: its 2x2 average (pool, ldp
 // channels a pixel) and its nearest 2x upsampling (up, ldu channels a pixel).
+// A data gradient (no bias, no ReLU of its own) may take the activation it is
+// the gradient of (act, an output of a ReLU): it is zeroed where act is not
+// positive, and its sum over the pixels is added to db.
 struct ConvAlso {
   bf16* pool = nullptr;
   int ldp = 0;
   bf16* up = nullptr;
   int ldu = 0;
+  const bf16* act = nullptr;
+  int lda = 0, offa = 0;
+  float* db = nullptr;
 };
 // Y = act(conv3x3(X, W) + bias), zero padding, on the tcgen05 tensor cores
 // (k_conv_tc.cu); Cin, Cout % 16 == 0, ldx, offx, ldy, offy % 8 == 0; wpk:
@@ -47,14 +53,17 @@ bool conv_tc_failed();
 int conv3x3_wgrad(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* G, int ldg, int offg, const bf16* X,
                    int ldx, int offx, float* dW);
 void avgpool(cudaStream_t s, int H, int W, int C, const bf16* X, int ldx, int offx, bf16* Y, int ldy, int offy);
-void avgpool_grad(cudaStream_t s, int H, int W, int C, const bf16* dY, int ldy, int offy, bf16* dX, int ldx, int offx,
-                  bool acc);
-void upsample_grad(cudaStream_t s, int H, int W, int C, const bf16* dY, int ldy, int offy, bf16* dX, int ldx, int offx,
-                   bool acc);
-void relu_bias_grad(cudaStream_t s, long npix, int C, bf16* G, int ldg, int offg, const bf16* Y, int ldy, int offy,
-                    float* db);
+// The gradient g of a ReLU output (act; ld and off of its view) from the next
+// level's: zeroed where act is not positive, its sum over the pixels added to
+// db.  avgpool_grad: g += dY / 4 over each 2x2 block (H, W: the size of g).
+// upsample_grad: g = the sum of each 2x2 block of dY (H, W: the size of dY).
+void avgpool_grad(cudaStream_t s, int H, int W, int C, const bf16* dY, int ldy, bf16* g, int ldg, int offg,
+                  const bf16* act, int lda, int offa, float* db);
+void upsample_grad(cudaStream_t s, int H, int W, int C, const bf16* dY, int ldy, bf16* g, int ldg, const bf16* act,
+                   int lda, float* db);
+// db: the sum of dout's channel 0 is added to it
 void mse(cudaStream_t s, long npix, const float* out, int ldo, const float* target, const float* mask, float inv_count,
-         bf16* dout, int ldd, double* loss);
+         bf16* dout, int ldd, double* loss, float* db);
 void adam(cudaStream_t s, long n, float* w, const float* g, float* m, float* v, bf16* wb, float lr, float b1, float b2,
           float eps, float c1, float c2);
 void to_bf16(cudaStream_t s, long n, const float* a, bf16* b);

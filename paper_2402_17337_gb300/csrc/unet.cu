@@ -244,43 +244,53 @@ int forward(ibm_unet* n, cudaStream_t s, float* outp, bool train) {
   return rc;
 }
 
-// one conv's backward: mask the output gradient, accumulate dW and db, and
-// write the input gradient (unless it is the network input)
-int conv_backward(ibm_unet* n, const Edge& e, cudaStream_t s, bool need_dx) {
+// one conv's backward: accumulate dW and write the input gradient (unless it
+// is the network input).  The output gradient comes masked by its ReLU, with db
+// summed, from the kernel that wrote it; from: the convolution that made this
+// one's input, if nothing else is added to that gradient, so that this one
+// masks and sums for it.
+int conv_backward(ibm_unet* n, const Edge& e, cudaStream_t s, bool need_dx, int from) {
   const Conv& c = n->conv[e.conv];
   Level& L = n->lv[level_of(n, e.x)];
   Act gy = grad_of(n, e.y), gx = grad_of(n, e.x);
-  const long npix = (long)L.H * L.W;
-  relu_bias_grad(s, npix, c.cout, gy.p, gy.ld, gy.off, c.relu ? e.y.p : nullptr, e.y.ld, e.y.off, n->grad + c.b);
   if (conv3x3_wgrad(s, L.H, L.W, c.cin, c.cout, gy.p, gy.ld, gy.off, e.x.p, e.x.ld, e.x.off, n->grad + c.w)) return -1;
+  ConvAlso also;
+  if (from >= 0) {
+    also.act = e.x.p;
+    also.lda = e.x.ld;
+    also.offa = e.x.off;
+    also.db = n->grad + n->conv[from].b;
+  }
   if (need_dx)
     return conv3x3(s, L.H, L.W, c.cout, c.cin, gy.p, gy.ld, gy.off, n->wpkf + c.pkf, nullptr, gx.p, gx.ld, gx.off,
-                   false, nullptr);
+                   false, nullptr, also);
   return 0;
 }
 
 int backward(ibm_unet* n, cudaStream_t s) {
   const int* w = n->w;
   std::vector<Edge> E = edges(n);
-  int rc = conv_backward(n, E[14], s, true);  // head -> d(d0)
+  auto db = [&](int conv) { return n->grad + n->conv[conv].b; };
+  int rc = conv_backward(n, E[14], s, true, 13);  // head -> d(d0)
   for (int l = 0, k = 12; l <= 2; ++l, k -= 2) {
     Level& L = n->lv[l];
-    rc |= conv_backward(n, E[k + 1], s, true);  // d(d_l) -> d(bb_l)
-    rc |= conv_backward(n, E[k], s, true);      // d(bb_l) -> d(cat_l), both parts
+    rc |= conv_backward(n, E[k + 1], s, true, k);  // d(d_l) -> d(bb_l)
+    rc |= conv_backward(n, E[k], s, true, -1);     // d(bb_l) -> d(cat_l), both parts
     // the upsampled part of cat_l comes from d_{l+1} (or e3)
     if (l < 2)
-      upsample_grad(s, L.H, L.W, L.cup, L.gcat, L.cup + w[l], 0, n->lv[l + 1].gd, L.cup, 0, false);
+      upsample_grad(s, L.H, L.W, L.cup, L.gcat, L.cup + w[l], n->lv[l + 1].gd, L.cup, n->lv[l + 1].d, L.cup, db(k - 1));
     else
-      upsample_grad(s, L.H, L.W, L.cup, L.gcat, L.cup + w[l], 0, n->ge3, L.cup, 0, false);
+      upsample_grad(s, L.H, L.W, L.cup, L.gcat, L.cup + w[l], n->ge3, L.cup, n->e3, L.cup, db(7));
   }
   // encoder, from the bottom: e_l's gradient is in the skip slice of gcat_l
   // (decoder path) plus the pooling path of level l+1
   for (int l = 3; l >= 0; --l) {
-    rc |= conv_backward(n, E[2 * l + 1], s, true);  // d(e_l) -> d(a_l)
-    rc |= conv_backward(n, E[2 * l], s, l > 0);      // d(a_l) -> d(in_l)
+    rc |= conv_backward(n, E[2 * l + 1], s, true, 2 * l);  // d(e_l) -> d(a_l)
+    rc |= conv_backward(n, E[2 * l], s, l > 0, -1);        // d(a_l) -> d(in_l)
     if (l > 0) {
       Level& P = n->lv[l - 1];
-      avgpool_grad(s, P.H, P.W, w[l - 1], n->lv[l].gin, w[l - 1], 0, P.gcat, P.cup + w[l - 1], P.cup, true);
+      avgpool_grad(s, P.H, P.W, w[l - 1], n->lv[l].gin, w[l - 1], P.gcat, P.cup + w[l - 1], P.cup, P.cat,
+                   P.cup + w[l - 1], P.cup, db(2 * l - 1));
     }
   }
   return rc;
@@ -428,7 +438,8 @@ int ibm_unet_train_step(ibm_unet* n, const float* feat, const float* target, int
   UCUDA(cudaMemsetAsync(n->grad, 0, n->nparam * 4, s));
   UCUDA(cudaMemsetAsync(n->loss_d, 0, 8, s));
   const long npix = (long)H * W;
-  mse(s, npix, n->outf, 1, target, nullptr, 1.f / (float)npix, n->gout, 16, n->loss_d);
+  mse(s, npix, n->outf, 1, target, nullptr, 1.f / (float)npix, n->gout, 16, n->loss_d,
+      n->grad + n->conv[14].b);
   if (backward(n, s)) return IBM_E_CUDA;
   if (apply) {
     n->adam_t += 1;
