@@ -34,8 +34,7 @@
 // memory and the CTA skips the rest of its work.
 //
 // The weight gradient (k_conv3x3_wgrad_tc, below) is a GEMM over pixels
-// whose operands come MN-major straight from TMA boxes of the same
-// [pixel][8 channels] form.
+// whose operands come MN-major from boxes of the same form.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -93,6 +92,13 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
       "[%5];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
       : "memory");
+}
+// adds an FP32 box of shared memory to global memory
+__device__ __forceinline__ void tma_add_3d(const CUtensorMap* map, uint32_t src, int c0, int c1, int c2) {
+  asm volatile("cp.reduce.async.bulk.tensor.3d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(
+                   reinterpret_cast<uint64_t>(map)),
+               "r"(src), "r"(c0), "r"(c1), "r"(c2)
+               : "memory");
 }
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
@@ -478,27 +484,36 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 // ------------------------------------------------------- weight gradient
 //
 // dW[co][tap][ci] += sum over pixels p of G[p][co] X[p + shift(tap)][ci], a
-// GEMM per tap with M = 128 output channels (a tile of them; rows beyond
-// Cout zero), N = NT
-// input channels, K = pixels.  Both operands come as TMA boxes of [pixel][8
-// channels], i.e. MN-major: a core matrix is 8 pixels (K) x 8 channels (MN),
-// 16 bytes per pixel; K groups of 8 pixels are 128 bytes apart, MN groups of
-// 8 channels one box apart.  A CTA owns one tap row dy (taps 3 dy .. 3 dy + 2,
-// one accumulator of NT columns each), one NT-channel tile and a range of
-// pixel chunks (P pixels of one image row); the X box of a chunk spans P + 2
-// pixels of row y + dy, and tap dx reads it dx pixels further.  After its
-// chunks the CTA adds its accumulators to dW (vector atomics).
+// GEMM with K = pixels, M = 128 output channels (a tile of them), and N = 3 CB:
+// CB input channels (32 or 16) of the three image rows that the tap rows dy
+// read.  One MMA per tap column dx and 16 pixels covers three taps, and a CTA
+// all nine (three accumulators of 3 CB columns), so G and X are loaded once for
+// them.  Both operands come as TMA boxes of [row][pixel][channels], i.e.
+// MN-major with the swizzle of a pixel's width: 8-pixel groups (K) are
+// contiguous; the leading byte offset takes A to its next channel block and B
+// to the next image row.  X boxes start one row and one pixel before the
+// chunk's (P pixels of RB rows) and dx moves the start by a pixel.  Rows of A
+// beyond Cout read whatever lies there: they only reach accumulator lanes that
+// nothing reads.  After its chunks the CTA adds its accumulators to dW with
+// TMA reductions.
+//
+// The MMAs bound the large layers (each reads 4 KB of G and 96 CB bytes of X
+// from shared memory at 128 bytes/clock), its fixed latency the small ones.  A
+// training step of 32/64/128/128 at 256x512: 839 us with a CTA per tap row,
+// N = 32 to 128 for each tap, boxes of 8 channels and vector atomics; 808 us
+// with this tile and vector atomics; 763 us as it is.
 struct WgGeom {
-  int P;                // pixels per chunk (a multiple of 16, <= 128)
-  int NT, ntiles_ci;    // input channels per tile, tiles
-  int co_tiles;         // tiles of 128 output channels
-  int a_region, b_region, a_bytes, b_bytes, stage_bytes, stages;
+  int P, RB, XW;            // pixels (a multiple of 16, <= 128) and rows of a chunk; pixels of an X box row
+  int CA, CB;               // channels of a block of G and of the tile of X
+  int g_block, x_row;       // bytes of a G box and of a row of the X box
+  int a_bytes, stage_bytes, stages;
+  int nci, co_tiles;        // tiles of input and of output channels
   int tmem_cols, chunks_x, nchunks, ksplit;
 };
 
 __global__ void __launch_bounds__(TC_THREADS, 1)
-    k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap tmG, const __grid_constant__ CUtensorMap tmX, int Cin,
-                       int Cout, float* __restrict__ dW, WgGeom G, unsigned int* __restrict__ err) {
+    k_conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap tmG, const __grid_constant__ CUtensorMap tmX,
+                       const __grid_constant__ CUtensorMap tmW, int Cout, WgGeom G, unsigned int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bar_full[TC_STAGES_MAX], bar_empty[TC_STAGES_MAX], bar_acc;
   __shared__ uint32_t tmem_slot;
@@ -506,15 +521,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   volatile int* abort = &abort_flag;
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // work unit: blockIdx.x = (ksplit part, tap row, input-channel tile,
-  // output-channel tile)
-  const int part = blockIdx.x % G.ksplit;
-  int rest = blockIdx.x / G.ksplit;
-  const int dy = rest % 3;
-  rest /= 3;
-  const int zt = rest % G.ntiles_ci, co0 = (rest / G.ntiles_ci) * 128;
-  const int cog = (Cout - co0) / 8 < 16 ? (Cout - co0) / 8 : 16;  // 8-channel groups of G in this tile
-  const int tx_bytes = cog * G.P * 16 + (G.NT / 8) * (G.P + 2) * 16;
+  // work unit: blockIdx.x = (ksplit part, input-channel tile, output-channel tile)
+  const int part = blockIdx.x % G.ksplit, unit = blockIdx.x / G.ksplit;
+  const int ci0 = unit % G.nci * G.CB, co0 = unit / G.nci * 128;
+  const int nb = (Cout - co0 < 128 ? Cout - co0 : 128) / G.CA;  // blocks of G in this tile
   const int c_begin = (int)((long)G.nchunks * part / G.ksplit), c_end = (int)((long)G.nchunks * (part + 1) / G.ksplit);
   const int nq = c_end - c_begin, S = G.stages;
   if (warp == 0) {
@@ -523,14 +533,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  // the MN groups of A beyond Cout are never loaded: zero them in every stage
-  const int zero_bytes = (16 - cog) * G.a_region;
-  for (int s = 0; s < S; ++s) {
-    uint4* z = reinterpret_cast<uint4*>(smem_raw + (sbase - smem_u32(smem_raw)) + s * G.stage_bytes +
-                                        cog * G.a_region);
-    for (int k = threadIdx.x; k < zero_bytes / 16; k += blockDim.x) z[k] = make_uint4(0, 0, 0, 0);
-  }
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic writes seen by the tensor cores
   if (threadIdx.x == 32) {
     for (int s = 0; s < S; ++s) {
       mbar_init(smem_u32(&bar_full[s]), 1);
@@ -543,6 +545,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   if (threadIdx.x == 128) {
     prefetch_map(&tmG);
     prefetch_map(&tmX);
+    prefetch_map(&tmW);
   }
   tc_fence_before();
   __syncthreads();
@@ -553,39 +556,43 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 
   if (warp == 4) {
     if (lane == 0) {
+      const int tx_bytes = nb * G.g_block + (G.RB + 2) * G.x_row;
       int issued = 0;
       for (int q = 0; q < nq; ++q) {
         const int s = q % S, c = c_begin + q;
         if (q >= S && !wait_or_abort(smem_u32(&bar_empty[s]), (uint32_t)(q / S - 1) & 1u, abort)) break;
-        const int x0 = (c % G.chunks_x) * G.P, y = c / G.chunks_x;
+        const int x0 = (c % G.chunks_x) * G.P, y0 = c / G.chunks_x * G.RB;
         const uint32_t st = sbase + s * G.stage_bytes, bar = smem_u32(&bar_full[s]);
         mbar_expect_tx(bar, tx_bytes);
-        for (int g = 0; g < cog; ++g) tma_load_3d(st + g * G.a_region, &tmG, co0 + 8 * g, x0, y, bar);
-        for (int g = 0; g < G.NT / 8; ++g)
-          tma_load_3d(st + G.a_bytes + g * G.b_region, &tmX, zt * G.NT + 8 * g, x0 - 1, y + dy - 1, bar);
+        for (int g = 0; g < nb; ++g) tma_load_3d(st + g * G.g_block, &tmG, co0 + g * G.CA, x0, y0, bar);
+        tma_load_3d(st + G.a_bytes, &tmX, ci0, x0 - 1, y0 - 1, bar);
         issued = q + 1;
       }
       if (*abort && issued > 0) mbar_wait(smem_u32(&bar_full[(issued - 1) % S]), (uint32_t)((issued - 1) / S) & 1u);
     }
     __syncwarp();
   } else if (warp == 5) {
-    // both operands MN-major (transpose bits), N = NT, M = 128
     if (elect_one()) {
-      const uint32_t idesc = instr_desc(G.NT) | (1u << 15) | (1u << 16);
-      const uint32_t a_hi = desc_hi(G.a_region), b_hi = desc_hi(G.b_region);
+      // both operands MN-major (transpose bits)
+      const uint32_t idesc = instr_desc(3 * G.CB) | (1u << 15) | (1u << 16);
+      const uint32_t a_hi = desc_hi_swizzled(2 * G.CA), b_hi = desc_hi_swizzled(2 * G.CB);
+      const uint32_t a_step = 2 * G.CA, b_step = 2 * G.CB, dx_step = G.CB / 8, cols = 3 * G.CB;  // / 16 bytes; columns
       int done = 0;
       for (int q = 0; q < nq; ++q) {
         const int s = q % S;
         if (!wait_or_abort(smem_u32(&bar_full[s]), (uint32_t)(q / S) & 1u, abort)) break;
         tc_fence_after();
         const uint32_t st = sbase + s * G.stage_bytes;
-        uint32_t a = desc_lo(st, 128), b = desc_lo(st + G.a_bytes, 128);
-        for (int ks = 0; ks < G.P / 16; ++ks) {
+        for (int r = 0; r < G.RB; ++r) {
+          uint32_t a = desc_lo(st + r * G.P * G.CA * 2, G.g_block);
+          uint32_t b = desc_lo(st + G.a_bytes + r * G.x_row, G.x_row);
+          for (int ks = 0; ks < G.P / 16; ++ks) {
 #pragma unroll
-          for (int t = 0; t < 3; ++t)
-            tc_mma(tmem + (uint32_t)(t * G.NT), a, a_hi, b + t, b_hi, idesc, (uint32_t)(q | ks));
-          a += 16;
-          b += 16;
+            for (int dx = 0; dx < 3; ++dx)
+              tc_mma(tmem + dx * cols, a, a_hi, b + dx * dx_step, b_hi, idesc, (uint32_t)(q | r | ks));
+            a += a_step;
+            b += b_step;
+          }
         }
         tc_commit(smem_u32(&bar_empty[s]));
         done = q + 1;
@@ -598,21 +605,34 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
     __syncwarp();
   } else if (nq > 0) {
-    // epilogue: lane = output channel co, 16 input channels per load
-    if (wait_or_abort(smem_u32(&bar_acc), 0u, abort)) {
+    // epilogue: lane = output channel, 16 input channels of a tap per load; the accumulators go to shared memory
+    // (free now) as one [co][CB] box per tap, swizzled against bank conflicts, and one TMA reduction per tap adds
+    // it to dW
+    const bool ok = wait_or_abort(smem_u32(&bar_acc), 0u, abort);
+    if (!ok && lane == 0) atomicOr_system(err, 1u);
+    const int row = threadIdx.x, rows = Cout < 128 ? Cout : 128;
+    if (ok && warp * 32 < rows) {
       tc_fence_after();
-      const int co = co0 + warp * 32 + lane;
-      for (int t = 0; t < 3; ++t)
-        for (int c0 = 0; c0 < G.NT; c0 += 16) {
+      unsigned char* base = smem_raw + (sbase - smem_u32(smem_raw)) + row * G.CB * 4;
+      const int swz = G.CB == 32 ? row & 7 : (row >> 1) & 3;
+      for (int t = 0; t < 9; ++t)
+        for (int c0 = 0; c0 < G.CB; c0 += 16) {
           float v[16];
-          tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(t * G.NT + c0), v);
-          if (co >= Cout || zt * G.NT + c0 >= Cin) continue;
-          float4* dst = reinterpret_cast<float4*>(dW + ((size_t)co * 9 + 3 * dy + t) * Cin + zt * G.NT + c0);
+          tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(t * G.CB + c0), v);
+          if (row >= rows) continue;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) atomicAdd(dst + j, make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]));
+          for (int j = 0; j < 4; ++j)
+            *reinterpret_cast<float4*>(base + t * rows * G.CB * 4 + (((c0 / 4 + j) ^ swz) * 16)) =
+                make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
         }
-    } else if (lane == 0) {
-      atomicOr_system(err, 1u);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    if (threadIdx.x == 0 && !*abort) {
+      // accumulator columns are [dx][dy][CB]: tap 3 dy + dx
+      for (int t = 0; t < 9; ++t) tma_add_3d(&tmW, sbase + t * rows * G.CB * 4, ci0, t % 3 * 3 + t / 3, co0);
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // shared memory has been read
     }
   }
   tc_fence_before();
@@ -755,34 +775,43 @@ int conv3x3_wgrad(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* G
     return -1;
   }
   WgGeom G{};
+  auto block = [](int C) { return C % 64 == 0 ? 64 : (C % 32 == 0 ? 32 : 16); };
   G.P = W >= 128 ? 128 : (pow2_at_least(W) < 16 ? 16 : pow2_at_least(W));
-  G.NT = Cin <= 128 ? Cin : 128;
-  G.ntiles_ci = (Cin + G.NT - 1) / G.NT;
+  G.RB = 256 / G.P;  // 256 pixels a chunk: 763 us a training step of 32/64/128/128 at 256x512, 765 with 128
+  G.XW = G.P + 8;
+  G.CA = block(Cout);
+  G.CB = Cin % 32 == 0 ? 32 : 16;  // 9 CB accumulator columns
+  G.nci = Cin / G.CB;
   G.co_tiles = (Cout + 127) / 128;
-  G.a_region = G.P * 16;
-  G.a_bytes = 16 * G.a_region;
-  G.b_region = ((G.P + 2) * 16 + 127) / 128 * 128;
-  G.b_bytes = (G.NT / 8) * G.b_region;
-  G.stage_bytes = (G.a_bytes + G.b_bytes + 1023) / 1024 * 1024;
-  G.stages = 3 * G.stage_bytes + 1024 <= TC_SMEM_MAX ? 3 : 2;
-  G.tmem_cols = pow2_at_least(3 * G.NT < 32 ? 32 : 3 * G.NT);
+  G.g_block = G.RB * G.P * G.CA * 2;
+  G.x_row = G.XW * G.CB * 2;
+  G.a_bytes = ((Cout < 128 ? Cout : 128) / G.CA * G.g_block + 1023) / 1024 * 1024;
+  G.stage_bytes = (G.a_bytes + (G.RB + 2) * G.x_row + 1023) / 1024 * 1024;
+  // the last stage's A reads 128 / CA blocks, also where fewer are loaded
+  const int over = 128 / G.CA * G.g_block - G.stage_bytes, extra = 1024 + (over > 0 ? over : 0);
+  G.stages = 4;
+  while (G.stages > 2 && G.stages * G.stage_bytes + extra > TC_SMEM_MAX) --G.stages;
+  G.tmem_cols = pow2_at_least(9 * G.CB);
   G.chunks_x = (W + G.P - 1) / G.P;
-  G.nchunks = H * G.chunks_x;
-  int smem = G.stages * G.stage_bytes + 1024;
+  G.nchunks = (H + G.RB - 1) / G.RB * G.chunks_x;
+  int smem = G.stages * G.stage_bytes + extra;
   const int smem_tmem = tmem_min_smem(G.tmem_cols);
   if (smem < smem_tmem) smem = smem_tmem;
   if (smem > TC_SMEM_MAX) {
     set_last_error("weight-gradient tile does not fit in shared memory");
     return -1;
   }
-  CUtensorMap mg, mx;
+  auto swizzle = [](int C) {
+    return C == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : (C == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
+  };
+  CUtensorMap mg, mx, mw;
   cuuint32_t estr[3] = {1, 1, 1};
   {
     cuuint64_t dims[3] = {(cuuint64_t)Cout, (cuuint64_t)W, (cuuint64_t)H};
     cuuint64_t strides[2] = {(cuuint64_t)ldg * 2, (cuuint64_t)W * ldg * 2};
-    cuuint32_t box[3] = {8, (cuuint32_t)G.P, 1};
+    cuuint32_t box[3] = {(cuuint32_t)G.CA, (cuuint32_t)G.P, (cuuint32_t)G.RB};
     if (enc(&mg, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<bf16*>(Gd + offg), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle(G.CA), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
       set_last_error("cuTensorMapEncodeTiled rejected a gradient view");
       return -1;
@@ -791,11 +820,22 @@ int conv3x3_wgrad(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* G
   {
     cuuint64_t dims[3] = {(cuuint64_t)Cin, (cuuint64_t)W, (cuuint64_t)H};
     cuuint64_t strides[2] = {(cuuint64_t)ldx * 2, (cuuint64_t)W * ldx * 2};
-    cuuint32_t box[3] = {8, (cuuint32_t)(G.P + 2), 1};
+    cuuint32_t box[3] = {(cuuint32_t)G.CB, (cuuint32_t)G.XW, (cuuint32_t)(G.RB + 2)};
     if (enc(&mx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<bf16*>(X + offx), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle(G.CB), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
       set_last_error("cuTensorMapEncodeTiled rejected an activation view");
+      return -1;
+    }
+  }
+  {
+    cuuint64_t dims[3] = {(cuuint64_t)Cin, 9, (cuuint64_t)Cout};
+    cuuint64_t strides[2] = {(cuuint64_t)Cin * 4, (cuuint64_t)Cin * 36};
+    cuuint32_t box[3] = {(cuuint32_t)G.CB, 1, (cuuint32_t)(Cout < 128 ? Cout : 128)};
+    if (enc(&mw, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, dW, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            G.CB == 32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
+      set_last_error("cuTensorMapEncodeTiled rejected a weight gradient");
       return -1;
     }
   }
@@ -812,7 +852,7 @@ int conv3x3_wgrad(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* G
   if (per_sm > 512 / G.tmem_cols) per_sm = 512 / G.tmem_cols;
   if (per_sm < 1) per_sm = 1;
   // split the pixel chunks so that the CTAs fill the device once
-  const int units = 3 * G.ntiles_ci * G.co_tiles;
+  const int units = G.nci * G.co_tiles;
   G.ksplit = (int)((long)nsm * per_sm / units);
   if (G.ksplit < 1) G.ksplit = 1;
   if (G.ksplit > G.nchunks) G.ksplit = G.nchunks;
@@ -826,7 +866,7 @@ int conv3x3_wgrad(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* G
   at[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = at;
   lc.numAttrs = 1;
-  if (cudaLaunchKernelEx(&lc, k_conv3x3_wgrad_tc, mg, mx, Cin, Cout, dW, G, err_dev) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&lc, k_conv3x3_wgrad_tc, mg, mx, mw, Cout, G, err_dev) != cudaSuccess) {
     set_last_error("weight-gradient launch failed");
     return -1;
   }
