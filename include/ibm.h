@@ -185,7 +185,7 @@ int ibm_poisson_solve(ibm_ctx* ctx, const double* b_dev, double* phi_dev, double
  * face coordinates and its own buffers, and every scratch value (the 1-D
  * coefficients and the residual-norm accumulator) lives in one fixed-size
  * static device array of the library, which each GPU that loads the library
- * holds (256 KB) until the process exits.
+ * holds (9.9 MB) until the process exits.
  *
  * Solves L_p phi = b on the grid with face coordinates xf (nx+1 host
  * doubles) and yf (ny+1 host doubles), homogeneous Neumann, by red-black SOR

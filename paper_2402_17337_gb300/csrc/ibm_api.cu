@@ -1941,7 +1941,7 @@ int ibm_create_grid(const ibm_grid_params* params, ibm_ctx** out) {
     rc = IBM_E_CUDA;
   if (!rc) rc = ensure_history(c, 1024);
   if (!rc && P.precision == 0) {
-    c->sor64 = sor64_plan(P.nx, P.ny, true);
+    c->sor64 = sor64_plan(P.nx, P.ny);
     if (c->sor64.kind != Sor64Plan::NONE) {
       // one block: the result, the norms' slots, the exchange words
       const size_t nt = c->sor64.kind == Sor64Plan::TILES ? sor64_max_tiles() : 0;

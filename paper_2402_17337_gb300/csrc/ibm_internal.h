@@ -138,6 +138,9 @@ struct Sor64Tiles {
   unsigned long long* norms;   // 4 words per tile
   unsigned first;              // exchanges are numbered from first + 1; no number is used twice on the buffers
 };
+// the most cells and tiles of a plan of tiles
+constexpr long kSor64TilesCells = 300000;
+constexpr int kSor64MaxTiles = 1024;
 // exchange numbers one launch may use
 constexpr unsigned kSor64Numbers = 1u << 16;
 enum { SOR64_MORE = 0, SOR64_OK, SOR64_NOCONV, SOR64_DIVERGED };
@@ -151,8 +154,7 @@ struct Sor64Plan {
   int nbx = 0, nby = 0, K = 0;
   size_t smem = 0;
 };
-// tiles: the caller can pass Sor64Tiles
-Sor64Plan sor64_plan(int nx, int ny, bool tiles);
+Sor64Plan sor64_plan(int nx, int ny);
 int sor64_max_tiles();
 cudaError_t launch_sor64(cudaStream_t s, const Sor64Plan& p, const Sor64Args& a, const Sor64Tiles& t, Sor64Result* out);
 

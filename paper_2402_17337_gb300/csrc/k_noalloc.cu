@@ -5,15 +5,17 @@
 // that forbids allocation on its hot path, or a real-time loop that cannot
 // take the device-wide synchronisation an allocation may cause.  This
 // variant of the red-black SOR pressure solve therefore keeps its scratch
-// (the 1-D coefficient arrays and the residual-norm accumulator) in one
-// file-scope __device__ array of fixed size, so the caller only passes its
-// own input and output buffers.  Every GPU that loads the library holds this
-// array (256 KB) until the process exits.
+// (the 1-D coefficient arrays, the residual-norm accumulator and the exchange
+// buffers of the tiles that keep a grid on chip) in one file-scope __device__
+// array of fixed size, so the caller only passes its own input and output
+// buffers.  Every GPU that loads the library holds this array (9.9 MB) until
+// the process exits.
 //
 // The iterates are those of ibm_poisson_solve on an FP64 (precision 0)
 // context of the same grid: same sweep order, same fma chains, same
 // reciprocal diagonal (1/(aE+aW+aN+aS), computed here on the device with the
 // same IEEE operations).
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -27,8 +29,11 @@ namespace {
 constexpr int NOALLOC_MAX_N = 8192;  // largest nx and ny
 constexpr int COEF = 4 * NOALLOC_MAX_N;
 
-// [0, COEF): pE, pW (x), pN, pS (y); then the norm accumulator and the gauge value
-static __device__ __align__(256) double g_noalloc_scratch[COEF + 8];
+// [0, COEF): pE, pW (x), pN, pS (y); the norm accumulator, the gauge value and
+// the sweeps' result; from TILES on the tiles' norms (4 words a tile) and
+// exchange words (4 a cell)
+constexpr int TILES = COEF + 8;
+static __device__ __align__(256) double g_noalloc_scratch[TILES + 4 * ibm::kSor64MaxTiles + 4 * ibm::kSor64TilesCells];
 
 constexpr int MAX_DEVICES = 64;
 double* g_scratch_addr[MAX_DEVICES] = {nullptr};
@@ -195,20 +200,37 @@ extern "C" int ibm_poisson_solve_noalloc(int nx, int ny, const double* xf, const
   double* ref = scratch + COEF + 1;
   const int m = check_every > 0 ? check_every : 8;
   const int maxs = max_sweeps > 0 ? max_sweeps : 1000000;
-  // a grid that one cluster holds: sweeps and checks on the device (the result
-  // in the scratch behind the gauge value)
-  const ibm::Sor64Plan plan = ibm::sor64_plan(nx, ny, false);
-  if (plan.kind == ibm::Sor64Plan::CLUSTER) {
+  // a grid that stays on chip: sweeps and checks on the device (rule and times
+  // in k_sor64.cu; a whole solve at 192x96 takes 6.3 ms, 24.6 with the launches
+  // per half-sweep below, at 384x192 17.6 and 51.3 ms)
+  const ibm::Sor64Plan plan = ibm::sor64_plan(nx, ny);
+  if (plan.kind != ibm::Sor64Plan::NONE) {
     ibm::Sor64Result* out = (ibm::Sor64Result*)(scratch + COEF + 2);
+    ibm::Sor64Tiles tiles{};
+    tiles.norms = (unsigned long long*)(scratch + TILES);
+    tiles.words = tiles.norms + 4 * ibm::sor64_max_tiles();
+    tiles.stride = 2 * (size_t)nx * ny;
+    const size_t tile_bytes = 32 * ((size_t)ibm::sor64_max_tiles() + (size_t)nx * ny);
     for (int done = 0;;) {
+      // exchange numbers are used once: the buffers are cleared at the start and when they run out
+      if (plan.kind == ibm::Sor64Plan::TILES && (done == 0 || tiles.first > UINT_MAX - 2 * ibm::kSor64Numbers)) {
+        const cudaError_t e = cudaMemsetAsync(tiles.norms, 0, tile_bytes, s);
+        if (e != cudaSuccess) return cuda_fail("cudaMemsetAsync of the exchange buffers", e);
+        tiles.first = 0;
+      }
       const ibm::Sor64Args a{nx, ny, nx, 0, g.pE, g.pW, g.pN, g.pS, phi_dev, b_dev, nullptr, omega, tol, m, maxs - done, 8192};
       ibm::Sor64Result r{};
-      cudaError_t e = ibm::launch_sor64(s, plan, a, ibm::Sor64Tiles{}, out);
+      cudaError_t e = ibm::launch_sor64(s, plan, a, tiles, out);
       if (e != cudaSuccess) return cuda_fail("the launch of the sweeps", e);
       e = cudaMemcpyAsync(&r, out, sizeof r, cudaMemcpyDeviceToHost, s);
       if (e != cudaSuccess) return cuda_fail("cudaMemcpyAsync of the result", e);
       e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return cuda_fail("the sweeps (cudaStreamSynchronize)", e);
+      tiles.first += ibm::kSor64Numbers;
+      if (r.late) {
+        ibm::set_last_error("ibm_poisson_solve_noalloc: a block waited too long for its neighbours");
+        return IBM_E_TIMEOUT;
+      }
       double v;
       std::memcpy(&v, &r.bits, sizeof v);
       if (sweeps) *sweeps = done + r.checked;
@@ -226,7 +248,7 @@ extern "C" int ibm_poisson_solve_noalloc(int nx, int ny, const double* xf, const
     }
   }
   dim3 blk(32, 8), grd_res((nx + 31) / 32, (ny + 7) / 8), grd_half(((nx + 1) / 2 + 31) / 32, (ny + 7) / 8);
-  for (int it = 0; plan.kind != ibm::Sor64Plan::CLUSTER; ++it) {
+  for (int it = 0; plan.kind == ibm::Sor64Plan::NONE; ++it) {
     if (it % m == 0) {
       unsigned long long bits = 0;
       cudaError_t e = cudaMemsetAsync(norm, 0, sizeof(unsigned long long), s);

@@ -92,17 +92,20 @@ constexpr size_t CL_SMEM = 100 * 1024;
 // Which kernel a grid takes (us per sweep, checks every 8 sweeps included;
 // the launch-per-half-sweep kernels of k_sor.cu in brackets):
 //   70x45    cluster 1.8 [10.4], tiles 2.1
-//   100x60   cluster 2.1, tiles 2.2
-//   133x67   cluster 2.6 [10.7], tiles 2.3
+//   110x56   cluster 2.1 [10.5]
+//   133x67   cluster 2.6 [10.7], tiles 2.9
+//   160x80   cluster 3.0 [11.0], tiles 2.9
+//   192x96   tiles 2.8 [11.0]
 //   192x128  cluster 4.8, tiles 2.7 [10]
+//   384x192  tiles 3.8 [11.0]
 //   512x256  tiles 5.1 [10.1]
 //   700x350  tiles 7.3 [10.2]
 //   1024x512 tiles 12 [10.3]
-// so one cluster up to kClusterCells, tiles up to kTilesCells, and above
+// so one cluster up to kClusterCells, tiles up to kSor64TilesCells, and above
 // that the kernels of k_sor.cu, whose launches are then long enough.  A
 // half-sweep's floor is its chain of eight dependent FP64 instructions, about
 // 160 clocks each, and a barrier: 0.9 us.
-constexpr long kClusterCells = 7500, kTilesCells = 300000;
+constexpr long kClusterCells = 10500;
 // Model of the tiles' time that picks their shape, in clocks, fitted to those
 // measurements: one exchange, one half-sweep's barrier and latency, and 32
 // updates (128 of FP64 issue, the rest shared memory).
@@ -332,7 +335,7 @@ __global__ void __launch_bounds__(TL_THREADS, 1) k_sor64_tiles(Sor64Args A, Sor6
       aS[c][k] = in ? A.pS[j] : 0.0;
       const size_t o = A.off + (size_t)j * A.pitch + i;
       bb[c][k] = in ? A.b[o] : 0.0;
-      dd[c][k] = in ? A.invd[o] : 0.0;
+      dd[c][k] = !in ? 0.0 : A.invd ? A.invd[o] : 1.0 / (aE[c][k] + aW[c][k] + aN[c][k] + aS[c][k]);
       pos[c][k] = in ? (j - Y0) * P + i - X0 : 0;
     }
   __syncthreads();
@@ -520,19 +523,19 @@ long tiles_list(int w, int h, int K) {
 }  // namespace
 
 // Which kernel a grid takes, from its size alone.
-Sor64Plan sor64_plan(int nx, int ny, bool tiles) {
+Sor64Plan sor64_plan(int nx, int ny) {
   Sor64Plan p;
   const Sor64Dev& d = sor64_device();
   if (d.cluster && ny >= d.cluster) {
     const int rows = (ny + d.cluster - 1) / d.cluster, w2 = (nx + 1) / 2;
     if (rows * w2 <= CL_THREADS * CL_CPT && sizeof(double) * (rows + 2) * (nx + 2) <= CL_SMEM &&
-        (!tiles || (long)nx * ny <= kClusterCells)) {
+        (!d.coop || (long)nx * ny <= kClusterCells)) {
       p.kind = Sor64Plan::CLUSTER;
       p.nbx = d.cluster;
       return p;
     }
   }
-  if (!tiles || !d.coop || d.sms < 1 || (long)nx * ny > kTilesCells) return p;
+  if (!d.coop || d.sms < 1 || d.sms > kSor64MaxTiles || (long)nx * ny > kSor64TilesCells) return p;
   // Tiles: the split and halo depth with the smallest modelled time per
   // half-sweep: the updates of the shrinking region, and an exchange every K
   // half-sweeps.

@@ -14,7 +14,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("nx,ny", [(5, 4), (9, 200), (64, 15), (33, 16), (17, 17), (128, 93), (129, 95), (41, 300),
-                                   (300, 41), (191, 129), (513, 257), (500, 500), (547, 548), (548, 549), (75, 100), (76, 100)])
+                                   (300, 41), (191, 129), (513, 257), (500, 500), (547, 548), (548, 549), (75, 100), (76, 100),
+                                   (105, 100), (106, 100)])
 @pytest.mark.parametrize("m,cap", [(8, 60), (3, 20), (1, 2), (7, 49)])
 def test_sweeps_on_chip_match_oracle(nx, ny, m, cap):
     import torch
@@ -63,3 +64,31 @@ def test_two_streams_and_threads_solve_at_once():
     for t in ts:
         t.join()
     assert all(out[k][0][0] == -3 and np.array_equal(out[k][1], out[0][1]) for k in range(3))
+
+
+@pytest.mark.parametrize("nx,ny", [(105, 100), (106, 100), (131, 67), (384, 193), (547, 548), (548, 549)])
+@pytest.mark.parametrize("m,cap", [(8, 60), (7, 49)])
+def test_allocation_free_solve_repeats_the_context_bit_for_bit(nx, ny, m, cap):
+    """Tiles in the static scratch, from the smallest grid that takes them to the first that does not; two calls,
+    the second on buffers that hold the first one's exchanges."""
+    import ctypes as C
+
+    import torch
+    import paper_2402_17337_gb300 as ibm
+    from paper_2402_17337_gb300 import build
+    build.build()
+    g = ibm.Solver(x0=0.0, x1=2.0 + nx / ny, y0=0.0, y1=1.5, nx=nx, ny=ny, hmin=0.0, dt=1.0)
+    xf, yf = g.grid()
+    fn, D = ibm.lib().ibm_poisson_solve_noalloc, C.POINTER(C.c_double)
+    fn.argtypes = [C.c_int, C.c_int, D, D, C.c_void_p, C.c_void_p, C.c_double, C.c_double, C.c_int, C.c_int,
+                   C.c_void_p, C.POINTER(C.c_int), C.POINTER(C.c_double)]
+    for seed in (1, 2):
+        bd = torch.tensor(W.random_field((ny, nx), seed=seed), device="cuda")
+        p, q = torch.zeros_like(bd), torch.zeros_like(bd)
+        torch.cuda.synchronize()
+        rc, sg, rg = g.poisson_solve(bd.data_ptr(), p.data_ptr(), 1e-300, m, cap)
+        sn, rn = C.c_int(-1), C.c_double(-1.0)
+        assert fn(nx, ny, xf.ctypes.data_as(D), yf.ctypes.data_as(D), bd.data_ptr(), q.data_ptr(), g.P.omega_p, 1e-300,
+                  m, cap, None, C.byref(sn), C.byref(rn)) == rc == -3
+        assert sn.value == sg and rn.value == rg
+        assert torch.equal(p, q)
