@@ -63,6 +63,7 @@ SOR32_TRAFFIC = {
     ("plunge_4096x2048", (80, 16, 16, 10)): 118.77504e6,
     ("plunge_2048x1024", (80, 16, 16, 9)): 25.23264e6,
     ("plunge_4096x2048", (80, 16, 16, 9)): 115.576576e6,
+    ("plunge_2048x1024", (80, 16, 8, 11)): 25.2224e6,
 }
 # warp instructions issued per launch of the FP32 sweep kernel (ncu smsp__inst_executed.sum of one
 # launch, profiles/k_sor32_rb_*.md), by workload and tile shape: the issue roofline of a kernel that is
@@ -76,6 +77,7 @@ SOR32_INST = {
     ("plunge_4096x2048", (80, 16, 16, 10)): 52.308382e6,
     ("plunge_2048x1024", (80, 16, 16, 9)): 13.40867e6,
     ("plunge_4096x2048", (80, 16, 16, 9)): 52.41571e6,
+    ("plunge_2048x1024", (80, 16, 8, 11)): 8.60388e6,
 }
 WORKLOADS = ("plunge_2048x1024", "plunge_4096x2048", "unet_1024x512", "batch64")
 METRIC = "cell-steps/s at div<1e-8: learned warm-start+mixed vs plain FP64, one GB300"
@@ -696,7 +698,8 @@ def main():
                          "peak_inst_per_s": peak_issue, "frac": inst / t_launch / peak_issue,
                          "note": f"warp instructions of one launch (ncu) over the live launch time, against "
                                  f"{n_sm} SMs x 4 issue slots per clock at {clk_mhz:.0f} MHz (sampled median)"}
-            roof = {"bound": "hbm", "kernel": f"k_sor32_rb (FP32 red-black SOR, tile {rows} rows x 128 cells, "
+            kernel = "k_sor32_tma" if prof["sor_form"] == 11 else "k_sor32_rb"
+            roof = {"bound": "hbm", "kernel": f"{kernel} (FP32 red-black SOR, tile {rows} rows x 128 cells, "
                                               f"{half} half-sweeps per launch, chosen by the autotuner)",
                     "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                     "frac": achieved / peaks["hbm_gbs"], "traffic": traffic, "launch_us": t_launch * 1e6,

@@ -43,7 +43,7 @@ extern "C" {
 #define IBM_E_CUDA (-2)     /* a CUDA call failed */
 #define IBM_E_NOCONV (-3)   /* an SOR solve hit max_sweeps before its tolerance */
 #define IBM_E_DIVERGED (-4) /* a residual norm became NaN or Inf */
-#define IBM_E_TIMEOUT (-5)  /* a bounded device-side wait gave up */
+#define IBM_E_TIMEOUT (-5)  /* a bounded device-side wait gave up (pressure sweeps, U-Net) */
 
 typedef struct ibm_ctx ibm_ctx;
 
@@ -215,7 +215,8 @@ int ibm_poisson_solve_noalloc(int nx, int ny, const double* xf, const double* yf
 /* Counters of a context.  With profiling on, each run of pressure SOR
  * launches between two residual checks is bracketed by CUDA events on the
  * context's stream; sweep_ms is the summed device time of those runs and
- * sweep_launches the number of launches they contain. */
+ * sweep_launches the number of launches they contain (on FP64 grids up to
+ * 300 000 cells one launch runs a whole solve with its residual checks). */
 typedef struct {
   long long launches;        /* kernels launched by this context */
   long long sweep_launches;  /* pressure SOR sweep launches inside timed runs */

@@ -335,7 +335,7 @@ void launch_dc_residual(cudaStream_t s, const Geo& g, int pk, const double* phi_
 // pdl: launch as a programmatic dependent of the previous kernel on the
 // stream (consecutive sweep launches outside graph capture).  With
 // zero_init = 0 the previous kernel must be a sweep launch of the same run:
-// forms 6 and 7 then read r and 1/d before waiting for it.
+// forms 6 to 11 then read r and 1/d before waiting for it.
 void launch_sor32(cudaStream_t s, int cfg, const Geo32& g, const float* e_in, float* e_out, const float* r,
                   const float* invd, float omega, int zero_init, int pdl = 0);
 

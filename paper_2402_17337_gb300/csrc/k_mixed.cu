@@ -1042,7 +1042,7 @@ __global__ void __launch_bounds__(32 * C::NY, C::MINB)
   // programmatic dependent launch (a no-op unless the launch asks for it):
   // this launch reads what the previous kernel wrote only after that kernel
   // has completed and its writes are visible, and then lets the next sweep
-  // launch start (forms 6 and 7 do both inside, after loading r and 1/d)
+  // launch start (forms 6 to 10 do both inside, after loading r and 1/d)
   if constexpr (C::V < 6) {
     griddep_wait();
     griddep_release();
@@ -1060,7 +1060,7 @@ __global__ void __launch_bounds__(32 * C::NY, C::MINB)
   // programmatic dependent launch (a no-op unless the launch asks for it):
   // the descriptor tables are rewritten between rounds, so every CTA waits
   // for the previous kernel before its first load and then lets the next
-  // launch start (forms 6 and 7 wait and release again inside; both return
+  // launch start (forms 6 to 10 wait and release again inside; both return
   // at once the second time)
   griddep_wait();
   griddep_release();
