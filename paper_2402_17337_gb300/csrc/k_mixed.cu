@@ -848,6 +848,13 @@ __device__ __forceinline__ void tma_field(void* dst, const CUtensorMap* map, int
       "l"(reinterpret_cast<uint64_t>(map)), "r"(k0), "r"(j0), "r"(0), "r"(bar)
       : "memory");
 }
+// Makes a tensor map in global memory that the host has rewritten by a copy
+// visible to this CTA's tensor copies.  Neither stream order nor
+// griddepcontrol.wait orders the proxy through which those read a map: without
+// this a copy may still use what the map's address held before.
+__device__ __forceinline__ void acquire_map(const CUtensorMap* map) {
+  asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(map) : "memory");
+}
 __device__ __forceinline__ void expect_bytes(unsigned bar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
@@ -1141,6 +1148,7 @@ __global__ void __launch_bounds__(32 * C::NY, C::MINB)
   griddep_wait();  // the descriptor tables are rewritten between rounds
   griddep_release();
   constexpr unsigned bytes = sizeof(float2) * S::field;
+  int acquired = -1;  // last case whose maps this CTA has acquired (its tiles come case by case)
   // one thread: the first tile at or after t of a case with sweeps left in this round, its descriptor into slot[w],
   // its copies on their way
   auto request = [&](int t, int w) {
@@ -1155,6 +1163,12 @@ __global__ void __launch_bounds__(32 * C::NY, C::MINB)
       slot[w] = c;
       const int u = t - c.first, k0 = u % c.tiles_x * S::TK - S::HK, j0 = u / c.tiles_x * C::TY - C::K;
       const CUtensorMap* m = reinterpret_cast<const CUtensorMap*>(c.maps);
+      if (lo != acquired) {
+        acquire_map(m + c.flip);
+        acquire_map(m + 2);
+        acquire_map(m + 3);
+        acquired = lo;
+      }
       expect_bytes(M.bar, zero_init ? 2 * bytes : 3 * bytes);
       tma_field(M.r, m + 2, k0, j0, M.bar);
       tma_field(M.d, m + 3, k0, j0, M.bar);

@@ -206,3 +206,63 @@ def test_batch_tiles_by_tma_match_the_tile_per_block_form_bit_for_bit(shape):
         B.close()
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+def test_batch_maps_follow_shapes_and_buffers_bit_for_bit():
+    """The persistent sweep kernels read each case's tensor maps from a table
+    that is rewritten in place: for every shape, and when a case's two
+    correction buffers have changed places (a solve of its own with an odd
+    number of launches).  One batch is tuned over all shapes and then goes
+    through them, with such solves in between, on the states a batch fixed to
+    shape 33 (form 10, no maps) goes through.  All five have 16 half-sweeps a
+    launch, so the fields are equal bit for bit; shape 42 (24 half-sweeps) is
+    compared with a batch that has used no other."""
+    import torch
+    from paper_2402_17337_gb300 import Batch, build
+    build.build()
+    cfgs = W.batch_small(3) + W.batch64()[:3]
+    cfgs[1].nx, cfgs[1].ny = 133, 67
+
+    def fields(ss):
+        return [s.get(f) for s in ss for f in ("u", "v", "p")]
+
+    def solve_alone(s):
+        """One launch of sweeps: the case's two correction buffers change places."""
+        s.set_sor_shape(33)
+        b = torch.tensor(W.random_field((s.P.ny, s.P.nx), seed=1), device="cuda")
+        x = torch.zeros_like(b)
+        torch.cuda.synchronize()
+        rc, sweeps, _ = s.poisson_solve(b.data_ptr(), x.data_ptr(), 1e-300, 8, 8)
+        assert (rc, sweeps) == (-3, 8)
+
+    def go(shapes, tuned):
+        ss = solvers(cfgs)
+        B = Batch(ss)
+        if tuned:
+            keep = [s.save_state() for s in ss]
+            B.step(1)
+            for s, k in zip(ss, keep):
+                s.load_state(k)
+        out = []
+        for n, k in enumerate(shapes):
+            B.set_sor_shape(k)
+            B.set_budgets(n % 2 == 0)
+            B.step(1)
+            out.append(fields(ss))
+            for s in ss[n % 2::2]:
+                solve_alone(s)
+        B.set_sor_shape(42)
+        if not tuned:  # a batch that has used no other shape of form 11
+            B.close()
+            B = Batch(ss)
+            B.set_sor_shape(42)
+        B.set_budgets(True)
+        B.step(1)
+        out.append(fields(ss))
+        B.close()
+        return out
+
+    shapes = (37, 41, 38, 40, 39, 41)
+    for a, b in zip(go(len(shapes) * (33,), False), go(shapes, True)):
+        for x, y in zip(a, b):
+            assert np.array_equal(x, y)
