@@ -160,6 +160,7 @@ struct ibm_ctx {
   Sor64Plan sor64;
   Sor64Tiles sor64_tiles{};
   size_t sor64_bytes = 0;  // of its norms and words
+  unsigned sor64_used = 0;  // exchange numbers used on them
   Sor64Result *sor64_res = nullptr, *sor64_host = nullptr;  // device; pinned, behind sc_host
   // history
   double *cl_d = nullptr, *cd_d = nullptr;
@@ -788,20 +789,15 @@ int read_norm(ibm_ctx* c, const unsigned long long* dev_bits, double* out) {
 }
 
 // The sweeps and checks of solve_poisson on the device (k_sor64.cu); the host
-// waits once per launch of up to kChunk64 sweeps.
-constexpr int kChunk64 = 8192;  // two exchanges or checks a sweep at most: well below kSor64Numbers
+// waits once per launch of up to kSor64Chunk sweeps.
 int solve_poisson_chip(ibm_ctx* c, double thr, int m, int maxs, int* sweeps, double* res) {
   const Geo& g = c->geo;
-  for (int done = 0;;) {
-    // exchange numbers are used once; when they run out the buffers are cleared
-    if (c->sor64.kind == Sor64Plan::TILES && c->sor64_tiles.first > UINT_MAX - 2 * kSor64Numbers) {
-      CUDA_TRY(cudaMemsetAsync(c->sor64_tiles.norms, 0, c->sor64_bytes, c->stream));
-      c->sor64_tiles.first = 0;
-    }
-    const Sor64Tiles t = c->sor64_tiles;
-    c->sor64_tiles.first += kSor64Numbers;
+  for (Sor64Progress run{m, maxs, kSor64Chunk};;) {
+    Sor64Tiles t = c->sor64_tiles;
+    if (sor64_reserve(&c->sor64_used, &t.first) && c->sor64.kind == Sor64Plan::TILES)
+      CUDA_TRY(cudaMemsetAsync(t.norms, 0, c->sor64_bytes, c->stream));
     const Sor64Args a{g.nx, g.ny, g.pitch, at(0, 0, g.pitch), g.pE, g.pW, g.pN, g.pS, c->phi, c->b, c->invd_p,
-                      c->P.omega_p, thr, m, maxs - done, kChunk64};
+                      c->P.omega_p, thr, run.span()};
     if (c->profiling) CUDA_TRY(cudaEventRecord(c->ev0, c->stream));
     CUDA_TRY(launch_sor64(c->stream, c->sor64, a, t, c->sor64_res));
     if (c->profiling) CUDA_TRY(cudaEventRecord(c->ev1, c->stream));
@@ -817,15 +813,17 @@ int solve_poisson_chip(ibm_ctx* c, double thr, int m, int maxs, int* sweeps, dou
       c->prof.sweep_cells += (long long)c->nx * c->ny;
     }
     if (r.late) return fail(IBM_E_TIMEOUT, "pressure solve: a block waited too long for its neighbours");
-    *sweeps = done + r.checked;
-    *res = bits_to_double(r.bits);
-    done += r.sweeps;
+    if (r.checked >= 0) {
+      *sweeps = (int)run.done + r.checked;
+      *res = bits_to_double(r.bits);
+    }
+    run.advance(r.sweeps, r.checked);
     switch (r.status) {
       case SOR64_OK: return IBM_OK;
       case SOR64_DIVERGED:
         return fail(IBM_E_DIVERGED, "pressure residual is not finite after %d sweeps", *sweeps);
       case SOR64_NOCONV:
-        return fail(IBM_E_NOCONV, "pressure solve: %d sweeps, residual %.3e > %.3e", done, *res, thr);
+        return fail(IBM_E_NOCONV, "pressure solve: %d sweeps, residual %.3e > %.3e", (int)run.done, *res, thr);
       default: break;
     }
   }

@@ -6,6 +6,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "sor64_loop.h"
+
 namespace ibm {
 
 // Named NVTX range over a scope (host side: it spans the enqueueing of the
@@ -119,8 +121,8 @@ void launch_poisson_res(cudaStream_t s, const Geo& g, const double* phi, const d
 void launch_poisson_res2(cudaStream_t s, const Geo& g, const double* phi_a, const double* phi_b, const double* b,
                          unsigned long long* bits_a, unsigned long long* bits_b);
 // FP64 SOR with the grid kept on chip and the residual checks on the device
-// (k_sor64.cu): one launch runs until the tolerance is met, maxs sweeps are
-// done or chunk sweeps have passed.  Element (i, j) of phi, b and invd lies at
+// (k_sor64.cu): one launch runs until the tolerance is met, the solve's sweeps
+// are done or its own have passed (span).  Element (i, j) of phi, b and invd lies at
 // off + j pitch + i; invd may be null for the cluster kernel (recomputed).
 struct Sor64Args {
   int nx, ny, pitch;
@@ -129,24 +131,21 @@ struct Sor64Args {
   double* phi;
   const double *b, *invd;
   double omega, thr;
-  int m, maxs, chunk;  // check every m sweeps
+  Sor64Span span;
 };
 struct Sor64Tiles {
   int nbx, nby, K;
   unsigned long long* words;   // 2 buffers of 2 words per cell
   size_t stride;               // words of one buffer
   unsigned long long* norms;   // 4 words per tile
-  unsigned first;              // exchanges are numbered from first + 1; no number is used twice on the buffers
+  unsigned first;              // exchanges and checks are numbered from first + 1 (sor64_reserve)
 };
 // the most cells and tiles of a plan of tiles
 constexpr long kSor64TilesCells = 300000;
 constexpr int kSor64MaxTiles = 1024;
-// exchange numbers one launch may use
-constexpr unsigned kSor64Numbers = 1u << 16;
-enum { SOR64_MORE = 0, SOR64_OK, SOR64_NOCONV, SOR64_DIVERGED };
 struct Sor64Result {
   unsigned long long bits;  // norm of the last check
-  int checked, sweeps;      // sweeps at the last check, sweeps done
+  int checked, sweeps;      // sweeps at the last check (-1: the launch made none), sweeps done
   int status, late;         // late: a CTA gave up a wait
 };
 struct Sor64Plan {

@@ -211,14 +211,13 @@ extern "C" int ibm_poisson_solve_noalloc(int nx, int ny, const double* xf, const
     tiles.words = tiles.norms + 4 * ibm::sor64_max_tiles();
     tiles.stride = 2 * (size_t)nx * ny;
     const size_t tile_bytes = 32 * ((size_t)ibm::sor64_max_tiles() + (size_t)nx * ny);
-    for (int done = 0;;) {
-      // exchange numbers are used once: the buffers are cleared at the start and when they run out
-      if (plan.kind == ibm::Sor64Plan::TILES && (done == 0 || tiles.first > UINT_MAX - 2 * ibm::kSor64Numbers)) {
+    unsigned used = UINT_MAX;  // numbers left on the scratch by another call: cleared at the start, and when they run out
+    for (ibm::Sor64Progress run{m, maxs, ibm::kSor64Chunk};;) {
+      if (ibm::sor64_reserve(&used, &tiles.first) && plan.kind == ibm::Sor64Plan::TILES) {
         const cudaError_t e = cudaMemsetAsync(tiles.norms, 0, tile_bytes, s);
         if (e != cudaSuccess) return cuda_fail("cudaMemsetAsync of the exchange buffers", e);
-        tiles.first = 0;
       }
-      const ibm::Sor64Args a{nx, ny, nx, 0, g.pE, g.pW, g.pN, g.pS, phi_dev, b_dev, nullptr, omega, tol, m, maxs - done, 8192};
+      const ibm::Sor64Args a{nx, ny, nx, 0, g.pE, g.pW, g.pN, g.pS, phi_dev, b_dev, nullptr, omega, tol, run.span()};
       ibm::Sor64Result r{};
       cudaError_t e = ibm::launch_sor64(s, plan, a, tiles, out);
       if (e != cudaSuccess) return cuda_fail("the launch of the sweeps", e);
@@ -226,16 +225,17 @@ extern "C" int ibm_poisson_solve_noalloc(int nx, int ny, const double* xf, const
       if (e != cudaSuccess) return cuda_fail("cudaMemcpyAsync of the result", e);
       e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return cuda_fail("the sweeps (cudaStreamSynchronize)", e);
-      tiles.first += ibm::kSor64Numbers;
       if (r.late) {
         ibm::set_last_error("ibm_poisson_solve_noalloc: a block waited too long for its neighbours");
         return IBM_E_TIMEOUT;
       }
-      double v;
-      std::memcpy(&v, &r.bits, sizeof v);
-      if (sweeps) *sweeps = done + r.checked;
-      if (res) *res = v;
-      done += r.sweeps;
+      if (r.checked >= 0) {
+        double v;
+        std::memcpy(&v, &r.bits, sizeof v);
+        if (sweeps) *sweeps = (int)run.done + r.checked;
+        if (res) *res = v;
+      }
+      run.advance(r.sweeps, r.checked);
       if (r.status == ibm::SOR64_DIVERGED) {
         ibm::set_last_error("ibm_poisson_solve_noalloc: residual is not finite");
         return IBM_E_DIVERGED;

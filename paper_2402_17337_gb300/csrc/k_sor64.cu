@@ -1,7 +1,8 @@
 // FP64 red-black SOR of the pressure equation with the grid kept on chip for
 // many sweeps (arXiv 2402.17337 Sec. 2.2, Sec. 3.1), including the residual
 // checks: one launch runs up to a few thousand sweeps and leaves when the
-// tolerance is met, so the host is asked once per launch, not once per check.
+// tolerance is met, so the host is asked once per launch, not once per check
+// (sor64_loop.h: when a launch checks and when it ends).
 //
 // The iterates are those of k_poisson_half / k_poisson_res (k_sor.cu): the
 // same fma chains in the same order, the same reciprocal diagonal, the norm
@@ -60,28 +61,10 @@ __device__ __forceinline__ double res64(double aE, double aW, double aN, double 
   return b - L;
 }
 
-// State of the sweep loop; every thread of the launch holds the same one, so
-// all leave together.  Follows the host loop of solve_poisson: a check before
-// the first sweep and every m sweeps, at most maxs sweeps.
-struct Loop {
-  int s, next;     // sweeps done, sweep count of the next check
-  int last, status;
-  unsigned long long bits;
-};
-
 // after a check with norm `bits`: true if the solve ends
-__device__ __forceinline__ bool check_done(Loop& L, unsigned long long bits, double thr, int m, int maxs) {
+__device__ __forceinline__ bool check_done(Sor64Loop& L, unsigned long long bits, const Sor64Args& A) {
   const double r = __longlong_as_double((long long)bits);
-  L.last = L.s;
-  L.bits = bits;
-  L.next = L.s + m;
-  if (!isfinite(r))
-    L.status = SOR64_DIVERGED;
-  else if (r <= thr)
-    L.status = SOR64_OK;
-  else if (L.s >= maxs)
-    L.status = SOR64_NOCONV;
-  return L.status != SOR64_MORE;
+  return L.checked(A.span, bits, isfinite(r), r <= A.thr);
 }
 
 // ------------------------------------------------------------ one cluster
@@ -175,9 +158,9 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_sor64_cluster(Sor64Args A, So
       if (in && r == rows - 1 && rank < nrank - 1) push[c][k][1] = map_rank(smem_addr(ph + i + 1), rank + 1);
     }
   cluster_sync();
-  Loop L{0, 0, 0, SOR64_MORE, 0ull};
+  Sor64Loop L(A.span);
   for (;;) {
-    if (L.s == L.next) {
+    if (L.check_due()) {
       unsigned long long v = 0ull;
 #pragma unroll
       for (int c = 0; c < 2; ++c)
@@ -198,14 +181,10 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_sor64_cluster(Sor64Args A, So
       }
       cluster_sync();
       v = warp_max(lane < nrank ? norms[lane] : 0ull);
-      if (check_done(L, v, A.thr, A.m, A.maxs)) break;
+      if (check_done(L, v, A)) break;
       // the next write to norms comes after another cluster barrier (the next half-sweep's)
     }
-    if (L.s >= A.maxs) {
-      L.status = SOR64_NOCONV;
-      break;
-    }
-    if (L.s >= A.chunk && L.s == L.last) break;  // hand back to the host, at a check
+    if (L.stop(A.span)) break;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
 #pragma unroll
@@ -393,10 +372,10 @@ __global__ void __launch_bounds__(TL_THREADS, 1) k_sor64_tiles(Sor64Args A, Sor6
     }
     __syncthreads();
   };
-  Loop L{0, 0, 0, SOR64_MORE, 0ull};
+  Sor64Loop L(A.span);
   int fresh = K;  // half-sweeps the halo is still good for (just loaded: all K)
   for (;;) {
-    if (L.s == L.next) {
+    if (L.check_due()) {
       if (fresh < 1) {
         if (!exchange()) { dead = true; break; }
         fresh = K;
@@ -436,13 +415,9 @@ __global__ void __launch_bounds__(TL_THREADS, 1) k_sor64_tiles(Sor64Args A, Sor6
       if (__syncthreads_or(late)) { dead = true; break; }
       v = warp_max(lane < TL_THREADS / 32 ? wmax[lane] : 0ull);
       __syncthreads();  // wmax is written again by the next check
-      if (check_done(L, v, A.thr, A.m, A.maxs)) break;
+      if (check_done(L, v, A)) break;
     }
-    if (L.s >= A.maxs) {
-      L.status = SOR64_NOCONV;
-      break;
-    }
-    if (L.s >= A.chunk && L.s == L.last) break;
+    if (L.stop(A.span)) break;
     if (fresh < 2) {
       if (!exchange()) { dead = true; break; }
       fresh = K;

@@ -92,3 +92,49 @@ def test_allocation_free_solve_repeats_the_context_bit_for_bit(nx, ny, m, cap):
                   m, cap, None, C.byref(sn), C.byref(rn)) == rc == -3
         assert sn.value == sg and rn.value == rg
         assert torch.equal(p, q)
+
+
+@pytest.mark.parametrize("nx,ny", [(70, 45), (513, 257)])
+@pytest.mark.parametrize("m,cap", [(3000, 20000), (65537, 131084)])
+def test_launches_between_checks_do_not_change_the_iterates(nx, ny, m, cap):
+    """A solve takes several launches whatever the interval between checks (here
+    longer than a launch, and no multiple of one): the same iterates bit for
+    bit as with a check every 8 sweeps, by the context and by the
+    allocation-free call.  The relaxation factor is small, so the iterates
+    still change at the end."""
+    import ctypes as C
+
+    import torch
+    import paper_2402_17337_gb300 as ibm
+    from paper_2402_17337_gb300 import build
+    build.build()
+    g = ibm.Solver(x0=0.0, x1=2.0 + nx / ny, y0=0.0, y1=1.5, nx=nx, ny=ny, hmin=0.0, dt=1.0, omega_p=0.05)
+    xf, yf = g.grid()
+    fn, D = ibm.lib().ibm_poisson_solve_noalloc, C.POINTER(C.c_double)
+    fn.argtypes = [C.c_int, C.c_int, D, D, C.c_void_p, C.c_void_p, C.c_double, C.c_double, C.c_int, C.c_int,
+                   C.c_void_p, C.POINTER(C.c_int), C.POINTER(C.c_double)]
+    b = W.random_field((ny, nx), seed=1)
+    b -= b.mean()
+    bd = torch.tensor(b, device="cuda")
+    out = []
+    for every in (8, m):
+        p = torch.zeros_like(bd)
+        torch.cuda.synchronize()
+        g.set_profiling(True)
+        rc, sweeps, res = g.poisson_solve(bd.data_ptr(), p.data_ptr(), 1e-300, every, cap)
+        assert (rc, sweeps) == (-3, cap // every * every)
+        assert g.profile()["sweep_launches"] >= cap // 8192
+        q = torch.zeros_like(bd)
+        torch.cuda.synchronize()
+        sn, rn = C.c_int(-1), C.c_double(-1.0)
+        assert fn(nx, ny, xf.ctypes.data_as(D), yf.ctypes.data_as(D), bd.data_ptr(), q.data_ptr(), g.P.omega_p, 1e-300,
+                  every, cap, None, C.byref(sn), C.byref(rn)) == rc
+        assert (sn.value, rn.value) == (sweeps, res)
+        assert torch.equal(p, q)
+        out.append(p)
+    assert torch.equal(*out)
+    p = torch.zeros_like(bd)
+    torch.cuda.synchronize()
+    g.poisson_solve(bd.data_ptr(), p.data_ptr(), 1e-300, 8, cap - 8)
+    assert not torch.equal(p, out[0])
+    g.close()
