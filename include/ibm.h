@@ -216,7 +216,8 @@ int ibm_poisson_solve_noalloc(int nx, int ny, const double* xf, const double* yf
  * launches between two residual checks is bracketed by CUDA events on the
  * context's stream; sweep_ms is the summed device time of those runs and
  * sweep_launches the number of launches they contain (on FP64 grids up to
- * 300 000 cells one launch runs a whole solve with its residual checks). */
+ * 300 000 cells a launch runs up to 512 sweeps, on the smallest 8192, with
+ * their residual checks). */
 typedef struct {
   long long launches;        /* kernels launched by this context */
   long long sweep_launches;  /* pressure SOR sweep launches inside timed runs */

@@ -789,10 +789,10 @@ int read_norm(ibm_ctx* c, const unsigned long long* dev_bits, double* out) {
 }
 
 // The sweeps and checks of solve_poisson on the device (k_sor64.cu); the host
-// waits once per launch of up to kSor64Chunk sweeps.
+// waits once per launch of up to sor64.chunk() sweeps.
 int solve_poisson_chip(ibm_ctx* c, double thr, int m, int maxs, int* sweeps, double* res) {
   const Geo& g = c->geo;
-  for (Sor64Progress run{m, maxs, kSor64Chunk};;) {
+  for (Sor64Progress run{m, maxs, c->sor64.chunk()};;) {
     Sor64Tiles t = c->sor64_tiles;
     if (sor64_reserve(&c->sor64_used, &t.first) && c->sor64.kind == Sor64Plan::TILES)
       CUDA_TRY(cudaMemsetAsync(t.norms, 0, c->sor64_bytes, c->stream));

@@ -152,6 +152,7 @@ struct Sor64Plan {
   enum Kind { NONE, CLUSTER, TILES } kind = NONE;
   int nbx = 0, nby = 0, K = 0;
   size_t smem = 0;
+  int chunk() const { return kind == TILES ? kSor64TilesChunk : kSor64Chunk; }  // most sweeps of a launch
 };
 Sor64Plan sor64_plan(int nx, int ny);
 int sor64_max_tiles();

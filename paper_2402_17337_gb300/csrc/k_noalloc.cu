@@ -212,7 +212,7 @@ extern "C" int ibm_poisson_solve_noalloc(int nx, int ny, const double* xf, const
     tiles.stride = 2 * (size_t)nx * ny;
     const size_t tile_bytes = 32 * ((size_t)ibm::sor64_max_tiles() + (size_t)nx * ny);
     unsigned used = UINT_MAX;  // numbers left on the scratch by another call: cleared at the start, and when they run out
-    for (ibm::Sor64Progress run{m, maxs, ibm::kSor64Chunk};;) {
+    for (ibm::Sor64Progress run{m, maxs, plan.chunk()};;) {
       if (ibm::sor64_reserve(&used, &tiles.first) && plan.kind == ibm::Sor64Plan::TILES) {
         const cudaError_t e = cudaMemsetAsync(tiles.norms, 0, tile_bytes, s);
         if (e != cudaSuccess) return cuda_fail("cudaMemsetAsync of the exchange buffers", e);

@@ -14,8 +14,15 @@ namespace ibm {
 
 enum { SOR64_MORE = 0, SOR64_OK, SOR64_NOCONV, SOR64_DIVERGED };
 
-// The most sweeps of one launch, whatever the interval between checks.
-constexpr int kSor64Chunk = 8192;
+// The most sweeps of one launch, whatever the interval between checks.  Tiles
+// hold most of every SM's registers while they run, so a kernel of another
+// stream that does not fit beside them waits for the end of their launch.  For
+// 8000 sweeps of 384x192 / 512x256 / 700x350, a 2048x2048 matrix product beside
+// them waits 28 / 43 / 64 ms with 8192 sweeps a launch, 3.3 / 5.2 / 7.8 ms with
+// 1024 and 1.5 / 2.4 / 3.8 ms with 512; the solves take 28.7 / 43.3 / 64.1 ms,
+// 28.8 / 43.4 / 64.2 and 29.0 / 43.6 / 64.4 (with 256: 2 % more).  A cluster
+// leaves 136 of 152 SMs free.
+constexpr int kSor64Chunk = 8192, kSor64TilesChunk = 512;
 // Exchange numbers a launch reserves: it sees the sweep counts 0 .. chunk, and
 // at each of them makes at most one exchange and one check.
 constexpr unsigned kSor64Numbers = 2u * (kSor64Chunk + 1);

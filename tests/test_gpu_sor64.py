@@ -138,3 +138,22 @@ def test_launches_between_checks_do_not_change_the_iterates(nx, ny, m, cap):
     g.poisson_solve(bd.data_ptr(), p.data_ptr(), 1e-300, 8, cap - 8)
     assert not torch.equal(p, out[0])
     g.close()
+
+
+@pytest.mark.parametrize("nx,ny,cap,launches", [(192, 96, 4096, 8), (192, 96, 4100, 9), (513, 257, 1500, 3),
+                                                (70, 45, 4096, 1)])
+def test_a_solve_on_every_SM_is_cut_into_short_launches(nx, ny, cap, launches):
+    """Tiles hold every SM, so a launch of theirs ends after 512 sweeps and lets
+    other streams' kernels in; a cluster leaves SMs free and goes on."""
+    import torch
+    from paper_2402_17337_gb300 import Solver, build
+    build.build()
+    g = Solver(x0=0.0, x1=2.0 + nx / ny, y0=0.0, y1=1.5, nx=nx, ny=ny, hmin=0.0, dt=1.0)
+    bd = torch.tensor(W.random_field((ny, nx), seed=1), device="cuda")
+    p = torch.zeros_like(bd)
+    torch.cuda.synchronize()
+    g.set_profiling(True)
+    rc, sweeps, _ = g.poisson_solve(bd.data_ptr(), p.data_ptr(), 1e-300, 8, cap)
+    assert (rc, sweeps) == (-3, cap // 8 * 8)
+    assert g.profile()["sweep_launches"] == launches
+    g.close()

@@ -79,7 +79,7 @@ int main() {
   const int maxs[] = {0, 1, 2, 7, 8, 60, 1024, 1025, 8192, 8193, 20000, 140000};
   for (int m : ms)
     for (int mx : maxs)
-      for (int chunk : {1, 5, 64, kSor64Chunk})
+      for (int chunk : {1, 5, kSor64TilesChunk, kSor64Chunk})
         for (int K = 2; K <= 8; K += 2)
           for (int conv : {-1, 0, 1, 3})
             if (chunk > 5 || mx <= 8192) solve(m, mx, chunk, K, conv);
