@@ -248,6 +248,14 @@ int ibm_tune(ibm_ctx* ctx);
 int ibm_sor_num_shapes(void);
 int ibm_set_sor_shape(ibm_ctx* ctx, int index);
 
+/* Limit of each device-side wait inside this context's pressure sweeps, in
+ * seconds at an SM clock of 2 GHz: the FP64 tiles' waits for their neighbours
+ * (default 1 s) and the FP32 sweeps' for a tile's copies (default 2 s; a batch
+ * takes the shortest of its cases).  A wait that runs out ends the solve with
+ * IBM_E_TIMEOUT; the pressure increment is then unspecified.  0: a wait that
+ * finds nothing ready runs out at once; < 0: the defaults again. */
+int ibm_set_wait_limit(ibm_ctx* ctx, double seconds);
+
 /* Relaxation factor of the pressure SOR (Sec. 2.2 leaves it free) from the
  * observed convergence: red-black SOR runs on the homogeneous pressure
  * system from a pseudo-random start until the residual has fallen by 1e-10

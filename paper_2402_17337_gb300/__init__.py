@@ -108,6 +108,7 @@ def lib():
             L.ibm_tune_omega.argtypes = [_VP, C.c_int, _D]
             L.ibm_set_sor_shape.argtypes = [_VP, C.c_int]
             L.ibm_sor_num_shapes.argtypes = []
+            L.ibm_set_wait_limit.argtypes = [_VP, C.c_double]
             L.ibm_omega_from_rate.argtypes = [C.c_double, C.c_double]
             L.ibm_omega_from_rate.restype = C.c_double
             L.ibm_batch_create.argtypes = [C.POINTER(_VP), C.c_int, C.POINTER(_VP)]
@@ -268,6 +269,10 @@ class Solver:
     def set_sor_shape(self, index):
         """Fixes the FP32 sweep tile shape (index into the library's table; -1: autotune)."""
         _check(lib().ibm_set_sor_shape(self._h, index))
+
+    def set_wait_limit(self, seconds):
+        """Limit of the device-side waits inside the pressure sweeps (0: run out at once; < 0: the defaults)."""
+        _check(lib().ibm_set_wait_limit(self._h, seconds))
 
     def tune_omega(self, sweeps=0):
         """Sets the pressure SOR relaxation factor from the observed convergence; returns it."""

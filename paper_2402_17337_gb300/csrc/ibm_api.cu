@@ -9,6 +9,7 @@
 #include <cstring>
 #include <map>
 #include <string>
+#include <tuple>
 #include <utility>
 #include <vector>
 
@@ -162,6 +163,7 @@ struct ibm_ctx {
   size_t sor64_bytes = 0;  // of its norms and words
   unsigned sor64_used = 0;  // exchange numbers used on them
   Sor64Result *sor64_res = nullptr, *sor64_host = nullptr;  // device; pinned, behind sc_host
+  long long wait = -1;  // limit of the sweep kernels' device-side waits, clocks (-1: each kernel's own)
   // history
   double *cl_d = nullptr, *cd_d = nullptr;
   int hist_cap = 0;
@@ -797,7 +799,7 @@ int solve_poisson_chip(ibm_ctx* c, double thr, int m, int maxs, int* sweeps, dou
     if (sor64_reserve(&c->sor64_used, &t.first) && c->sor64.kind == Sor64Plan::TILES)
       CUDA_TRY(cudaMemsetAsync(t.norms, 0, c->sor64_bytes, c->stream));
     const Sor64Args a{g.nx, g.ny, g.pitch, at(0, 0, g.pitch), g.pE, g.pW, g.pN, g.pS, c->phi, c->b, c->invd_p,
-                      c->P.omega_p, thr, run.span()};
+                      c->P.omega_p, thr, run.span(), c->wait < 0 ? kSor64Wait : c->wait};
     if (c->profiling) CUDA_TRY(cudaEventRecord(c->ev0, c->stream));
     CUDA_TRY(launch_sor64(c->stream, c->sor64, a, t, c->sor64_res));
     if (c->profiling) CUDA_TRY(cudaEventRecord(c->ev1, c->stream));
@@ -886,6 +888,9 @@ int solve_poisson(ibm_ctx* c, double tol, double rtol, int m, int maxs, int* swe
 // alike.
 double sor32_tie_break(int cfg) { return sor32_half_sweeps(cfg) == 16 ? 1.0 : 1.05; }
 
+// limit of form 11's waits in this context
+long long sor32_wait(const ibm_ctx* c) { return c->wait < 0 ? kSor32Wait : c->wait; }
+
 // Autotuner of the FP32 sweep kernel: times every tile shape on this
 // context's grid and arrays (CUDA events, a few launches each) and keeps the
 // fastest per full sweep.  Runs before the first mixed solve; the arrays'
@@ -896,17 +901,18 @@ int tune_sor32(ibm_ctx* c) {
   CUDA_TRY(cudaEventCreate(&a));
   CUDA_TRY(cudaEventCreate(&b));
   const float omega = (float)c->P.omega_p;
+  const long long wait = sor32_wait(c);
   double best = 1e300;
   int best_cfg = 0;
   for (int cfg = 0; cfg < sor32_num_configs(); ++cfg) {
     const int reps = 8;
     for (int w = 0; w < 2; ++w) {
-      launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, 1, 1);
+      launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, 1, 1, wait);
       std::swap(c->e32, c->e32b);
     }
     CUDA_TRY(cudaEventRecord(a, c->stream));
     for (int l = 0; l < reps; ++l) {
-      launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, l == 0 ? 1 : 0, 1);
+      launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, l == 0 ? 1 : 0, 1, wait);
       std::swap(c->e32, c->e32b);
     }
     CUDA_TRY(cudaEventRecord(b, c->stream));
@@ -1024,6 +1030,7 @@ int solve_poisson_mixed(ibm_ctx* c, double tol, int maxs, int* sweeps, double* r
   double prev = 0.0;
   int pending = 0;
   const float omega = (float)c->P.omega_p;
+  const long long wait = sor32_wait(c);
   for (;;) {
     if (pending) CUDA_TRY(cudaEventRecord(c->ev1, c->stream));
     CUDA_TRY(cudaMemsetAsync(&c->sc->res_bits, 0, 8, c->stream));
@@ -1061,7 +1068,7 @@ int solve_poisson_mixed(ibm_ctx* c, double tol, int maxs, int* sweeps, double* r
     if (c->profiling) CUDA_TRY(cudaEventRecord(c->ev0, c->stream));
     for (int l = 0; l < inner / K2; ++l) {
       // read e32, write e32b, swap: the final correction ends in e32
-      launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, l == 0 ? 1 : 0, 1);
+      launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, l == 0 ? 1 : 0, 1, wait);
       std::swap(c->e32, c->e32b);
       c->prof.launches += 1;
       if (c->profiling) pending += 1;
@@ -1349,7 +1356,7 @@ struct ibm_batch {
   struct Graphs {
     cudaGraphExec_t first = nullptr, pair = nullptr, many = nullptr;
   };
-  std::map<std::pair<int, int>, Graphs> graphs;
+  std::map<std::tuple<int, int, long long>, Graphs> graphs;  // by active cases, tiles, wait limit
   ibm_profile prof{};
 
   void drop_graphs() {
@@ -1421,10 +1428,18 @@ int batch_sor_tables(ibm_batch* B, int cfg, const std::vector<int>& act, int* ti
   return IBM_OK;
 }
 
+// limit of form 11's waits: the shortest of the cases'
+long long batch_wait(const ibm_batch* B) {
+  long long w = LLONG_MAX;
+  for (const ibm_ctx* c : B->cs) w = std::min(w, sor32_wait(c));
+  return w;
+}
+
 void batch_launch_pair(ibm_batch* B, int na, int tiles, int zero_first, int pdl) {
   const int n = (int)B->cs.size();
-  launch_sor32_batch(B->stream, B->cfg, B->d_sor, na, tiles, zero_first, pdl);
-  launch_sor32_batch(B->stream, B->cfg, B->d_sor + n, na, tiles, 0, pdl);
+  const long long wait = batch_wait(B);
+  launch_sor32_batch(B->stream, B->cfg, B->d_sor, na, tiles, zero_first, pdl, 0, wait);
+  launch_sor32_batch(B->stream, B->cfg, B->d_sor + n, na, tiles, 0, pdl, 0, wait);
 }
 
 int batch_capture(ibm_batch* B, int na, int tiles, int pairs, int zero_first, cudaGraphExec_t* out) {
@@ -1447,7 +1462,7 @@ int batch_sweeps(ibm_batch* B, int na, int tiles, int pairs) {
     CUDA_TRY(cudaGetLastError());
     return IBM_OK;
   }
-  auto key = std::make_pair(na, tiles);
+  auto key = std::make_tuple(na, tiles, batch_wait(B));
   auto it = B->graphs.find(key);
   if (it == B->graphs.end()) {
     if (B->graphs.size() >= 512) B->drop_graphs();
@@ -1615,9 +1630,10 @@ int batch_solve(ibm_batch* B, const std::vector<double>& thr, std::vector<ibm_st
     if (B->budgets) {
       // direct launches (programmatic dependents): the pair index varies per launch
       B->prof.launches += 2 * round_pairs;
+      const long long wait = batch_wait(B);
       for (int q = 0; q < round_pairs; ++q) {
-        launch_sor32_batch(B->stream, B->cfg, B->d_sor, (int)act.size(), tiles, q == 0, 1, q);
-        launch_sor32_batch(B->stream, B->cfg, B->d_sor + n, (int)act.size(), tiles, 0, 1, q);
+        launch_sor32_batch(B->stream, B->cfg, B->d_sor, (int)act.size(), tiles, q == 0, 1, q, wait);
+        launch_sor32_batch(B->stream, B->cfg, B->d_sor + n, (int)act.size(), tiles, 0, 1, q, wait);
       }
       CUDA_TRY(cudaGetLastError());
     } else {
@@ -2381,6 +2397,13 @@ int ibm_set_sor_shape(ibm_ctx* c, int index) {
   }
   c->sor_cfg = index;
   c->sor_us = 0.0;
+  return IBM_OK;
+}
+
+int ibm_set_wait_limit(ibm_ctx* c, double seconds) {
+  if (!c) return fail(IBM_E_INVAL, "null context");
+  if (!std::isfinite(seconds)) return fail(IBM_E_INVAL, "the wait limit must be finite");
+  c->wait = seconds < 0.0 ? -1 : (long long)std::fmin(seconds * 2e9, 1e15);
   return IBM_OK;
 }
 

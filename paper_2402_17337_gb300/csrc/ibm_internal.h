@@ -132,7 +132,9 @@ struct Sor64Args {
   const double *b, *invd;
   double omega, thr;
   Sor64Span span;
+  long long wait;  // limit of a CTA's wait for another, clocks
 };
+constexpr long long kSor64Wait = 2000000000ll;  // about 1 s at the SM clock
 struct Sor64Tiles {
   int nbx, nby, K;
   unsigned long long* words;   // 2 buffers of 2 words per cell
@@ -252,6 +254,7 @@ struct DcCase {
 };
 // true once a sweep kernel has given up a bounded wait for a tile's copies
 bool sor32_failed();
+constexpr long long kSor32Wait = 4000000000ll;  // its limit: about 2 s at the SM clock
 // form 11: a case's four tensor maps (Sor32Case::maps; host memory, then copied to the device, 64-byte aligned)
 size_t sor32_maps_bytes();
 bool sor32_case_maps(int cfg, const Geo32& g, const float* e, const float* eb, const float* r, const float* invd,
@@ -262,7 +265,7 @@ cudaError_t sor32_batch_prepare(int cfg);
 // stream (direct launches; the kernel waits for it before its first load)
 // q: index of the launch pair within the round (cases with pairs <= q skip it)
 void launch_sor32_batch(cudaStream_t s, int cfg, const Sor32Case* cases_dev, int ncases, int total_tiles,
-                        int zero_init, int pdl = 0, int q = 0);
+                        int zero_init, int pdl = 0, int q = 0, long long wait = kSor32Wait);
 void launch_dc_residual_batch(cudaStream_t s, const DcCase* cases_dev, int ncases, int total_blocks);
 
 // geometric multigrid on the FP32 correction equation (k_mg.cu)
@@ -335,8 +338,9 @@ void launch_dc_residual(cudaStream_t s, const Geo& g, int pk, const double* phi_
 // pdl: launch as a programmatic dependent of the previous kernel on the
 // stream (consecutive sweep launches outside graph capture).  With
 // zero_init = 0 the previous kernel must be a sweep launch of the same run:
-// forms 6 to 11 then read r and 1/d before waiting for it.
+// forms 6 to 11 then read r and 1/d before waiting for it.  wait: limit of
+// form 11's wait for a tile's copies, clocks (0: every wait gives up).
 void launch_sor32(cudaStream_t s, int cfg, const Geo32& g, const float* e_in, float* e_out, const float* r,
-                  const float* invd, float omega, int zero_init, int pdl = 0);
+                  const float* invd, float omega, int zero_init, int pdl = 0, long long wait = kSor32Wait);
 
 }  // namespace ibm

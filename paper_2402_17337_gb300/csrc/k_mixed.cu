@@ -818,13 +818,12 @@ struct Sor32ShapeV11 {
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
-constexpr long long kSorWaitCycles = 4000000000ll;  // about 2 s at the SM clock
-
 // waits for the phase with the given parity of an mbarrier; false (and *err
-// set) if it has not completed within kSorWaitCycles
-__device__ __forceinline__ bool sor_wait(unsigned bar, unsigned parity, unsigned* err) {
+// set) if it has not completed within limit clocks (0: gives up without a look)
+__device__ __forceinline__ bool sor_wait(unsigned bar, unsigned parity, unsigned* err, long long limit) {
   long long t0 = 0;
   for (;;) {
+    if (limit <= 0) break;
     unsigned ok;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
@@ -834,11 +833,10 @@ __device__ __forceinline__ bool sor_wait(unsigned bar, unsigned parity, unsigned
     if (ok) return true;
     const long long now = clock64();
     if (!t0) t0 = now;
-    if (now - t0 > kSorWaitCycles) {
-      atomicOr_system(err, 1u);
-      return false;
-    }
+    if (now - t0 > limit) break;
   }
+  atomicOr_system(err, 1u);
+  return false;
 }
 // one array of a tile: box {64 packed columns, LY rows, 2 colours} at (k0, j0, 0)
 __device__ __forceinline__ void tma_field(void* dst, const CUtensorMap* map, int k0, int j0, unsigned bar) {
@@ -894,7 +892,7 @@ __device__ __forceinline__ void setup_v11(const TileMem<S>& M, int NY) {
 template <int TY, int K, int NY, class Next>
 __device__ __forceinline__ bool sor32_tile_v11(const Geo32& g, float* __restrict__ e_out, float omega, float omc,
                                                int zero_init, int k0, int j0, const TileMem<Sor32ShapeV11<TY, K, NY>>& M,
-                                               unsigned parity, unsigned* err, Next next) {
+                                               unsigned parity, unsigned* err, long long wait, Next next) {
   using S = Sor32ShapeV11<TY, K, NY>;
   constexpr int HK = S::HK, TK = S::TK, LY = S::LY, RPT = S::RPT;
   constexpr unsigned FULL = 0xffffffffu;
@@ -919,7 +917,7 @@ __device__ __forceinline__ bool sor32_tile_v11(const Geo32& g, float* __restrict
     cN[q] = rowok ? g.pN[j] : 0.f;
     cS[q] = rowok ? g.pS[j] : 0.f;
   }
-  const bool late = !sor_wait(M.bar, parity, err);
+  const bool late = !sor_wait(M.bar, parity, err, wait);
   if (__syncthreads_or(late)) return false;  // and every warp is past the edge rows of the tile before
 #pragma unroll
   for (int q = 0; q < RPT; ++q)
@@ -1094,7 +1092,7 @@ template <class C>
 __global__ void __launch_bounds__(32 * C::NY, C::MINB)
     k_sor32_tma(const __grid_constant__ CUtensorMap me, const __grid_constant__ CUtensorMap mr,
                 const __grid_constant__ CUtensorMap md, const Geo32 g, float* __restrict__ e_out, float omega,
-                float omc, int zero_init, int nbx, int ntiles, unsigned* __restrict__ err) {
+                float omc, int zero_init, int nbx, int ntiles, unsigned* __restrict__ err, long long wait) {
   using S = Sor32ShapeV11<C::TY, C::K, C::NY>;
   extern __shared__ __align__(1024) unsigned char smem_tile[];
   const TileMem<S> M(smem_tile);
@@ -1128,7 +1126,7 @@ __global__ void __launch_bounds__(32 * C::NY, C::MINB)
       fetch_rd(t);
       if (!zero_init) fetch_e(t);
     };
-    if (!sor32_tile_v11<C::TY, C::K, C::NY>(g, e_out, omega, omc, zero_init, k0, j0, M, n & 1u, err, next)) return;
+    if (!sor32_tile_v11<C::TY, C::K, C::NY>(g, e_out, omega, omc, zero_init, k0, j0, M, n & 1u, err, wait, next)) return;
   }
 }
 
@@ -1137,7 +1135,7 @@ __global__ void __launch_bounds__(32 * C::NY, C::MINB)
 template <class C>
 __global__ void __launch_bounds__(32 * C::NY, C::MINB)
     k_sor32_tma_batch(const Sor32Case* __restrict__ cases, int ncases, int ntiles, int zero_init, int q,
-                      unsigned* __restrict__ err) {
+                      unsigned* __restrict__ err, long long wait) {
   using S = Sor32ShapeV11<C::TY, C::K, C::NY>;
   extern __shared__ __align__(1024) unsigned char smem_tile[];
   __shared__ Sor32Case slot[2];  // descriptors of the current and the next tile's case
@@ -1186,7 +1184,7 @@ __global__ void __launch_bounds__(32 * C::NY, C::MINB)
     const int u = t - c.first, k0 = u % c.tiles_x * S::TK - S::HK, j0 = u / c.tiles_x * C::TY - C::K;
     auto next = [&] { request(t + gridDim.x, w ^ 1); };
     // next() runs before the tile's half-sweeps, whose barriers make slot[w ^ 1] visible
-    if (!sor32_tile_v11<C::TY, C::K, C::NY>(c.g, c.e_out, c.omega, 1.f - c.omega, zero_init, k0, j0, M, n & 1u, err, next)) return;
+    if (!sor32_tile_v11<C::TY, C::K, C::NY>(c.g, c.e_out, c.omega, 1.f - c.omega, zero_init, k0, j0, M, n & 1u, err, wait, next)) return;
   }
 }
 
@@ -1247,8 +1245,9 @@ int sm_count() {
 // [2.38] on 2048x1024; (88, 16, 12) 6.35 [10.5] on 4096x2048.
 struct Sor32Config {
   int TY, K, NY, V;
-  void (*launch)(cudaStream_t, const Geo32&, const float*, float*, const float*, const float*, float, int, int);
-  void (*launch_batch)(cudaStream_t, const Sor32Case*, int, int, int, int, int);
+  void (*launch)(cudaStream_t, const Geo32&, const float*, float*, const float*, const float*, float, int, int,
+                 long long);
+  void (*launch_batch)(cudaStream_t, const Sor32Case*, int, int, int, int, int, long long);
   cudaError_t (*prepare)();
   void (*tiles)(const Geo32&, int*, int*);
 };
@@ -1270,7 +1269,7 @@ cudaError_t prepare_shape() {
 
 template <class C>
 void launch_shape(cudaStream_t s, const Geo32& g, const float* e_in, float* e_out, const float* r, const float* invd,
-                  float omega, int zero_init, int pdl) {
+                  float omega, int zero_init, int pdl, long long wait) {
   static bool attr = false;
   if (!attr) {
     prepare_shape<C>();
@@ -1299,7 +1298,8 @@ void launch_shape(cudaStream_t s, const Geo32& g, const float* e_in, float* e_ou
       sor_no_maps();
       return;
     }
-    cudaLaunchKernelEx(&lc, k_sor32_tma<C>, me, mr, md, g, e_out, omega, 1.f - omega, zero_init, (int)grd.x, ntiles, err);
+    cudaLaunchKernelEx(&lc, k_sor32_tma<C>, me, mr, md, g, e_out, omega, 1.f - omega, zero_init, (int)grd.x, ntiles, err,
+                       wait);
   } else {
     cudaLaunchKernelEx(&lc, k_sor32_rb<C>, g, e_in, e_out, r, invd, omega, zero_init);
   }
@@ -1307,7 +1307,7 @@ void launch_shape(cudaStream_t s, const Geo32& g, const float* e_in, float* e_ou
 
 template <class C>
 void launch_shape_batch(cudaStream_t s, const Sor32Case* cases, int ncases, int total_tiles, int zero_init,
-                        int pdl, int q) {
+                        int pdl, int q, long long wait) {
   if (total_tiles <= 0) return;
   cudaLaunchConfig_t lc{};
   lc.gridDim = dim3(total_tiles);
@@ -1327,7 +1327,7 @@ void launch_shape_batch(cudaStream_t s, const Sor32Case* cases, int ncases, int 
       return;
     }
     lc.gridDim = dim3(std::min(total_tiles, sm_count() * C::MINB));
-    cudaLaunchKernelEx(&lc, k_sor32_tma_batch<C>, cases, ncases, total_tiles, zero_init, q, err);
+    cudaLaunchKernelEx(&lc, k_sor32_tma_batch<C>, cases, ncases, total_tiles, zero_init, q, err, wait);
   } else {
     cudaLaunchKernelEx(&lc, k_sor32_rb_batch<C>, cases, ncases, zero_init, q);
   }
@@ -1387,8 +1387,8 @@ void launch_dc_residual(cudaStream_t s, const Geo& g, int pk, const double* phi_
 }
 
 void launch_sor32(cudaStream_t s, int cfg, const Geo32& g, const float* e_in, float* e_out, const float* r,
-                  const float* invd, float omega, int zero_init, int pdl) {
-  kConfigs[cfg].launch(s, g, e_in, e_out, r, invd, omega, zero_init, pdl);
+                  const float* invd, float omega, int zero_init, int pdl, long long wait) {
+  kConfigs[cfg].launch(s, g, e_in, e_out, r, invd, omega, zero_init, pdl, wait);
 }
 
 void sor32_tiles(int cfg, const Geo32& g, int* tiles_x, int* tiles_y) { kConfigs[cfg].tiles(g, tiles_x, tiles_y); }
@@ -1396,8 +1396,8 @@ void sor32_tiles(int cfg, const Geo32& g, int* tiles_x, int* tiles_y) { kConfigs
 cudaError_t sor32_batch_prepare(int cfg) { return kConfigs[cfg].prepare(); }
 
 void launch_sor32_batch(cudaStream_t s, int cfg, const Sor32Case* cases_dev, int ncases, int total_tiles,
-                        int zero_init, int pdl, int q) {
-  kConfigs[cfg].launch_batch(s, cases_dev, ncases, total_tiles, zero_init, pdl, q);
+                        int zero_init, int pdl, int q, long long wait) {
+  kConfigs[cfg].launch_batch(s, cases_dev, ncases, total_tiles, zero_init, pdl, q, wait);
 }
 
 bool sor32_failed() {

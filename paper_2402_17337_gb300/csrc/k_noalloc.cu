@@ -217,7 +217,7 @@ extern "C" int ibm_poisson_solve_noalloc(int nx, int ny, const double* xf, const
         const cudaError_t e = cudaMemsetAsync(tiles.norms, 0, tile_bytes, s);
         if (e != cudaSuccess) return cuda_fail("cudaMemsetAsync of the exchange buffers", e);
       }
-      const ibm::Sor64Args a{nx, ny, nx, 0, g.pE, g.pW, g.pN, g.pS, phi_dev, b_dev, nullptr, omega, tol, run.span()};
+      const ibm::Sor64Args a{nx, ny, nx, 0, g.pE, g.pW, g.pN, g.pS, phi_dev, b_dev, nullptr, omega, tol, run.span(), ibm::kSor64Wait};
       ibm::Sor64Result r{};
       cudaError_t e = ibm::launch_sor64(s, plan, a, tiles, out);
       if (e != cudaSuccess) return cuda_fail("the launch of the sweeps", e);

@@ -214,8 +214,6 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_sor64_cluster(Sor64Args A, So
 constexpr int TL_THREADS = 640;
 constexpr int TL_CPT = 2;  // cells of one colour a thread owns at most
 
-constexpr long long kWaitCycles = 2000000000ll;  // about 1 s at the SM clock
-
 // A double with its exchange number: two 8-byte words {half, number}, each
 // written and read whole, so a reader that sees the number in both has the
 // value and needs no flag or fence (a fence here waits for every store of the
@@ -231,12 +229,12 @@ __device__ __forceinline__ bool peek(const unsigned long long* p, unsigned no, u
   v = (lo & 0xffffffffull) | (hi << 32);
   return (unsigned)(lo >> 32) == no && (unsigned)(hi >> 32) == no;
 }
-// waits for exchange number no at p; false after kWaitCycles
-__device__ __forceinline__ bool fetch(const unsigned long long* p, unsigned no, unsigned long long& v) {
+// waits for exchange number no at p; false after limit clocks (0: unless it is there already)
+__device__ __forceinline__ bool fetch(const unsigned long long* p, unsigned no, unsigned long long& v, long long limit) {
   if (peek(p, no, v)) return true;
   const long long t0 = clock64();
   while (!peek(p, no, v))
-    if (clock64() - t0 > kWaitCycles) return false;
+    if (clock64() - t0 >= limit) return false;
   return true;
 }
 
@@ -270,7 +268,7 @@ __device__ __forceinline__ void perimeter(int x, int y, int w, int h, int u, int
 // colour are listed tile first, then ring by ring outwards, so those of
 // half-sweep h are the first of the list; a thread keeps the coefficients, b
 // and the reciprocal diagonal of its TL_CPT entries in registers.  All CTAs
-// are resident at once (cooperative launch); a wait that lasts about a second
+// are resident at once (cooperative launch); a wait that lasts A.wait clocks
 // gives up and the launch reports it.
 __global__ void __launch_bounds__(TL_THREADS, 1) k_sor64_tiles(Sor64Args A, Sor64Tiles T, Sor64Result* __restrict__ out) {
   extern __shared__ __align__(16) double sm64[];
@@ -353,7 +351,7 @@ __global__ void __launch_bounds__(TL_THREADS, 1) k_sor64_tiles(Sor64Args A, Sor6
         perimeter(x0 - q, y0 - q, w + 2 * q, h + 2 * q, u, i, j);
         if (i < 0 || i >= nx || j < 0 || j >= ny) continue;
         unsigned long long v;
-        late = !fetch(buf + 2 * ((size_t)j * nx + i), no, v);
+        late = !fetch(buf + 2 * ((size_t)j * nx + i), no, v, A.wait);
         ph[(j - Y0) * P + i - X0] = __longlong_as_double((long long)v);
       }
       total += n;
@@ -406,7 +404,7 @@ __global__ void __launch_bounds__(TL_THREADS, 1) k_sor64_tiles(Sor64Args A, Sor6
       bool late = false;
       for (int t = tid; t < nb && !late; t += TL_THREADS) {
         unsigned long long b;
-        late = !fetch(slots + 2 * t, no, b);
+        late = !fetch(slots + 2 * t, no, b, A.wait);
         v = b > v ? b : v;
       }
       v = warp_max(v);

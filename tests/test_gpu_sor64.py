@@ -157,3 +157,31 @@ def test_a_solve_on_every_SM_is_cut_into_short_launches(nx, ny, cap, launches):
     assert (rc, sweeps) == (-3, cap // 8 * 8)
     assert g.profile()["sweep_launches"] == launches
     g.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(192, 96), (513, 257)])
+def test_a_wait_that_runs_out_ends_the_solve_and_leaves_the_context_usable(nx, ny):
+    """With a limit of 0 a tile gives up at the first neighbour that has not
+    posted yet: the kernel ends normally, the call reports IBM_E_TIMEOUT, and
+    with the default limit the same context solves as a new one does."""
+    import torch
+    from paper_2402_17337_gb300 import IBM_E_TIMEOUT, Solver, build
+    build.build()
+    kw = dict(x0=0.0, x1=2.0 + nx / ny, y0=0.0, y1=1.5, nx=nx, ny=ny, hmin=0.0, dt=1.0)
+    bd = torch.tensor(W.random_field((ny, nx), seed=1), device="cuda")
+
+    def solve(g):
+        p = torch.zeros_like(bd)
+        torch.cuda.synchronize()
+        return g.poisson_solve(bd.data_ptr(), p.data_ptr(), 1e-300, 8, 400), p
+
+    g, fresh = Solver(**kw), Solver(**kw)
+    want = solve(fresh)
+    for _ in range(3):
+        g.set_wait_limit(0.0)
+        assert solve(g)[0][0] == IBM_E_TIMEOUT
+        g.set_wait_limit(-1.0)
+        got = solve(g)
+        assert got[0] == want[0] and torch.equal(got[1], want[1])
+    g.close()
+    fresh.close()
