@@ -918,7 +918,11 @@ __device__ __forceinline__ bool sor32_tile_v11(const Geo32& g, float* __restrict
     cS[q] = rowok ? g.pS[j] : 0.f;
   }
   const bool late = !sor_wait(M.bar, parity, err, wait);
-  if (__syncthreads_or(late)) return false;  // and every warp is past the edge rows of the tile before
+  if (__syncthreads_or(late)) {  // and every warp is past the edge rows of the tile before
+    // the copies have landed, or a full wait for them has passed, before this shared memory may be another CTA's
+    sor_wait(M.bar, parity, err, kSor32Wait);
+    return false;
+  }
 #pragma unroll
   for (int q = 0; q < RPT; ++q)
 #pragma unroll
