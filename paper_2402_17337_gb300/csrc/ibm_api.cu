@@ -156,14 +156,21 @@ struct ibm_ctx {
   double *au = nullptr, *av = nullptr, *qband = nullptr, *rowsum = nullptr;
   double* partials = nullptr;
   DevScalars* sc = nullptr;
-  DevScalars* sc_host = nullptr;  // pinned mirror
+  // host memory that the device writes, in one block that starts at sc_host
+  struct Pinned {
+    DevScalars sc;
+    Sor64Result sor64;
+    unsigned sor_err;  // form 11 of the FP32 sweeps: a wait has given up
+  };
+  DevScalars* sc_host = nullptr;  // mirror of sc
   // FP64 sweeps kept on chip (precision 0)
   Sor64Plan sor64;
   Sor64Tiles sor64_tiles{};
   size_t sor64_bytes = 0;  // of its norms and words
   unsigned sor64_used = 0;  // exchange numbers used on them
-  Sor64Result *sor64_res = nullptr, *sor64_host = nullptr;  // device; pinned, behind sc_host
+  Sor64Result *sor64_res = nullptr, *sor64_host = nullptr;  // device; pinned
   long long wait = -1;  // limit of the sweep kernels' device-side waits, clocks (-1: each kernel's own)
+  unsigned* sor_err = nullptr;  // pinned
   // history
   double *cl_d = nullptr, *cd_d = nullptr;
   int hist_cap = 0;
@@ -780,12 +787,22 @@ int solve_poisson_mg(ibm_ctx* c, double tol, int maxc, int* cycles, double* res)
   }
 }
 
+// Whether a wait of the sweep launches that wrote to err gave up; reported
+// once (the stream has been waited for, and such a kernel ends normally, so the
+// solve that asks has failed and nothing else).
+bool sor32_gave_up(unsigned* err) {
+  volatile unsigned* e = err;
+  if (!*e) return false;
+  *e = 0u;
+  return true;
+}
+
 // Reads one norm accumulator back (waits for the stream).
 int read_norm(ibm_ctx* c, const unsigned long long* dev_bits, double* out) {
   CUDA_TRY(cudaMemcpyAsync(&c->sc_host->res_bits, dev_bits, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                            c->stream));
   CUDA_TRY(cudaStreamSynchronize(c->stream));
-  if (sor32_failed()) return fail(IBM_E_TIMEOUT, "a sweep kernel gave up a bounded wait");
+  if (sor32_gave_up(c->sor_err)) return fail(IBM_E_TIMEOUT, "a sweep kernel gave up a bounded wait");
   *out = bits_to_double(c->sc_host->res_bits);
   return IBM_OK;
 }
@@ -888,8 +905,8 @@ int solve_poisson(ibm_ctx* c, double tol, double rtol, int m, int maxs, int* swe
 // alike.
 double sor32_tie_break(int cfg) { return sor32_half_sweeps(cfg) == 16 ? 1.0 : 1.05; }
 
-// limit of form 11's waits in this context
-long long sor32_wait(const ibm_ctx* c) { return c->wait < 0 ? kSor32Wait : c->wait; }
+// form 11's waits in this context
+SorWait sor32_wait(const ibm_ctx* c) { return SorWait{c->sor_err, c->wait < 0 ? kSor32Wait : c->wait}; }
 
 // Autotuner of the FP32 sweep kernel: times every tile shape on this
 // context's grid and arrays (CUDA events, a few launches each) and keeps the
@@ -901,18 +918,18 @@ int tune_sor32(ibm_ctx* c) {
   CUDA_TRY(cudaEventCreate(&a));
   CUDA_TRY(cudaEventCreate(&b));
   const float omega = (float)c->P.omega_p;
-  const long long wait = sor32_wait(c);
+  const SorWait wait = sor32_wait(c);
   double best = 1e300;
   int best_cfg = 0;
   for (int cfg = 0; cfg < sor32_num_configs(); ++cfg) {
     const int reps = 8;
     for (int w = 0; w < 2; ++w) {
-      launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, 1, 1, wait);
+      CUDA_TRY(launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, 1, 1, wait));
       std::swap(c->e32, c->e32b);
     }
     CUDA_TRY(cudaEventRecord(a, c->stream));
     for (int l = 0; l < reps; ++l) {
-      launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, l == 0 ? 1 : 0, 1, wait);
+      CUDA_TRY(launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, l == 0, 1, wait));
       std::swap(c->e32, c->e32b);
     }
     CUDA_TRY(cudaEventRecord(b, c->stream));
@@ -1030,7 +1047,7 @@ int solve_poisson_mixed(ibm_ctx* c, double tol, int maxs, int* sweeps, double* r
   double prev = 0.0;
   int pending = 0;
   const float omega = (float)c->P.omega_p;
-  const long long wait = sor32_wait(c);
+  const SorWait wait = sor32_wait(c);
   for (;;) {
     if (pending) CUDA_TRY(cudaEventRecord(c->ev1, c->stream));
     CUDA_TRY(cudaMemsetAsync(&c->sc->res_bits, 0, 8, c->stream));
@@ -1068,7 +1085,7 @@ int solve_poisson_mixed(ibm_ctx* c, double tol, int maxs, int* sweeps, double* r
     if (c->profiling) CUDA_TRY(cudaEventRecord(c->ev0, c->stream));
     for (int l = 0; l < inner / K2; ++l) {
       // read e32, write e32b, swap: the final correction ends in e32
-      launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, l == 0 ? 1 : 0, 1, wait);
+      CUDA_TRY(launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, l == 0, 1, wait));
       std::swap(c->e32, c->e32b);
       c->prof.launches += 1;
       if (c->profiling) pending += 1;
@@ -1337,6 +1354,7 @@ struct ibm_batch {
   Sor32Case *h_sor = nullptr, *d_sor = nullptr;  // tables A (e32 -> e32b) at [0, n), B (e32b -> e32) at [n, 2n)
   DcCase *h_dc = nullptr, *d_dc = nullptr;
   unsigned long long *h_bits = nullptr, *d_bits = nullptr;
+  unsigned* h_err = nullptr;  // form 11: a wait has given up
   // tensor maps of every case's sweep arrays (sweep form 11) and what they were made for
   unsigned char *h_maps = nullptr, *d_maps = nullptr;
   std::vector<std::pair<int, const float*>> maps_of;
@@ -1375,7 +1393,7 @@ struct ibm_batch {
     if (d_sor) cudaFree(d_sor);
     if (d_dc) cudaFree(d_dc);
     if (d_bits) cudaFree(d_bits);
-    for (void* q : {(void*)h_maps, (void*)h_cases, (void*)h_first, (void*)h_hres, (void*)h_hswp, (void*)h_rb})
+    for (void* q : {(void*)h_err, (void*)h_maps, (void*)h_cases, (void*)h_first, (void*)h_hres, (void*)h_hswp, (void*)h_rb})
       if (q) cudaFreeHost(q);
     for (void* q : {(void*)d_maps, (void*)d_cases, (void*)d_first, (void*)d_hres, (void*)d_hswp, (void*)d_rb})
       if (q) cudaFree(q);
@@ -1428,16 +1446,16 @@ int batch_sor_tables(ibm_batch* B, int cfg, const std::vector<int>& act, int* ti
   return IBM_OK;
 }
 
-// limit of form 11's waits: the shortest of the cases'
-long long batch_wait(const ibm_batch* B) {
-  long long w = LLONG_MAX;
-  for (const ibm_ctx* c : B->cs) w = std::min(w, sor32_wait(c));
+// form 11's waits in this batch; their limit is the shortest of the cases'
+SorWait batch_wait(const ibm_batch* B) {
+  SorWait w{B->h_err, LLONG_MAX};
+  for (const ibm_ctx* c : B->cs) w.limit = std::min(w.limit, sor32_wait(c).limit);
   return w;
 }
 
 void batch_launch_pair(ibm_batch* B, int na, int tiles, int zero_first, int pdl) {
   const int n = (int)B->cs.size();
-  const long long wait = batch_wait(B);
+  const SorWait wait = batch_wait(B);
   launch_sor32_batch(B->stream, B->cfg, B->d_sor, na, tiles, zero_first, pdl, 0, wait);
   launch_sor32_batch(B->stream, B->cfg, B->d_sor + n, na, tiles, 0, pdl, 0, wait);
 }
@@ -1462,7 +1480,7 @@ int batch_sweeps(ibm_batch* B, int na, int tiles, int pairs) {
     CUDA_TRY(cudaGetLastError());
     return IBM_OK;
   }
-  auto key = std::make_tuple(na, tiles, batch_wait(B));
+  auto key = std::make_tuple(na, tiles, batch_wait(B).limit);
   auto it = B->graphs.find(key);
   if (it == B->graphs.end()) {
     if (B->graphs.size() >= 512) B->drop_graphs();
@@ -1567,7 +1585,7 @@ int batch_solve(ibm_batch* B, const std::vector<double>& thr, std::vector<ibm_st
                              B->stream));
     CUDA_TRY(cudaStreamSynchronize(B->stream));
     CUDA_TRY(cudaGetLastError());
-    if (sor32_failed()) return fail(IBM_E_TIMEOUT, "a sweep kernel gave up a bounded wait");
+    if (sor32_gave_up(B->h_err)) return fail(IBM_E_TIMEOUT, "a sweep kernel gave up a bounded wait");
     if (timing) {
       float ms = 0.f;
       CUDA_TRY(cudaEventElapsedTime(&ms, B->t0, B->t1));
@@ -1630,7 +1648,7 @@ int batch_solve(ibm_batch* B, const std::vector<double>& thr, std::vector<ibm_st
     if (B->budgets) {
       // direct launches (programmatic dependents): the pair index varies per launch
       B->prof.launches += 2 * round_pairs;
-      const long long wait = batch_wait(B);
+      const SorWait wait = batch_wait(B);
       for (int q = 0; q < round_pairs; ++q) {
         launch_sor32_batch(B->stream, B->cfg, B->d_sor, (int)act.size(), tiles, q == 0, 1, q, wait);
         launch_sor32_batch(B->stream, B->cfg, B->d_sor + n, (int)act.size(), tiles, 0, 1, q, wait);
@@ -1951,8 +1969,17 @@ int ibm_create_grid(const ibm_grid_params* params, ibm_ctx** out) {
   rc |= c->alloc(&c->sc, 1);
   rc |= c->alloc(&c->partials, 4 * RED_BLOCKS);
   if (!rc) rc = setup_geometry(c);
-  if (!rc && cudaMallocHost((void**)&c->sc_host, sizeof(DevScalars) + sizeof(Sor64Result)) != cudaSuccess)
-    rc = IBM_E_CUDA;
+  if (!rc) {
+    ibm_ctx::Pinned* pin = nullptr;
+    if (cudaMallocHost((void**)&pin, sizeof *pin) != cudaSuccess) {
+      rc = IBM_E_CUDA;
+    } else {
+      c->sc_host = &pin->sc;
+      c->sor64_host = &pin->sor64;
+      c->sor_err = &pin->sor_err;
+      *c->sor_err = 0u;
+    }
+  }
   if (!rc) rc = ensure_history(c, 1024);
   if (!rc && P.precision == 0) {
     c->sor64 = sor64_plan(P.nx, P.ny);
@@ -1967,7 +1994,6 @@ int ibm_create_grid(const ibm_grid_params* params, ibm_ctx** out) {
       c->sor64_tiles.norms = (unsigned long long*)(blk + 32);
       c->sor64_tiles.words = c->sor64_tiles.norms + 4 * nt;
       c->sor64_tiles.stride = words / 2;
-      c->sor64_host = (Sor64Result*)(c->sc_host + 1);
     }
   }
   // band arrays exist (1 x 1) even without a body
@@ -2439,6 +2465,8 @@ int ibm_batch_create(ibm_ctx* const* cases, int n, ibm_batch** out) {
   ok = ok && cudaMalloc((void**)&B->d_sor, 2 * n * sizeof(Sor32Case)) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&B->d_dc, n * sizeof(DcCase)) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&B->d_bits, n * sizeof(unsigned long long)) == cudaSuccess;
+  ok = ok && cudaMallocHost((void**)&B->h_err, sizeof(unsigned)) == cudaSuccess;
+  if (ok) *B->h_err = 0u;
   ok = ok && cudaMallocHost((void**)&B->h_maps, n * sor32_maps_bytes()) == cudaSuccess;
   ok = ok && cudaMalloc((void**)&B->d_maps, n * sor32_maps_bytes()) == cudaSuccess;
   ok = ok && cudaMallocHost((void**)&B->h_cases, n * sizeof(StepCase)) == cudaSuccess;

@@ -252,9 +252,14 @@ struct DcCase {
   float* r32;
   unsigned long long* res_bits;
 };
-// true once a sweep kernel has given up a bounded wait for a tile's copies
-bool sor32_failed();
-constexpr long long kSor32Wait = 4000000000ll;  // its limit: about 2 s at the SM clock
+// Form 11's bounded wait for a tile's copies: what it sets (host memory the
+// device can write, one word per context or batch) and its limit, clocks (0:
+// every wait gives up).
+constexpr long long kSor32Wait = 4000000000ll;  // about 2 s at the SM clock
+struct SorWait {
+  unsigned* err = nullptr;
+  long long limit = kSor32Wait;
+};
 // form 11: a case's four tensor maps (Sor32Case::maps; host memory, then copied to the device, 64-byte aligned)
 size_t sor32_maps_bytes();
 bool sor32_case_maps(int cfg, const Geo32& g, const float* e, const float* eb, const float* r, const float* invd,
@@ -265,7 +270,7 @@ cudaError_t sor32_batch_prepare(int cfg);
 // stream (direct launches; the kernel waits for it before its first load)
 // q: index of the launch pair within the round (cases with pairs <= q skip it)
 void launch_sor32_batch(cudaStream_t s, int cfg, const Sor32Case* cases_dev, int ncases, int total_tiles,
-                        int zero_init, int pdl = 0, int q = 0, long long wait = kSor32Wait);
+                        int zero_init, int pdl, int q, const SorWait& wait);
 void launch_dc_residual_batch(cudaStream_t s, const DcCase* cases_dev, int ncases, int total_blocks);
 
 // geometric multigrid on the FP32 correction equation (k_mg.cu)
@@ -338,9 +343,9 @@ void launch_dc_residual(cudaStream_t s, const Geo& g, int pk, const double* phi_
 // pdl: launch as a programmatic dependent of the previous kernel on the
 // stream (consecutive sweep launches outside graph capture).  With
 // zero_init = 0 the previous kernel must be a sweep launch of the same run:
-// forms 6 to 11 then read r and 1/d before waiting for it.  wait: limit of
-// form 11's wait for a tile's copies, clocks (0: every wait gives up).
-void launch_sor32(cudaStream_t s, int cfg, const Geo32& g, const float* e_in, float* e_out, const float* r,
-                  const float* invd, float omega, int zero_init, int pdl = 0, long long wait = kSor32Wait);
+// forms 6 to 11 then read r and 1/d before waiting for it.  wait: form
+// 11's, whose launch fails (and nothing runs) if its tensor maps cannot be made.
+cudaError_t launch_sor32(cudaStream_t s, int cfg, const Geo32& g, const float* e_in, float* e_out, const float* r,
+                  const float* invd, float omega, int zero_init, int pdl = 0, const SorWait& wait = SorWait{});
 
 }  // namespace ibm

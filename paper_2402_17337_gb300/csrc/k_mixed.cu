@@ -1192,26 +1192,6 @@ __global__ void __launch_bounds__(32 * C::NY, C::MINB)
   }
 }
 
-// a flag the form-11 kernels set when a wait gives up; mapped host memory, so
-// the host reads it without a device synchronisation
-unsigned* sor_error_flag(unsigned** dev) {
-  static unsigned *host = nullptr, *devp = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void *h = nullptr, *d = nullptr;
-    if (cudaHostAlloc(&h, sizeof(unsigned), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) return;
-    host = static_cast<unsigned*>(h);
-    *host = 0u;
-    if (cudaHostGetDevicePointer(&d, h, 0) == cudaSuccess) devp = static_cast<unsigned*>(d);
-  });
-  *dev = devp;
-  return host;
-}
-
-// nothing was launched for want of a tensor map or of the flag: reported as a failed wait is
-bool g_no_maps = false;
-void sor_no_maps() { g_no_maps = true; }
-
 // tensor map of a colour-split array [2][ny][pk] with boxes of 64 columns, rows rows, both colours
 bool tile_map(CUtensorMap* m, const Geo32& g, const float* p, int rows) {
   static PFN_cuTensorMapEncodeTiled_v12000 enc = nullptr;
@@ -1249,9 +1229,9 @@ int sm_count() {
 // [2.38] on 2048x1024; (88, 16, 12) 6.35 [10.5] on 4096x2048.
 struct Sor32Config {
   int TY, K, NY, V;
-  void (*launch)(cudaStream_t, const Geo32&, const float*, float*, const float*, const float*, float, int, int,
-                 long long);
-  void (*launch_batch)(cudaStream_t, const Sor32Case*, int, int, int, int, int, long long);
+  cudaError_t (*launch)(cudaStream_t, const Geo32&, const float*, float*, const float*, const float*, float, int, int,
+                        const SorWait&);
+  void (*launch_batch)(cudaStream_t, const Sor32Case*, int, int, int, int, int, const SorWait&);
   cudaError_t (*prepare)();
   void (*tiles)(const Geo32&, int*, int*);
 };
@@ -1272,8 +1252,8 @@ cudaError_t prepare_shape() {
 }
 
 template <class C>
-void launch_shape(cudaStream_t s, const Geo32& g, const float* e_in, float* e_out, const float* r, const float* invd,
-                  float omega, int zero_init, int pdl, long long wait) {
+cudaError_t launch_shape(cudaStream_t s, const Geo32& g, const float* e_in, float* e_out, const float* r,
+                         const float* invd, float omega, int zero_init, int pdl, const SorWait& wait) {
   static bool attr = false;
   if (!attr) {
     prepare_shape<C>();
@@ -1295,23 +1275,19 @@ void launch_shape(cudaStream_t s, const Geo32& g, const float* e_in, float* e_ou
     const int ntiles = (int)(grd.x * grd.y);
     lc.gridDim = dim3(std::min(ntiles, sm_count() * C::MINB));
     CUtensorMap me, mr, md;
-    unsigned* err = nullptr;
-    sor_error_flag(&err);
     constexpr int LY = C::TY + 2 * C::K;
-    if (!err || !tile_map(&me, g, e_in, LY) || !tile_map(&mr, g, r, LY) || !tile_map(&md, g, invd, LY)) {
-      sor_no_maps();
-      return;
-    }
-    cudaLaunchKernelEx(&lc, k_sor32_tma<C>, me, mr, md, g, e_out, omega, 1.f - omega, zero_init, (int)grd.x, ntiles, err,
-                       wait);
+    if (!wait.err || !tile_map(&me, g, e_in, LY) || !tile_map(&mr, g, r, LY) || !tile_map(&md, g, invd, LY))
+      return cudaErrorNotSupported;
+    return cudaLaunchKernelEx(&lc, k_sor32_tma<C>, me, mr, md, g, e_out, omega, 1.f - omega, zero_init, (int)grd.x,
+                              ntiles, wait.err, wait.limit);
   } else {
-    cudaLaunchKernelEx(&lc, k_sor32_rb<C>, g, e_in, e_out, r, invd, omega, zero_init);
+    return cudaLaunchKernelEx(&lc, k_sor32_rb<C>, g, e_in, e_out, r, invd, omega, zero_init);
   }
 }
 
 template <class C>
 void launch_shape_batch(cudaStream_t s, const Sor32Case* cases, int ncases, int total_tiles, int zero_init,
-                        int pdl, int q, long long wait) {
+                        int pdl, int q, const SorWait& wait) {
   if (total_tiles <= 0) return;
   cudaLaunchConfig_t lc{};
   lc.gridDim = dim3(total_tiles);
@@ -1324,14 +1300,9 @@ void launch_shape_batch(cudaStream_t s, const Sor32Case* cases, int ncases, int 
   lc.attrs = at;
   lc.numAttrs = pdl ? 1 : 0;
   if constexpr (C::V == 11) {
-    unsigned* err = nullptr;
-    sor_error_flag(&err);
-    if (!err) {
-      sor_no_maps();
-      return;
-    }
     lc.gridDim = dim3(std::min(total_tiles, sm_count() * C::MINB));
-    cudaLaunchKernelEx(&lc, k_sor32_tma_batch<C>, cases, ncases, total_tiles, zero_init, q, err, wait);
+    cudaLaunchKernelEx(&lc, k_sor32_tma_batch<C>, cases, ncases, total_tiles, zero_init, q, wait.err,
+                       wait.limit);
   } else {
     cudaLaunchKernelEx(&lc, k_sor32_rb_batch<C>, cases, ncases, zero_init, q);
   }
@@ -1390,9 +1361,9 @@ void launch_dc_residual(cudaStream_t s, const Geo& g, int pk, const double* phi_
   k_dc_residual<<<nt < 1216 ? nt : 1216, dim3(32, 8), 0, s>>>(g, pk, add_e ? phi_out : phi_in, b, r32, res_bits);
 }
 
-void launch_sor32(cudaStream_t s, int cfg, const Geo32& g, const float* e_in, float* e_out, const float* r,
-                  const float* invd, float omega, int zero_init, int pdl, long long wait) {
-  kConfigs[cfg].launch(s, g, e_in, e_out, r, invd, omega, zero_init, pdl, wait);
+cudaError_t launch_sor32(cudaStream_t s, int cfg, const Geo32& g, const float* e_in, float* e_out, const float* r,
+                         const float* invd, float omega, int zero_init, int pdl, const SorWait& wait) {
+  return kConfigs[cfg].launch(s, g, e_in, e_out, r, invd, omega, zero_init, pdl, wait);
 }
 
 void sor32_tiles(int cfg, const Geo32& g, int* tiles_x, int* tiles_y) { kConfigs[cfg].tiles(g, tiles_x, tiles_y); }
@@ -1400,14 +1371,8 @@ void sor32_tiles(int cfg, const Geo32& g, int* tiles_x, int* tiles_y) { kConfigs
 cudaError_t sor32_batch_prepare(int cfg) { return kConfigs[cfg].prepare(); }
 
 void launch_sor32_batch(cudaStream_t s, int cfg, const Sor32Case* cases_dev, int ncases, int total_tiles,
-                        int zero_init, int pdl, int q, long long wait) {
+                        int zero_init, int pdl, int q, const SorWait& wait) {
   kConfigs[cfg].launch_batch(s, cases_dev, ncases, total_tiles, zero_init, pdl, q, wait);
-}
-
-bool sor32_failed() {
-  unsigned* dev = nullptr;
-  const unsigned* host = sor_error_flag(&dev);
-  return g_no_maps || (host && *(volatile const unsigned*)host != 0u);
 }
 
 size_t sor32_maps_bytes() { return 4 * sizeof(CUtensorMap); }
