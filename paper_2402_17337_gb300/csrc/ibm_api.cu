@@ -910,7 +910,8 @@ SorWait sor32_wait(const ibm_ctx* c) { return SorWait{c->sor_err, c->wait < 0 ? 
 
 // Autotuner of the FP32 sweep kernel: times every tile shape on this
 // context's grid and arrays (CUDA events, a few launches each) and keeps the
-// fastest per full sweep.  Runs before the first mixed solve; the arrays'
+// fastest per full sweep; a shape whose launch is refused or gives up a wait
+// has no time.  Runs before the first mixed solve; the arrays'
 // contents are rewritten by the solve (each inner solve starts from e = 0
 // and the residual kernel rewrites r).
 int tune_sor32(ibm_ctx* c) {
@@ -920,20 +921,20 @@ int tune_sor32(ibm_ctx* c) {
   const float omega = (float)c->P.omega_p;
   const SorWait wait = sor32_wait(c);
   double best = 1e300;
-  int best_cfg = 0;
+  int best_cfg = -1;
   for (int cfg = 0; cfg < sor32_num_configs(); ++cfg) {
     const int reps = 8;
-    for (int w = 0; w < 2; ++w) {
-      CUDA_TRY(launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, 1, 1, wait));
+    cudaError_t e = cudaSuccess;
+    for (int l = -2; l < reps && e == cudaSuccess; ++l) {
+      if (l == 0) CUDA_TRY(cudaEventRecord(a, c->stream));
+      e = launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, l <= 0, 1, wait);
       std::swap(c->e32, c->e32b);
     }
-    CUDA_TRY(cudaEventRecord(a, c->stream));
-    for (int l = 0; l < reps; ++l) {
-      CUDA_TRY(launch_sor32(c->stream, cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, omega, l == 0, 1, wait));
-      std::swap(c->e32, c->e32b);
-    }
+    if (e == cudaErrorNotSupported) continue;
+    CUDA_TRY(e);
     CUDA_TRY(cudaEventRecord(b, c->stream));
     CUDA_TRY(cudaEventSynchronize(b));
+    if (sor32_gave_up(c->sor_err)) continue;
     float ms = 0.f;
     CUDA_TRY(cudaEventElapsedTime(&ms, a, b));
     const double us_sweep = sor32_tie_break(cfg) * 1e3 * ms / (reps * (sor32_half_sweeps(cfg) / 2));
@@ -946,6 +947,7 @@ int tune_sor32(ibm_ctx* c) {
   CUDA_TRY(cudaGetLastError());
   cudaEventDestroy(a);
   cudaEventDestroy(b);
+  if (best_cfg < 0) return fail(IBM_E_CUDA, "no sweep shape could be launched");
   c->sor_cfg = best_cfg;
   c->sor_us = best / sor32_tie_break(best_cfg);
   return IBM_OK;
@@ -1412,8 +1414,9 @@ constexpr int kPairsPerGraph = 8;
 // Sweep tables of the cases act[0..na) for tile shape cfg; *tiles receives
 // the CTAs of one launch; pairs (may be NULL: no limit) the launch pairs of
 // the round per active case.  Copied to the device on the batch's stream.
+// Maps that cannot be made are an error, or reported in *no_maps if given.
 int batch_sor_tables(ibm_batch* B, int cfg, const std::vector<int>& act, int* tiles,
-                     const std::vector<int>* pairs = nullptr) {
+                     const std::vector<int>* pairs = nullptr, bool* no_maps = nullptr) {
   const int n = (int)B->cs.size(), na = (int)act.size();
   int first = 0;
   // maps of the shape and of the buffers each case has now (a case stepped alone may have swapped its two)
@@ -1424,8 +1427,14 @@ int batch_sor_tables(ibm_batch* B, int cfg, const std::vector<int>& act, int* ti
     ibm_ctx* c = B->cs[i];
     const std::pair<int, const float*> key{cfg, c->e32};
     if (B->maps_of[i] == key) continue;
-    if (!sor32_case_maps(cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, B->h_maps + i * mb))
+    if (!sor32_case_maps(cfg, c->geo32, c->e32, c->e32b, c->r32, c->invd32, B->h_maps + i * mb)) {
+      B->maps_of.clear();  // those made so far are not on the device
+      if (no_maps) {
+        *no_maps = true;
+        return IBM_OK;
+      }
       return fail(IBM_E_CUDA, "batch case %d: tensor maps of the sweep arrays", i);
+    }
     B->maps_of[i] = key;
     remade = true;
   }
@@ -1503,20 +1512,23 @@ int batch_sweeps(ibm_batch* B, int na, int tiles, int pairs) {
   return IBM_OK;
 }
 
-// Common tile shape of the batch: every shape timed over all cases.
+// Common tile shape of the batch: every shape timed over all cases (as in
+// tune_sor32, without those that cannot be launched or give up a wait).
 int batch_tune(ibm_batch* B) {
   const int n = (int)B->cs.size();
   std::vector<int> all(n);
   for (int i = 0; i < n; ++i) all[i] = i;
   double best = 1e300;
-  int best_cfg = 0;
+  int best_cfg = -1;
   const bool graphs = B->use_graphs;
   B->use_graphs = false;
   for (int cfg = 0; cfg < sor32_num_configs(); ++cfg) {
     CUDA_TRY(sor32_batch_prepare(cfg));
     B->cfg = cfg;
     int tiles = 0;
-    int rc = batch_sor_tables(B, cfg, all, &tiles);
+    bool no_maps = false;
+    int rc = batch_sor_tables(B, cfg, all, &tiles, nullptr, &no_maps);
+    if (no_maps) continue;
     if (!rc) rc = batch_sweeps(B, n, tiles, 1);
     CUDA_TRY(cudaEventRecord(B->t0, B->stream));
     const int pairs = 3;
@@ -1527,6 +1539,7 @@ int batch_tune(ibm_batch* B) {
     }
     CUDA_TRY(cudaEventRecord(B->t1, B->stream));
     CUDA_TRY(cudaEventSynchronize(B->t1));
+    if (sor32_gave_up(B->h_err)) continue;
     float ms = 0.f;
     CUDA_TRY(cudaEventElapsedTime(&ms, B->t0, B->t1));
     const double us = sor32_tie_break(cfg) * 1e3 * ms / (2 * pairs * (sor32_half_sweeps(cfg) / 2));
@@ -1537,6 +1550,7 @@ int batch_tune(ibm_batch* B) {
   }
   B->use_graphs = graphs;
   B->cfg = best_cfg;
+  if (best_cfg < 0) return fail(IBM_E_CUDA, "no sweep shape could be launched");
   B->sor_us = best / sor32_tie_break(best_cfg);
   B->drop_graphs();
   return IBM_OK;

@@ -96,3 +96,22 @@ def test_a_wait_that_runs_out_fails_the_solve_that_ran_it_and_no_other():
         late.set_wait_limit(-1.0)
         got = solve(late)
         assert got[0] == want[1][0] and torch.equal(got[1], want[1][1])
+
+
+def test_the_autotuner_leaves_out_shapes_that_do_not_run():
+    """A shape whose launches give up has a short time and no result.  With the
+    limit 0 all of form 11 does: the tuners of a context and of a batch take
+    another form, and the solves that follow converge."""
+    from paper_2402_17337_gb300 import Batch, Solver, build
+    from paper_2402_17337_gb300 import workloads as W
+    build.build()
+    ss = [Solver.from_config(c, precision=1) for c in W.batch_small(3)]
+    for s in ss:
+        s.set_wait_limit(0.0)
+    for s in ss[:2]:
+        st = s.step(1)
+        assert 3 <= s.profile()["sor_form"] <= 10 and st["div_max"] <= 1e-8
+    B = Batch(ss)
+    for st in B.step(1):
+        assert st["div_max"] <= 1e-8
+    assert 3 <= B.profile()["sor_form"] <= 10
