@@ -17,7 +17,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libibm.so")
 SOURCES = ["ibm_api.cu", "k_step.cu", "k_sor.cu", "k_sor64.cu", "k_mixed.cu", "k_noalloc.cu", "k_mg.cu", "k_nn.cu", "k_conv_tc.cu",
            "unet.cu", "k_ws.cu"]
-HEADERS = ["ibm_internal.h", "sor64_loop.h", "nn_internal.h", os.path.join("..", "..", "include", "ibm.h")]
+HEADERS = ["ibm_internal.h", "sor64_loop.h", "per_device.h", "nn_internal.h", os.path.join("..", "..", "include", "ibm.h")]
 NVCC = os.environ.get("NVCC", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--fmad=false", "-Xcompiler", "-fPIC,-ffp-contract=off",

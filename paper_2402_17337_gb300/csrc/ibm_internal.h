@@ -6,9 +6,15 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "per_device.h"
 #include "sor64_loop.h"
 
 namespace ibm {
+
+inline int current_device() {
+  int d = -1;
+  return cudaGetDevice(&d) == cudaSuccess ? d : -1;
+}
 
 // Named NVTX range over a scope (host side: it spans the enqueueing of the
 // phase's kernels and any host waits inside it; a profiler attached to the

@@ -24,7 +24,6 @@
 // one CTA.  All arrays use the colour-split layout rb_at of the FP32 sweeps.
 #include <algorithm>
 #include <cstdint>
-#include <mutex>
 
 #include "ibm_internal.h"
 
@@ -550,10 +549,9 @@ void launch_fcg_update(cudaStream_t s, const MgLevel& L, const float* p, const f
 // Fills T's shared-memory offsets for its n levels (nx, ny of lv set, finest
 // first); false if the levels do not fit the CTA (threads or shared memory).
 bool mg_low_layout(MgLow& T) {
-  static bool ok = false;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    ok = cudaFuncSetAttribute(k_mg_low, cudaFuncAttributeMaxDynamicSharedMemorySize, kLowSmem) == cudaSuccess;
+  static PerDevice<bool> limit_set;
+  const bool ok = limit_set.get(current_device(), [] {
+    return cudaFuncSetAttribute(k_mg_low, cudaFuncAttributeMaxDynamicSharedMemorySize, kLowSmem) == cudaSuccess;
   });
   long off = 0, coff = 0;
   for (int l = 0; l < T.n; ++l) {

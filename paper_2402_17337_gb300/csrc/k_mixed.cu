@@ -1213,13 +1213,13 @@ bool tile_map(CUtensorMap* m, const Geo32& g, const float* p, int rows) {
 }
 
 int sm_count() {
-  static const int n = [] {
-    int d = 0, v = 0;
-    cudaGetDevice(&d);
+  static PerDevice<int> n;
+  const int d = current_device();
+  return n.get(d, [d] {
+    int v = 0;
     cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, d);
     return v;
-  }();
-  return n;
+  });
 }
 
 // Tile shapes the autotuner chooses from.  Of form 11 (us per sweep, the best
@@ -1236,8 +1236,8 @@ struct Sor32Config {
   void (*tiles)(const Geo32&, int*, int*);
 };
 
-// dynamic shared memory limits of both kernels of a shape; set once, outside
-// any stream capture
+// dynamic shared memory limits of both kernels of a shape; set once per device,
+// outside any stream capture
 template <class C>
 cudaError_t prepare_shape() {
   if constexpr (C::V == 11) {
@@ -1254,11 +1254,9 @@ cudaError_t prepare_shape() {
 template <class C>
 cudaError_t launch_shape(cudaStream_t s, const Geo32& g, const float* e_in, float* e_out, const float* r,
                          const float* invd, float omega, int zero_init, int pdl, const SorWait& wait) {
-  static bool attr = false;
-  if (!attr) {
-    prepare_shape<C>();
-    attr = true;
-  }
+  static PerDevice<cudaError_t> prepared;
+  const cudaError_t ready = prepared.get(current_device(), prepare_shape<C>);
+  if (ready != cudaSuccess) return ready;
   const int ncol = (g.nx + 1) / 2;
   dim3 grd((ncol + C::TK - 1) / C::TK, (g.ny + C::TY - 1) / C::TY);
   cudaLaunchConfig_t lc{};

@@ -20,7 +20,6 @@
 // and SM; what the launch-per-half-sweep form spent on top of that was the
 // launch (about 2.3 us) and, every check, a host wait (about 15 us).
 #include <cstdint>
-#include <mutex>
 #include <type_traits>
 
 #include "ibm_internal.h"
@@ -450,13 +449,11 @@ struct Sor64Dev {
   int sms = 0, coop = 0, smem = 0, cluster = 0;
 };
 
-const Sor64Dev& sor64_device() {
-  static Sor64Dev dev[64];
-  static std::once_flag once[64];
-  static const Sor64Dev none;
-  int d = 0;
-  if (cudaGetDevice(&d) != cudaSuccess || d < 0 || d >= 64) return none;
-  std::call_once(once[d], [d] {
+Sor64Dev sor64_device() {
+  static PerDevice<Sor64Dev> dev;
+  const int d = current_device();
+  if (d < 0) return Sor64Dev{};
+  return dev.get(d, [d] {
     Sor64Dev v;
     cudaDeviceGetAttribute(&v.sms, cudaDevAttrMultiProcessorCount, d);
     cudaDeviceGetAttribute(&v.coop, cudaDevAttrCooperativeLaunch, d);
@@ -480,9 +477,8 @@ const Sor64Dev& sor64_device() {
       if (cudaOccupancyMaxActiveClusters(&n, k_sor64_cluster, &lc) == cudaSuccess && n > 0) v.cluster = c;
     }
     cudaGetLastError();
-    dev[d] = v;
+    return v;
   });
-  return dev[d];
 }
 
 size_t tiles_smem(int w, int h, int K) { return sizeof(double) * (size_t)(w + 2 * K) * (h + 2 * K); }
@@ -498,7 +494,7 @@ long tiles_list(int w, int h, int K) {
 // Which kernel a grid takes, from its size alone.
 Sor64Plan sor64_plan(int nx, int ny) {
   Sor64Plan p;
-  const Sor64Dev& d = sor64_device();
+  const Sor64Dev d = sor64_device();
   if (d.cluster && ny >= d.cluster) {
     const int rows = (ny + d.cluster - 1) / d.cluster, w2 = (nx + 1) / 2;
     if (rows * w2 <= CL_THREADS * CL_CPT && sizeof(double) * (rows + 2) * (nx + 2) <= CL_SMEM &&
