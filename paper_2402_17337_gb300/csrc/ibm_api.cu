@@ -684,7 +684,7 @@ void nn_cycle(ibm_ctx* c) {
   launch_mg_prolong(c->stream, B, B.e[B.cur], A, A.e[A.cur]);
   launch_sor32(c->stream, c->mg_shape, A.g, A.e[A.cur], A.e[A.cur ^ 1], A.r, A.invd, 1.0f, 0);
   A.cur ^= 1;
-  c->prof.launches += c->pc_pre + 6 + unet_forward_launches();
+  c->prof.launches += c->pc_pre + 6 + unet_forward_launches(B.g.ny, B.g.nx);
 }
 
 // One iteration of flexible conjugate gradients, FCG(1), on level 0's
@@ -709,7 +709,7 @@ void fcg_iter(ibm_ctx* c, int first) {
 }
 
 int fcg_launches(const ibm_ctx* c) {
-  if (c->pc_kind == 1) return c->pc_pre + 6 + unet_forward_launches() + 3;
+  if (c->pc_kind == 1) return c->pc_pre + 6 + unet_forward_launches(c->mg[1].g.ny, c->mg[1].g.nx) + 3;
   return 4 * c->mg_low_first + 1 + 3;
 }
 
@@ -1243,7 +1243,7 @@ int step_pre(ibm_ctx* c, ibm_step_stats* st, double* thr) {
       rc = read_norm(c, &c->sc->res_bits, &r_learned);  // waits for the stream
       if (rc) return rc;
       r_plain = bits_to_double(c->sc_host->res2_bits);
-      c->prof.launches += unet_forward_launches() + 2;
+      c->prof.launches += unet_forward_launches(c->Hc, c->Wc) + 2;
       c->prof.ws_applied += 1;
       if (r_learned < 0.5 * r_plain)
         c->prof.ws_kept += 1;

@@ -330,7 +330,7 @@ void launch_ws_apply(cudaStream_t s, const Geo& g, int Hc, int Wc, const float* 
 void launch_ws_target(cudaStream_t s, const Geo& g, int Hc, int Wc, const double* phi_new, const double* phi_old,
                       const DevScalars* sc, double cT, const unsigned long long* ws_max, float* target);
 // kernels launched by one ibm_unet_forward
-int unet_forward_launches();
+int unet_forward_launches(int H, int W);
 // U-Net coarse level of the two-level preconditioner: channel 0 of feat from
 // level C's residual (max into *smax), and C's correction from the output
 void launch_nnp_features(cudaStream_t s, const MgLevel& C, float* feat, unsigned long long* smax);

@@ -744,6 +744,11 @@ int pow2_at_least(int v) {
 
 }  // namespace
 
+// pixels of a tile row: those of a narrow image, else the tile's
+static int conv_tile_width(int W) { return W >= TC_M ? TC_M : (pow2_at_least(W) < 8 ? 8 : pow2_at_least(W)); }
+
+bool conv3x3_pools(int H, int W) { return conv_tile_width(W) == TC_M && H % 2 == 0 && W % 2 == 0; }
+
 size_t packed_conv_weights(int Cin, int Cout) { return (size_t)Cout * 9 * Cin; }
 
 PackJob pack_job(int Cin, int Cout, const bf16* w, bf16* wpk, bool flip) {
@@ -893,7 +898,7 @@ int conv3x3(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* X, int 
     return -1;
   }
   TcGeom G{};
-  G.TW = W >= TC_M ? TC_M : (pow2_at_least(W) < 8 ? 8 : pow2_at_least(W));
+  G.TW = conv_tile_width(W);
   G.R = TC_M / G.TW;
   G.copies = G.R == 1 ? 1 : 3;
   G.boxw = G.R == 1 ? G.TW + 2 : G.TW;
@@ -918,7 +923,7 @@ int conv3x3(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* X, int 
       if (rb * G.NT <= 64 && (long)G.tiles_x * G.tiles_z * ((H + rb - 1) / rb) >= 152) G.RB = rb;
   // the pooling in the epilogue takes two rows of a tile
   if (also.pool && G.R == 1 && G.RB == 1 && 2 * G.NT <= 256) G.RB = 2;
-  const bool pool = also.pool && G.R == 1 && G.RB % 2 == 0 && H % 2 == 0 && W % 2 == 0;
+  const bool pool = also.pool && conv3x3_pools(H, W);
   if (!pool) also.pool = nullptr;
   if (pooled) *pooled = pool;
   // Channels per chunk: the most of which two stages fit.  A TMA box moves

@@ -27,11 +27,13 @@ struct ConvAlso {
 // (k_conv_tc.cu); Cin, Cout % 16 == 0, ldx, offx, ldy, offy % 8 == 0; wpk:
 // the weights packed by pack_conv_weights; Y may be null (only the other
 // outputs are wanted); yf: optional FP32 copy of output channel 0, [H][W].
-// *pooled: whether also.pool was written (a layer of narrow tiles cannot; the
-// caller then pools).  Returns 0, or -1 with ibm_last_error set.
+// *pooled: whether also.pool was written (conv3x3_pools; else the caller pools).  Returns 0, or -1 with ibm_last_error set.
 int conv3x3(cudaStream_t s, int H, int W, int Cin, int Cout, const bf16* X, int ldx, int offx, const bf16* wpk,
             const float* bias, bf16* Y, int ldy, int offy, bool relu, float* yf, ConvAlso also = ConvAlso{},
             bool* pooled = nullptr);
+// whether a convolution of an H x W image can write its 2x2 average: rows of a
+// whole tile, more than 64 pixels, and even sizes
+bool conv3x3_pools(int H, int W);
 // elements of the packed weights of a convolution with Cin inputs and Cout
 // outputs, and the packing of w[Cout][9][Cin] (flip: of the data-gradient
 // operator of a layer with weights w[Cin][9][Cout], W'[co][tap][ci] =

@@ -406,9 +406,13 @@ int ibm_unet_grads(const ibm_unet* n, float* host, long long count) {
 }  // extern "C"
 
 namespace ibm {
-// kernels one forward pass launches: input packing and 15 convolutions (a
-// level narrower than 128 pixels pools in a kernel of its own)
-int unet_forward_launches() { return 1 + 15; }
+// kernels one forward pass launches: input packing, 15 convolutions, and a
+// pooling for each of the upper levels whose convolutions cannot pool
+int unet_forward_launches(int H, int W) {
+  int n = 1 + 15;
+  for (int l = 0; l < 3; ++l) n += conv3x3_pools(H >> l, W >> l) ? 0 : 1;
+  return n;
+}
 }  // namespace ibm
 
 extern "C" {
