@@ -63,7 +63,7 @@ struct ibm_unet {
   // activations for the current size
   int H = 0, W = 0;
   Level lv[4];
-  bf16 *e3 = nullptr, *ge3 = nullptr, *out = nullptr, *gout = nullptr;
+  bf16 *e3 = nullptr, *ge3 = nullptr, *gout = nullptr;
   float *outf = nullptr;
   double* loss_d = nullptr;
   std::vector<void*> act_allocs;
@@ -133,7 +133,6 @@ int ensure_acts(ibm_unet* n, int H, int W) {
   size_t px3 = (size_t)n->lv[3].H * n->lv[3].W, px0 = (size_t)H * W;
   B(&n->e3, px3, w[3]);
   B(&n->ge3, px3, w[3]);
-  B(&n->out, px0, 16);
   B(&n->gout, px0, 16);
   rc |= dalloc(n, (void**)&n->outf, px0 * sizeof(float));
   if (rc) return IBM_E_CUDA;
@@ -142,7 +141,8 @@ int ensure_acts(ibm_unet* n, int H, int W) {
   return IBM_OK;
 }
 
-// conv index, its input and its output (views into the level buffers)
+// conv index, its input and its output (views into the level buffers; the head,
+// which writes FP32 only, has its output's gradient there)
 struct Edge {
   int conv;
   Act x, y;
@@ -164,7 +164,7 @@ std::vector<Edge> edges(ibm_unet* n) {
     e.push_back({k, cat, bb});
     e.push_back({k + 1, bb, d});
   }
-  e.push_back({14, Act{n->lv[0].d, w[0], 0, w[0]}, Act{n->out, 16, 0, 16}});
+  e.push_back({14, Act{n->lv[0].d, w[0], 0, w[0]}, Act{n->gout, 16, 0, 16}});
   return e;
 }
 
@@ -177,7 +177,7 @@ Act grad_of(ibm_unet* n, const Act& a) {
       if (pr[0] == a.p) return Act{pr[1], a.ld, a.off, a.c};
   }
   if (a.p == n->e3) return Act{n->ge3, a.ld, a.off, a.c};
-  if (a.p == n->out) return Act{n->gout, a.ld, a.off, a.c};
+  if (a.p == n->gout) return a;
   return Act{};
 }
 
