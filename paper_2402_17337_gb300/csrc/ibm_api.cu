@@ -2026,6 +2026,9 @@ int ibm_create_grid(const ibm_grid_params* params, ibm_ctx** out) {
                      sizeof(double), P.ny, cudaMemcpyHostToDevice) != cudaSuccess)
       rc = IBM_E_CUDA;
   }
+  // the buffers are cleared on the legacy stream, which the context's own does not wait for: an exchange word of the
+  // FP64 tiles cleared under a running launch would be waited for in vain
+  if (!rc && cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) rc = IBM_E_CUDA;
   if (rc) {
     std::string keep = g_err;
     delete c;
