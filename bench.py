@@ -438,7 +438,8 @@ def run_batch(args):
         nbytes = SOR32_BYTES_PER_CELL_LAUNCH * prof["sweep_cells"]
         achieved = nbytes / (prof["sweep_ms"] / 1e3) / 1e9
         rows, half, _ = prof["sor_shape"]
-        roof = {"bound": "hbm", "kernel": f"k_sor32_rb_batch (FP32 red-black SOR over the tiles of every active "
+        kernel = "k_sor32_tma_batch" if prof["sor_form"] == 11 else "k_sor32_rb_batch"
+        roof = {"bound": "hbm", "kernel": f"{kernel} (FP32 red-black SOR over the tiles of every active "
                                           f"case, tile {rows} rows x 128 cells, {half} half-sweeps per launch)",
                 "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"],
                 "traffic": None, "launch_us": 1e3 * prof["sweep_ms"] / prof["sweep_launches"],
@@ -503,8 +504,7 @@ def run_batch(args):
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
             "dtype": "f32 sweeps, f64 residual/update/norms", "data": "synthetic",
             "config": batch_config(cfgs, world),
-            "details": {"path": "mixed, batched, " + ("graph replay" if args.batch_launch == "graphs" else
-                                                      "direct programmatic dependent launches"),
+            "details": {"path": "mixed, batched, per-case sweep budgets, direct programmatic dependent launches",
                         "warm_start": "previous increment", "sor_us_per_sweep_whole_batch": prof["sor_us_per_sweep"],
                         "poisson_sweeps_per_step_sum": statistics.mean(sum(x["sweeps_p"] for x in st)
                                                                        for st in stats),

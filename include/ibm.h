@@ -183,9 +183,10 @@ int ibm_poisson_solve(ibm_ctx* ctx, const double* b_dev, double* phi_dev, double
  * real-time loop that cannot take the device-wide synchronisation an
  * allocation may cause.  It needs no context: the caller passes the grid's
  * face coordinates and its own buffers, and every scratch value (the 1-D
- * coefficients and the residual-norm accumulator) lives in one fixed-size
- * static device array of the library, which each GPU that loads the library
- * holds (9.9 MB) until the process exits.
+ * coefficients, the residual norm, the sweeps' result and the words through
+ * which the tiles of a grid of up to 300 000 cells exchange their halos) lives
+ * in one fixed-size static device array of the library, which each GPU that
+ * loads the library holds (9.9 MB) until the process exits.
  *
  * Solves L_p phi = b on the grid with face coordinates xf (nx+1 host
  * doubles) and yf (ny+1 host doubles), homogeneous Neumann, by red-black SOR
