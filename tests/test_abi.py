@@ -162,3 +162,10 @@ def test_noalloc_solve_rejects_non_increasing_faces_before_touching_the_device()
                 None, None, None)
         assert rc == ibm.IBM_E_INVAL
         assert f"{axis}[{k}]".encode() in ibm.lib().ibm_last_error()
+
+
+def test_wait_limit_rejects_a_null_handle_before_touching_the_device():
+    from paper_2402_17337_gb300 import build
+    build.build()
+    import paper_2402_17337_gb300 as ibm
+    assert ibm.lib().ibm_set_wait_limit(None, 1.0) == ibm.IBM_E_INVAL and ibm.lib().ibm_last_error()
