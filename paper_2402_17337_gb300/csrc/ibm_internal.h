@@ -352,6 +352,6 @@ void launch_dc_residual(cudaStream_t s, const Geo& g, int pk, const double* phi_
 // forms 6 to 11 then read r and 1/d before waiting for it.  wait: form
 // 11's, whose launch fails (and nothing runs) if its tensor maps cannot be made.
 cudaError_t launch_sor32(cudaStream_t s, int cfg, const Geo32& g, const float* e_in, float* e_out, const float* r,
-                  const float* invd, float omega, int zero_init, int pdl = 0, const SorWait& wait = SorWait{});
+                         const float* invd, float omega, int zero_init, int pdl = 0, const SorWait& wait = SorWait{});
 
 }  // namespace ibm

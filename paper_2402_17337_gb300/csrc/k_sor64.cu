@@ -1,8 +1,8 @@
 // FP64 red-black SOR of the pressure equation with the grid kept on chip for
 // many sweeps (arXiv 2402.17337 Sec. 2.2, Sec. 3.1), including the residual
-// checks: one launch runs up to a few thousand sweeps and leaves when the
-// tolerance is met, so the host is asked once per launch, not once per check
-// (sor64_loop.h: when a launch checks and when it ends).
+// checks: one launch runs hundreds (tiles) or thousands (cluster) of sweeps and
+// leaves when the tolerance is met, so the host is asked once per launch, not
+// once per check (sor64_loop.h: when a launch checks and when it ends).
 //
 // The iterates are those of k_poisson_half / k_poisson_res (k_sor.cu): the
 // same fma chains in the same order, the same reciprocal diagonal, the norm
